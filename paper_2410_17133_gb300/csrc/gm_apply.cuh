@@ -23,6 +23,7 @@
 
 #include "gm_bulk.cuh"
 #include "gm_bulk32.cuh"
+#include "gm_bulkfx.cuh"
 
 __device__ inline void gm_pcg_alpha_from(PcgScalars* sc, double pq)
 {
@@ -356,7 +357,70 @@ inline BulkArgs<T> gm_bulk_args(gm_ctx* c, double cK, double cApu, double cAup, 
     b.zu = nullptr; b.zp = nullptr; b.pu_new = nullptr; b.pp_new = nullptr;
     b.beta = nullptr; b.part = nullptr;
     b.fs = nullptr; b.cFS = T(0);
+    b.cfx = T(1); b.accumulate = 0;
     return b;
+}
+
+// Shared-memory opt-in of the fixed-point kernels, once per device (at bind).
+template <int CLS>
+static int gm_fx_setup(int dev)
+{
+    static bool done[64] = {};
+    if (done[dev & 63]) return 0;
+    auto set = [](const void* k, size_t n) {
+        return (int)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+    };
+    int e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_K, false>, gm_fx_smem<GM_M_K>());
+    if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_K, true>, gm_fx_smem<GM_M_K>());
+    if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_APU, false>, gm_fx_smem<GM_M_APU>());
+    if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_AUP, false>, gm_fx_smem<GM_M_AUP>());
+    if (!e) done[dev & 63] = true;
+    return e;
+}
+
+// One FP64 block by the fixed-point kernel; returns the number of CTAs.  A CTA
+// (two per SM: their registers) marches its planes plus a halo layer, and looks
+// over its inputs first, which costs about half a layer.
+template <int CLS, int MODE, bool DOT>
+static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accumulate, cudaStream_t s)
+{
+    const int gx = (c->nx + 1 + 14) / 15, gy = (c->ny + 1 + 14) / 15, np = c->g.nplanes;
+    int zc = c->zchunk_override;
+    if (zc <= 0) {
+        long long best = -1;
+        for (int z = 1; z <= np; ++z) {
+            const long long ctas = (long long)gx * gy * ((np + z - 1) / z);
+            const long long cost = ((ctas + 2 * c->sm_count - 1) / (2 * c->sm_count)) * (2 * z + 3);
+            if (best < 0 || cost < best) { best = cost; zc = z; }
+        }
+    }
+    const int gz = (np + zc - 1) / zc;
+    b.zchunk = zc;
+    b.cfx = factor;
+    b.accumulate = accumulate ? 1 : 0;
+    gm_bulk_fx_kernel<CLS, MODE, DOT><<<dim3(gx, gy, gz), 256, gm_fx_smem<MODE>(), s>>>(b, c->Rfx, c->R64);
+    c->applies++;
+    c->launches++;
+    return gx * gy * gz;
+}
+
+// New search direction p = z + beta p_old of a K_T solve, constrained entries 0
+// (the fixed-point product needs the whole direction before it can scale it).
+static __global__ void __launch_bounds__(256)
+gm_pcg_dir_kernel(long long N, const double* z, const double* p_old, double* p, const uint8_t* mask,
+                  const PcgScalars* sc)
+{
+    if (sc->done) return;
+    const double beta = sc->beta;
+    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
+         n += (long long)gridDim.x * blockDim.x) {
+        const unsigned m = mask[n];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const long long k = c * N + n;
+            p[k] = ((m >> c) & 1u) ? 0.0 : fma(beta, p_old[k], z[k]);
+        }
+    }
 }
 
 template <typename T, int CLS, int MODE>
@@ -371,12 +435,27 @@ static void gm_apply_launch_t(gm_ctx* c, const RefOps<T>& R, double cK, double c
     b.xu = xu; b.xp = xp; b.yu = yu; b.yp = yp;
     b.skip = skip;
     constexpr int BULK = MODE & (GM_M_K | GM_M_APU | GM_M_AUP | GM_M_S | GM_M_C);
-    if constexpr (std::is_same<T, float>::value && (BULK == GM_M_K || BULK == (GM_M_S | GM_M_C)))
-        gm_bulk32_launch<CLS, BULK, false>(c, b, s);
-    else
-        gm_bulk_apply_kernel<T, CLS, BULK, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
-    c->applies++;
-    c->launches++;
+    if constexpr (std::is_same<T, double>::value) {
+        // block by block: K_b, A_pu and A_up in fixed point, S and C in FP64
+        constexpr int FLOW = BULK & (GM_M_S | GM_M_C);
+        if constexpr ((BULK & GM_M_K) != 0) gm_fx_launch<CLS, GM_M_K, false>(c, b, cK, false, s);
+        if constexpr ((BULK & GM_M_APU) != 0) gm_fx_launch<CLS, GM_M_APU, false>(c, b, cApu, (BULK & GM_M_K) != 0, s);
+        if constexpr (FLOW != 0) {
+            b.zchunk = zchunk;
+            b.accumulate = 0;
+            gm_bulk_apply_kernel<T, CLS, FLOW, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+            c->applies++;
+            c->launches++;
+        }
+        if constexpr ((BULK & GM_M_AUP) != 0) gm_fx_launch<CLS, GM_M_AUP, false>(c, b, cAup, FLOW != 0, s);
+    } else {
+        if constexpr (BULK == GM_M_K || BULK == (GM_M_S | GM_M_C))
+            gm_bulk32_launch<CLS, BULK, false>(c, b, s);
+        else
+            gm_bulk_apply_kernel<T, CLS, BULK, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+        c->applies++;
+        c->launches++;
+    }
     // K_b alone has no fault term: the bulk kernel's product is complete
     constexpr bool FAULT_TERMS = (MODE & (GM_M_KF | GM_M_APU | GM_M_AUP | GM_M_S | GM_M_C)) != 0;
     if (FAULT_TERMS && c->g.kf >= 0) {
@@ -431,12 +510,21 @@ static void gm_pcg_apply_t(gm_ctx* c, const RefOps<T>& R, const T* z, const T* p
     if (U) { b.xu = p_old; b.zu = z; b.pu_new = p_new; b.yu = q; b.xp = nullptr; b.yp = nullptr; }
     else { b.xp = p_old; b.zp = z; b.pp_new = p_new; b.yp = q; b.xu = nullptr; b.yu = nullptr; }
     constexpr int BULK = MODE & (GM_M_K | GM_M_S | GM_M_C);
-    if constexpr (std::is_same<T, float>::value)
+    if constexpr (std::is_same<T, float>::value) {
         nbulk = gm_bulk32_launch<CLS, BULK, true>(c, b, s);
-    else
+        c->applies++;
+        c->launches++;
+    } else if constexpr (U) {
+        const int nblk = (int)std::min<long long>((c->N + 255) / 256, GM_RED_BLOCKS);
+        gm_pcg_dir_kernel<<<nblk, 256, 0, s>>>(c->N, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
+        c->launches++;
+        b.xu = p_new;
+        nbulk = gm_fx_launch<CLS, GM_M_K, true>(c, b, 1.0, false, s);
+    } else {
         gm_bulk_apply_kernel<T, CLS, BULK, true><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
-    c->applies++;
-    c->launches++;
+        c->applies++;
+        c->launches++;
+    }
     if (c->g.kf >= 0) {
         FaultArgs<T> f = gm_fault_args<T>(c, cK, 0, 0, cS, cC, U);
         if (U) { f.xu = p_new; f.yu = q; f.xp = nullptr; f.yp = nullptr; }

@@ -50,19 +50,24 @@ int gm_launch_pcg_apply_f64(gm_ctx* c, int which, const double* z, const double*
 // smoother adds the cohesive term of the lip pairs itself.
 int gm_launch_bulk_k_f64(gm_ctx* c, const double* x, double* y, cudaStream_t s, const int* skip)
 {
-    int gx, gy, gz, zchunk;
-    gm_bulk_geometry(c, &gx, &gy, &gz, &zchunk);
     BulkArgs<double> b = gm_bulk_args<double>(c, 1.0, 0.0, 0.0, 0.0, 0.0, c->dE64.as<double>(), c->dK64.as<double>());
-    b.zchunk = zchunk;
     b.xu = x; b.xp = nullptr; b.yu = y; b.yp = nullptr;
     b.skip = skip;
-    const dim3 grid(gx, gy, gz);
     switch (c->cls) {
-    case GM_CLS_BOX: gm_bulk_apply_kernel<double, GM_CLS_BOX, GM_M_K, false><<<grid, 256, 0, s>>>(b, c->R64); break;
-    case GM_CLS_MONO: gm_bulk_apply_kernel<double, GM_CLS_MONO, GM_M_K, false><<<grid, 256, 0, s>>>(b, c->R64); break;
-    default: gm_bulk_apply_kernel<double, GM_CLS_GEN, GM_M_K, false><<<grid, 256, 0, s>>>(b, c->R64); break;
+    case GM_CLS_BOX: gm_fx_launch<GM_CLS_BOX, GM_M_K, false>(c, b, 1.0, false, s); break;
+    case GM_CLS_MONO: gm_fx_launch<GM_CLS_MONO, GM_M_K, false>(c, b, 1.0, false, s); break;
+    default: gm_fx_launch<GM_CLS_GEN, GM_M_K, false>(c, b, 1.0, false, s); break;
     }
-    c->applies++;
-    GM_LAUNCHED(c);
+    if (cudaError_t e = cudaGetLastError(); e != cudaSuccess)
+        return c->set_err(GM_ECUDA, std::string("bulk launch: ") + cudaGetErrorString(e));
+    return GM_OK;
+}
+
+int gm_prepare_fx(gm_ctx* c)
+{
+    const int e = c->cls == GM_CLS_BOX ? gm_fx_setup<GM_CLS_BOX>(c->device)
+                : c->cls == GM_CLS_MONO ? gm_fx_setup<GM_CLS_MONO>(c->device)
+                                        : gm_fx_setup<GM_CLS_GEN>(c->device);
+    if (e) return c->set_err(GM_ECUDA, std::string("fixed-point kernel set-up: ") + cudaGetErrorString((cudaError_t)e));
     return GM_OK;
 }

@@ -44,9 +44,32 @@ constexpr int gm_bulk_min_blocks()
          : (CLS == GM_CLS_BOX && (MODE == GM_M_K || MODE == (GM_M_S | GM_M_C))) ? 3 : 2;
 }
 
+// Shared memory of one tile: two node planes and the face tuples.
+template <typename T, int MODE>
+struct BulkTileSmem {
+    static constexpr int NI = ((MODE & (GM_M_K | GM_M_AUP)) ? 3 : 0) + ((MODE & (GM_M_APU | GM_M_S | GM_M_C)) ? 1 : 0);
+    static constexpr int NO = ((MODE & (GM_M_K | GM_M_APU)) ? 3 : 0) + ((MODE & (GM_M_AUP | GM_M_S | GM_M_C)) ? 1 : 0);
+    T plane[2][NI][17 * 17];
+    T face[NO][4][256];
+};
+
+// Per-CTA sum of `dot` to part[cta] in a fixed order: warp shuffles, then warps.
+__device__ inline void gm_cta_dot(double dot, double* sh, double* part)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dot;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double sacc = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) sacc += sh[w];
+        part[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = sacc;
+    }
+}
+
 template <typename T, int CLS, int MODE, bool PCG>
-__global__ void __launch_bounds__(256, gm_bulk_min_blocks<T, CLS, MODE>())
-gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
+__device__ __forceinline__ void gm_bulk_tile(const BulkArgs<T>& a, const RefOps<T>& R, BulkTileSmem<T, MODE>& sm)
 {
     constexpr bool DO_K = (MODE & GM_M_K) != 0;
     constexpr bool DO_APU = (MODE & GM_M_APU) != 0;
@@ -64,10 +87,8 @@ gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
     constexpr ParPat PP = gm_make_parpat(CLS);
     static_assert(!PCG || (NI == NO && (NI == 3 || NI == 1)), "PCG mode needs a square single-field-group operator");
 
-    if (a.skip != nullptr && *a.skip != 0) return;
-
-    __shared__ T s_plane[2][NI][17 * 17];
-    __shared__ T s_face[NO][4][256];
+    auto& s_plane = sm.plane;
+    auto& s_face = sm.face;
 
     const GridDesc& g = a.g;
     const int tid = threadIdx.x;
@@ -337,7 +358,8 @@ gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
                                 s_face[f][2][tid - 16] + s_face[f][3][tid - 17];
                     if (OUT_U && f < 3) {
                         const T y = ((m >> f) & 1u) ? T(0) : v;
-                        a.yu[f * N + node] = y;
+                        if (sizeof(T) == 8 && a.accumulate) a.yu[f * N + node] += y;
+                        else a.yu[f * N + node] = y;
                         if constexpr (PCG) {
                             // own_cur holds z + beta p_old of this node, masked at load
                             a.pu_new[f * N + node] = own_cur[f];
@@ -347,7 +369,8 @@ gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
                         // raw value on a tied slave lip: the fault kernel folds it
                         const bool slave = g.tied && kk == g.kf + 1;
                         const T y = (!slave && ((m >> 3) & 1u)) ? T(0) : v;
-                        a.yp[node] = y;
+                        if (sizeof(T) == 8 && a.accumulate) a.yp[node] += y;
+                        else a.yp[node] = y;
                         if constexpr (PCG) {
                             const T pn = slave ? T(0) : own_cur[IPI];
                             a.pp_new[node] = pn;
@@ -366,18 +389,16 @@ gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
     }
 
     if constexpr (PCG) {
-        // per-CTA partial of p . Ap (fixed order: warp shuffles, then warps)
         __shared__ double sh[8];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, o);
-        if ((tid & 31) == 0) sh[tid >> 5] = dot;
-        __syncthreads();
-        if (tid == 0) {
-            double sacc = 0.0;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) sacc += sh[w];
-            const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-            a.part[cta] = sacc;
-        }
+        gm_cta_dot(dot, sh, a.part);
     }
+}
+
+template <typename T, int CLS, int MODE, bool PCG>
+__global__ void __launch_bounds__(256, gm_bulk_min_blocks<T, CLS, MODE>())
+gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
+{
+    if (a.skip != nullptr && *a.skip != 0) return;
+    __shared__ BulkTileSmem<T, MODE> sm;
+    gm_bulk_tile<T, CLS, MODE, PCG>(a, R, sm);
 }

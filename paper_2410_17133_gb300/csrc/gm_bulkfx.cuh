@@ -1,0 +1,362 @@
+// FP64 bulk products in wide fixed point (gm_fixed.cuh): K_b (u -> u), A_pu
+// (p -> u) and A_up (u -> p) of gm_bulk.cuh, same operator, tiling and march.
+//
+// Why: the FP64 kernel is bound by the FP64 pipe (2 lanes per clock and SM).
+// In the parity basis a K_b element takes about 210 FP64 instructions, 64
+// issue slots each; the same element takes about 2200 integer instructions here
+// (560 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
+// per product: K_T on 128^3 dipping cells 1254 -> 403; K_T + A_pu + A_up on
+// 61x127x46 cells sheared both ways 683 -> 229; J on 8^3 cells 89 -> 62.
+//
+// Each CTA first looks over its inputs: the largest exponent sets the tile's
+// unit, and the smallest of the elements' largest exponents says how far the
+// field is graded inside the tile.  Where the fixed-point error (2^-69 of the
+// tile's largest term) could exceed the rounding of FP64 arithmetic in some
+// element - values graded by more than a.fx_grade bits inside the tile, not
+// finite, or near the ends of the exponent range - the CTA runs the FP64 tile
+// of gm_bulk.cuh instead, so every element is at least as exact as in FP64.
+//
+// A thread owns one face, 16 x 16 faces per CTA.  The limbs of the element's
+// modes take 63 registers and those of the carried tuples 36: kept in registers
+// (232 a thread, 8 warps per SM) the kernel waited for the latency of its own
+// multiply-add chains (issue slots 33 % used); with the carry in shared memory
+// and both planes of a layer transformed from the ring of staged planes it
+// runs 16 warps per SM.  Chunks of planes are as long as fill whole waves (the
+// halo layer of a chunk costs as much as an owned one).  The two node rows of
+// a face column meet by a shuffle in x and one shared word per limb in y.
+#pragma once
+
+#include "gm_bulk.cuh"
+#include "gm_fixed.cuh"
+
+template <int MODE>
+struct FxSmem {
+    static constexpr int NI = MODE == GM_M_APU ? 1 : 3, NO = MODE == GM_M_AUP ? 1 : 3;
+    static constexpr bool CARRY = MODE == GM_M_K;      // K_b: the carried tuples live here, not in registers
+    int plane[3][NI][3][17 * 17];                      // ring of node planes, limb by limb
+    int face[2][NO][3][256];                           // upper node row of the faces, by plane parity
+    int carry[CARRY ? NO * 12 : 1][CARRY ? 256 : 1];
+};
+template <int MODE>
+constexpr size_t gm_fx_smem()
+{
+    return sizeof(FxSmem<MODE>) > sizeof(BulkTileSmem<double, MODE>) ? sizeof(FxSmem<MODE>)
+                                                                     : sizeof(BulkTileSmem<double, MODE>);
+}
+
+// The FP64 tile as a function of its own: it needs twice the registers, and
+// inlined its spills would reach into the fixed-point part.
+template <int CLS, int MODE>
+__device__ __noinline__ void gm_fx_fp64_tile(const BulkArgs<double>& a, const RefOps<double>& R, void* sm)
+{
+    gm_bulk_tile<double, CLS, MODE, false>(a, R, *static_cast<BulkTileSmem<double, MODE>*>(sm));
+}
+
+template <int CLS, int MODE, bool DOT>
+__global__ void __launch_bounds__(256, 2)
+gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_constant__ RefFx F, const __grid_constant__ RefOps<double> R)
+{
+    constexpr bool DO_K = MODE == GM_M_K;
+    constexpr bool DO_APU = MODE == GM_M_APU;
+    constexpr bool DO_AUP = MODE == GM_M_AUP;
+    static_assert(DO_K || DO_APU || DO_AUP, "one block at a time");
+    static_assert(!DOT || DO_K, "the dot product belongs to K_b");
+    constexpr int NI = DO_APU ? 1 : 3;
+    constexpr int NO = DO_AUP ? 1 : 3;
+    constexpr int TN = 17, PL = TN * TN;
+    constexpr ParPat PP = gm_make_parpat(CLS);
+    extern __shared__ __align__(16) unsigned char raw[];
+    __shared__ int s_mx[8], s_mn[8];
+    __shared__ double s_dot[8];
+
+    if (a.skip != nullptr && *a.skip != 0) return;
+
+    const GridDesc& g = a.g;
+    const int tid = threadIdx.x;
+    const int tx = tid & 15, ty = tid >> 4;
+    const int x0 = blockIdx.x * 15, y0 = blockIdx.y * 15;
+    const int fi = x0 - 1 + tx, fj = y0 - 1 + ty;
+    const bool fval = fi >= 0 && fi < g.nx && fj >= 0 && fj < g.ny;
+    const int z0 = blockIdx.z * a.zchunk;
+    const int z1 = min(z0 + a.zchunk, g.nplanes);
+    const int N = (int)g.N, nb = (int)g.nb, rowlen = g.nx + 1;
+    const double* xin = DO_APU ? a.xp : a.xu;
+    auto layer_exists = [&](int kb) -> bool { return kb >= 0 && kb + 1 < g.nplanes && kb != g.kf; };
+    auto layer_index = [&](int kb) -> int { return (g.kf >= 0 && kb > g.kf) ? kb - 1 : kb; };
+    // node whose value plane kk's node takes: a tied upper lip reads the pressure of the lower lip
+    auto src_plane = [&](int kk) -> int { return (DO_APU && g.tied && kk == g.kf + 1) ? kk - 1 : kk; };
+
+    // ---- the tile's unit and grading -------------------------------------
+    const int kbeg = layer_exists(z0 - 1) ? z0 - 1 : z0;
+    const int kend = layer_exists(z1 - 1) ? z1 : z1 - 1;      // last plane read
+    int mx = 0, mn = 0x7fffffff;
+    {
+        int below = 0;
+        for (int kk = kbeg; kk <= kend; ++kk) {
+            int m4 = 0;
+            if (fval) {
+                const int node0 = src_plane(kk) * nb + fj * rowlen + fi;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int node = node0 + (q & 1) + (q >> 1) * rowlen;
+                    const unsigned m = a.mask[node];
+#pragma unroll
+                    for (int f = 0; f < NI; ++f) {
+                        const int hi = __ldg(reinterpret_cast<const int*>(xin + (long long)f * N + node) + 1) & 0x7fffffff;
+                        if (!((m >> (DO_APU ? 3 : f)) & 1u)) m4 = max(m4, hi);
+                    }
+                }
+                if (layer_exists(kk - 1) && kk > kbeg) {
+                    const int e = max(below, m4);
+                    mx = max(mx, e);
+                    if (e != 0) mn = min(mn, e);
+                }
+            }
+            below = m4;
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        if ((tid & 31) == 0) { s_mx[tid >> 5] = mx; s_mn[tid >> 5] = mn; }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) { mx = max(mx, s_mx[w]); mn = min(mn, s_mn[w]); }
+    }
+    mx >>= 20;
+    mn = min(mn >> 20, mx);
+    const int top = mx == 0 ? 1023 : mx;
+    const int qe = (top - 1022 - GM_FX_IN) + (DO_K ? F.eK + F.topE - 1022 : F.eA);
+    const bool fixed_ok = top < 0x7ff && top >= 100 && qe >= -1000 && qe <= 900 &&
+                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : F.gradeA));
+    if (!fixed_ok) {
+        // uniform over the CTA
+        gm_fx_fp64_tile<CLS, MODE>(a, R, raw);
+        if constexpr (DOT) {
+            // the thread's own outputs times its inputs, off the lips
+            double dot = 0.0;
+            const int gi = x0 - 1 + tx, gj = y0 - 1 + ty;
+            if (tx >= 1 && ty >= 1 && gi <= g.nx && gj <= g.ny)
+                for (int kk = z0; kk < z1; ++kk) {
+                    if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) continue;
+                    const int node = kk * nb + gj * rowlen + gi;
+#pragma unroll
+                    for (int f = 0; f < 3; ++f)
+                        dot = fma(a.xu[(long long)f * N + node], a.yu[(long long)f * N + node], dot);
+                }
+            gm_cta_dot(dot, s_dot, a.part);
+        }
+        return;
+    }
+    FxSmem<MODE>& S = *reinterpret_cast<FxSmem<MODE>*>(raw);
+    const double scale = gm_fx_real((int64_t)(qe + 1023) << 52) * a.cfx;
+
+    // ---- staging: tile nodes tid and tid + 256 ------------------------------
+    int sl_off[2];
+    bool sl_in[2];
+#pragma unroll
+    for (int sl = 0; sl < 2; ++sl) {
+        const int idx = tid + sl * 256;
+        const int ni = idx % TN, nj = idx / TN;
+        const int gi = x0 - 1 + ni, gj = y0 - 1 + nj;
+        sl_in[sl] = idx < PL && gi >= 0 && gi <= g.nx && gj >= 0 && gj <= g.ny;
+        sl_off[sl] = gi + rowlen * gj;
+    }
+    double pf[2][NI];
+    auto fetch = [&](int kk) {
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl) {
+#pragma unroll
+            for (int f = 0; f < NI; ++f) pf[sl][f] = 0.0;
+            if (!sl_in[sl]) continue;
+            const int node = src_plane(kk) * nb + sl_off[sl];
+            const unsigned m = a.mask[node];
+#pragma unroll
+            for (int f = 0; f < NI; ++f)
+                if (!((m >> (DO_APU ? 3 : f)) & 1u)) pf[sl][f] = xin[(long long)f * N + node];
+        }
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl) {
+            if (tid + sl * 256 >= PL) continue;
+#pragma unroll
+            for (int f = 0; f < NI; ++f) {
+                int l[3];
+                gm_fx_from_double(pf[sl][f], top, l);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) S.plane[buf][f][i][tid + sl * 256] = l[i];
+            }
+        }
+    };
+    // xy part of the forward transform of the face, limb by limb
+    auto fwd_xy = [&](int buf, int f, int (&t)[4][3]) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int* s = &S.plane[buf][f][i][ty * TN + tx];
+            const int v00 = s[0], v10 = s[1], v01 = s[TN], v11 = s[TN + 1];
+            const int a0 = v00 + v10, a1 = v00 - v10, b0 = v01 + v11, b1 = v01 - v11;
+            t[0][i] = a0 + b0;
+            t[1][i] = a1 + b1;
+            t[2][i] = a0 - b0;
+            t[3][i] = a1 - b1;
+        }
+    };
+
+    // top contributions of the layer below, per output field and tuple
+    constexpr bool SC = FxSmem<MODE>::CARRY;
+    int rcarry[SC ? 1 : NO][4][3];
+#pragma unroll
+    for (int f = 0; f < NO; ++f)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if constexpr (SC) S.carry[(f * 4 + q) * 3 + i][tid] = 0;
+                else rcarry[f][q][i] = 0;
+            }
+
+    // Output mode `s` of field c from the element's input modes xv.
+    auto out_mode = [&](const int (&xv)[NI * 8][3], int c, int s, const int (&E)[3], int (&y)[3]) {
+        FxAcc acc{0, 0, 0};
+        if constexpr (DO_K) {
+#pragma unroll
+            for (int j = 0; j < 24; ++j)
+                if (PP.k[c * 8 + s][j] >= 0 && (j & 7) != 0) {
+                    const int* k = F.k[PP.k[c * 8 + s][j]];
+                    gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+                }
+            int r[3];
+            gm_fx_carry(acc, r);
+            FxAcc ae{0, 0, 0};
+            gm_fx_mac(ae, r, E[2], E[1], E[0]);
+            gm_fx_carry(ae, y);
+        } else if constexpr (DO_APU) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (PP.a[c * 8 + s][j] >= 0) {
+                    const int* k = F.a[PP.a[c * 8 + s][j]];
+                    gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+                }
+            gm_fx_carry(acc, y);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 24; ++j)
+                if (PP.a[j][s] >= 0 && (j & 7) != 0) {
+                    const int* k = F.a[PP.a[j][s]];
+                    gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+                }
+            gm_fx_carry_signed(acc, y);
+        }
+    };
+
+    // Layer kb between planes kb and kb + 1 of the ring.  With `plane`, field by
+    // field: complete the face tuples of plane kb, transform them back and
+    // exchange; in any case the layer's top contributions become the carry.
+    int low[NO][3];
+    auto layer = [&](int kb, bool exists, bool plane) {
+        const bool work = exists && fval;
+        int xv[NI * 8][3];
+        int E[3] = {0, 0, 0};
+        if (work) {
+            double Ed = 0.0;
+            if constexpr (DO_K) Ed = a.E[fi + (long long)g.nx * (fj + (long long)g.ny * layer_index(kb))];
+            const int sb = (kb - kbeg) % 3, st = (kb + 1 - kbeg) % 3;
+#pragma unroll
+            for (int f = 0; f < NI; ++f) {
+                int b[4][3], t[4][3];
+                fwd_xy(sb, f, b);
+                fwd_xy(st, f, t);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        xv[f * 8 + q][i] = b[q][i] + t[q][i];
+                        xv[f * 8 + q + 4][i] = b[q][i] - t[q][i];
+                    }
+            }
+            if constexpr (DO_K) gm_fx_coef(Ed, F.topE, E);
+        }
+#pragma unroll
+        for (int c = 0; c < NO; ++c) {
+            int o[4][3];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+                if (work) {
+                    if (DO_AUP || q != 0) out_mode(xv, c, q, E, lo);   // mode 0 of u carries no force
+                    out_mode(xv, c, q + 4, E, hi);
+                }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if constexpr (SC) {
+                        int& cy = S.carry[(c * 4 + q) * 3 + i][tid];
+                        o[q][i] = cy + lo[i] + hi[i];
+                        cy = lo[i] - hi[i];
+                    } else {
+                        o[q][i] = rcarry[c][q][i] + lo[i] + hi[i];
+                        rcarry[c][q][i] = lo[i] - hi[i];
+                    }
+                }
+            }
+            if (plane) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const int c0 = o[0][i] + o[1][i], c1 = o[0][i] - o[1][i];
+                    const int d0 = o[2][i] + o[3][i], d1 = o[2][i] - o[3][i];
+                    const int p10 = __shfl_up_sync(0xffffffffu, c1 + d1, 1, 16);
+                    const int p11 = __shfl_up_sync(0xffffffffu, c1 - d1, 1, 16);
+                    low[c][i] = c0 + d0 + p10;
+                    S.face[kb & 1][c][i][tid] = c0 - d0 + p11;
+                }
+            }
+        }
+    };
+
+    double dot = 0.0;
+    const int gi = x0 - 1 + tx, gj = y0 - 1 + ty;
+    const bool owner = tx >= 1 && ty >= 1 && gi <= g.nx && gj <= g.ny;
+    auto node_stage = [&](int kk) {
+        if (!owner) return;
+        const int node = kk * nb + gj * rowlen + gi;
+        const unsigned m = a.mask[node];
+        const bool lip = g.kf >= 0 && (kk == g.kf || kk == g.kf + 1);
+        // raw value on a tied slave lip: the fault kernel folds it
+        const bool slave = DO_AUP && g.tied && kk == g.kf + 1;
+#pragma unroll
+        for (int f = 0; f < NO; ++f) {
+            const int(&up)[3][256] = S.face[kk & 1][f];
+            const double v = scale * gm_fx_to_double(low[f][0] + up[0][tid - 16], low[f][1] + up[1][tid - 16],
+                                                     low[f][2] + up[2][tid - 16]);
+            double* y = DO_AUP ? a.yp + node : a.yu + (long long)f * N + node;
+            const bool fixed = !slave && ((m >> (DO_AUP ? 3 : f)) & 1u);
+            if (a.accumulate) {
+                if (!fixed) *y += v;
+            } else {
+                *y = fixed ? 0.0 : v;
+            }
+            if constexpr (DOT)
+                if (!lip && !fixed) dot = fma(a.xu[(long long)f * N + node], v, dot);
+        }
+    };
+
+    // Plane k sits in ring slot (k - kbeg) % 3.  While layer kk is computed,
+    // plane kk + 2 is on its way into registers; it is stored over plane kk - 1,
+    // which nobody reads after this iteration's barrier.  The nodes of plane
+    // kk - 1 are written after that barrier too, so a layer needs one barrier.
+    fetch(kbeg);
+    store(0);
+    if (kbeg + 1 <= kend) {
+        fetch(kbeg + 1);
+        store(1);
+    }
+    for (int kk = kbeg; kk < z1; ++kk) {
+        const bool next = kk + 2 <= kend;
+        if (next) fetch(kk + 2);
+        __syncthreads();
+        if (kk > z0) node_stage(kk - 1);
+        layer(kk, layer_exists(kk), kk >= z0);
+        if (next) store((kk + 2 - kbeg) % 3);
+    }
+    __syncthreads();
+    node_stage(z1 - 1);
+    if constexpr (DOT) gm_cta_dot(dot, s_dot, a.part);
+}

@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "gm_fixed.cuh"
 #include "gm_internal.cuh"
 
 #define GM_VERSION "gm-gb300 0.1"
@@ -123,12 +124,63 @@ bool ref_cell(const double h[3], const double sh[2], double nu, double K[24][24]
 
 inline double hsgn(int s, int a) { return (gm_popc3(s & a) & 1) ? -1.0 : 1.0; }
 
+// signed limbs of v 2^-e (|v| < 2^e), v = hi + lo, to 78 bits
+void fx_limbs(double hi, double lo, int e, int (&l)[3])
+{
+    __int128 n = (__int128)std::nearbyint(std::ldexp(hi, 78 - e)) + (__int128)std::nearbyint(std::ldexp(lo, 78 - e));
+    const int sg = n < 0 ? -1 : 1;
+    if (n < 0) n = -n;
+    l[0] = sg * (int)(n & GM_FX_MASK);
+    l[1] = sg * (int)((n >> GM_FX_RADIX) & GM_FX_MASK);
+    l[2] = sg * (int)(n >> (2 * GM_FX_RADIX));
+}
+
+// Fixed-point copy of the reference operators: scaled by the power of two that
+// bounds the absolute sum of every row (twice that for the couplings).
+void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat& PP, double alpha, double Emin,
+             double Emax, RefFx& F)
+{
+    std::memset(&F, 0, sizeof(F));
+    double ks = 0.0, as = 0.0;
+    for (int i = 0; i < 24; ++i) {
+        double t = 0.0, u = 0.0;
+        for (int j = 0; j < 24; ++j)
+            if (PP.k[i][j] >= 0) t += std::fabs(Kt[i][j]);
+        for (int j = 0; j < 8; ++j)
+            if (PP.a[i][j] >= 0) u += std::fabs(alpha * At[i][j]);
+        ks = std::max(ks, t);
+        as = std::max(as, u);
+    }
+    for (int j = 0; j < 8; ++j) {
+        double u = 0.0;
+        for (int i = 0; i < 24; ++i)
+            if (PP.a[i][j] >= 0) u += std::fabs(alpha * At[i][j]);
+        as = std::max(as, u);
+    }
+    F.eK = ks > 0.0 ? std::ilogb(ks) + 1 : 0;
+    F.eA = (as > 0.0 ? std::ilogb(as) + 1 : 0) + 1;
+    for (int i = 0; i < 24; ++i) {
+        for (int j = 0; j < 24; ++j)
+            if (PP.k[i][j] >= 0) fx_limbs(Kt[i][j], 0.0, F.eK, F.k[PP.k[i][j]]);
+        for (int j = 0; j < 8; ++j)
+            if (PP.a[i][j] >= 0) {
+                const double hi = alpha * At[i][j];
+                fx_limbs(hi, std::fma(alpha, At[i][j], -hi), F.eA, F.a[PP.a[i][j]]);
+            }
+    }
+    // moduli: limbs are exact while the smallest is within 2^25 of the largest;
+    // what a low modulus loses against the tile's unit comes off the grading
+    F.topE = std::ilogb(Emax) + 1023;
+    F.gradeK = GM_FX_GRADE - (std::ilogb(Emax) - std::ilogb(Emin));
+    F.gradeA = GM_FX_GRADE;
+}
+
 // Parity transform and packing of the entries the class's pattern allows;
 // returns false if an entry outside the pattern is not negligible (the cell
 // does not belong to the class, or the pattern rule does not hold).
 template <int CLS>
 bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8],
-              const double L[8][8], RefOps<double>& R)
+              const double L[8][8], RefOps<double>& R, RefFx& F, double alpha, double Emin, double Emax)
 {
     constexpr ParPat PP = gm_make_parpat(CLS);
     static double Kt[24][24], At[24][8], Mt[8][8], Lt[8][8];   // index (c*8+s)
@@ -188,6 +240,7 @@ bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8
             if (PP.l[i][j] >= 0) R.L[PP.l[i][j]] = Lt[i][j];
             else if (std::fabs(Lt[i][j]) > tol * lmax) return false;
         }
+    make_fx(Kt, At, PP, alpha, Emin, Emax, F);
     return true;
 }
 
@@ -823,9 +876,11 @@ int bind_impl(gm_ctx* c)
            : (c->shear[1] == 0.0 ? GM_CLS_MONO : GM_CLS_GEN);
     static double K[24][24], A[24][8], M[8][8], L[8][8];
     if (!ref_cell(c->h, c->shear, c->nu, K, A, M, L)) return c->set_err(GM_EINVAL, "bind: degenerate cell");
-    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64)
-            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64)
-                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64);
+    const auto Er = std::minmax_element(c->E.begin(), c->E.end());
+    const double E0 = *Er.first, E1 = *Er.second;
+    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1)
+            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1)
+                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1);
     if (!ok) return c->set_err(GM_EINVAL, "bind: cell operators break the expected parity pattern");
     cast_ref(c->R64, c->R32);
     for (int i = 0; i < GM_PP_MAXK; ++i) c->R32p.K[i] = make_float2(c->R32.K[i], c->R32.K[i]);
@@ -896,11 +951,10 @@ int bind_impl(gm_ctx* c)
     if (const char* pp = std::getenv("GM_PAIR_PREC")) c->pair_prec = std::atoi(pp) != 0;
     // reduction partials: the fixed-grid reductions use 2 * GM_RED_BLOCKS slots,
     // a fused PCG step one per bulk CTA plus one per fault block
-    // (bulk kernels: at most one CTA per 15 x 15 tile and pair of node planes)
+    // (bulk kernels: at most one CTA per 15 x 15 tile and node plane)
     const int gxp = (c->nx + 1 + 14) / 15, gyp = (c->ny + 1 + 14) / 15;
     const long long xyp = (long long)gxp * gyp;
-    const long long zcp = c->zchunk_override > 0 ? std::min<long long>(2, c->zchunk_override) : 2LL;
-    c->bulk_grid = (int)(xyp * ((c->g.nplanes + zcp - 1) / zcp));
+    c->bulk_grid = (int)(xyp * c->g.nplanes);
     const size_t part_bytes = (size_t)8 * std::max<long long>(4LL * GM_RED_BLOCKS,
                                                               c->bulk_grid + (c->g.nb + 255) / 256 + 64);
     struct A_ { DevBuf* b; size_t bytes; } allocs[] = {
@@ -1001,6 +1055,8 @@ int bind_impl(gm_ctx* c)
     }
     c->bound = true;   // loads upload below needs the grid
     int rc = gm_prepare_bulk32(c);
+    if (rc) return rc;
+    rc = gm_prepare_fx(c);
     if (rc) { c->bound = false; return rc; }
     rc = upload_loads(c);
     if (rc) { c->bound = false; return rc; }

@@ -160,6 +160,18 @@ struct RefPairs32 {
     float2 L[GM_PP_MAXL];
 };
 
+// The pattern entries of K_b and of alpha A as signed 26-bit limbs (gm_fixed.cuh,
+// least significant first): entry = (limbs as a fraction) 2^eK or 2^eA, scaled so
+// that the absolute sum of a row is at most 1 (K) or 1/2 (A: 36 results meet in
+// a node).  topE is the biased exponent of the largest Young's modulus; gradeK,
+// gradeA the grading of an input inside a tile, in bits, up to which the
+// fixed-point error stays below the rounding of FP64.
+struct RefFx {
+    int k[GM_PP_MAXK][3];
+    int a[GM_PP_MAXA][3];
+    int eK, eA, topE, gradeK, gradeA;
+};
+
 // Per-node mask bits: 1,2,4 = ux,uy,uz fixed, 8 = p fixed.
 // Tied upper-lip pressures are slaves (handled by index, not by this mask).
 
@@ -208,6 +220,10 @@ struct BulkArgs {
     // storage block uses cS + cFS * fs[e] instead of cS when fs is non-null
     const T* fs;
     T cFS;
+    // FP64 blocks launched one by one: the block's factor (alpha is in its
+    // coefficients), and whether it adds to the output or overwrites it
+    T cfx;
+    int accumulate;
 };
 
 template <typename T>
@@ -401,6 +417,7 @@ struct gm_ctx {
     RefOps<double> R64{};
     RefOps<float> R32{};
     RefPairs32 R32p{};
+    RefFx Rfx{};
     double Kblk_ref[8][9] = {};   // nodal 3x3 diagonal blocks of K_ref (E = 1)
     double Mdiag_ref[8] = {}, Ldiag_ref[8] = {};
     double Aq = 0, nrm[3] = {0, 0, 1}, t1[3] = {1, 0, 0}, t2[3] = {0, 1, 0};
@@ -512,6 +529,7 @@ int gm_launch_diag(gm_ctx* c, cudaStream_t s);            // dK (bulk), dA (need
 int gm_launch_block_jacobi(gm_ctx* c, cudaStream_t s);    // K_T 3x3 inverse blocks
 // multigrid preconditioner of the FP32 K_T solves (gm_mg.cu)
 int gm_prepare_bulk32(gm_ctx* c);                     // kernel attributes, at bind
+int gm_prepare_fx(gm_ctx* c);
 int gm_launch_bulk_k_f32(gm_ctx* c, const float* x, float* y, cudaStream_t s, const int* skip);
 int gm_launch_bulk_k_f64(gm_ctx* c, const double* x, double* y, cudaStream_t s, const int* skip);
 int gm_mg_prepare(gm_ctx* c, int prec, cudaStream_t s);   // GM_EINVAL: grid not coarsenable (caller falls back)
