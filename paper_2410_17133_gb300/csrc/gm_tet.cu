@@ -1,7 +1,9 @@
-// Matrix-free operators on unstructured P1 tetrahedra (include/gm_tet.h).
+// Operators on unstructured P1 tetrahedra (include/gm_tet.h).
 //
 // Each element's shape-function gradients G (4 x 3, constant on the element)
-// and volume V are computed once on the host.  An apply runs one thread per
+// and volume V are computed once on the host.  The operators are assembled from
+// them into block rows when mesh and materials are set (gm_tet_csr.cuh).  A mesh
+// whose rows do not fit the device is applied matrix-free, one warp per
 // node: the node walks its incident (element, local vertex) list in a fixed
 // order, recomputes that element's strain / pressure sums from the element's
 // four vertices and adds the element's row for itself.  No atomics, so the
@@ -14,6 +16,7 @@
 //   C:    y_a = (k/mu) V g_a . sum_b g_b p_b
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -140,12 +143,14 @@ struct DBuf {
         if (e != cudaSuccess) p = nullptr;
         return e;
     }
+    void drop() { if (p) cudaFree(p); p = nullptr; }
     template <typename T> T* as() const { return static_cast<T*>(p); }
 };
 
 }  // namespace
 
 #include "gm_tet_pcg.cuh"
+#include "gm_tet_csr.cuh"
 
 // Largest node, tetrahedron or fault-triangle count: all device index arithmetic
 // (12 gradients per element, 9 frame entries per pair, 3N field offsets) is in
@@ -160,6 +165,10 @@ struct gm_tet {
     bool has_mesh = false, has_mat = false;
     double E = 0, nu = 0, alpha = 0, Mb = 0, k = 0, mu_f = 0;
     DBuf G64, G32, V64, V32, tets, rowptr, adj;
+    // assembled rows (gm_tet_csr.cuh); false where they do not fit the device
+    bool csr_ready = false;
+    long long nnz = 0;
+    DBuf crow, ccol, cK64, cA64, cSC64, cK32, cA32, cSC32;
     // time stepping
     std::vector<double> hG, hV;            // element gradients and volumes (host copy)
     std::vector<double> hX;                // node coordinates (host copy, point-major)
@@ -167,7 +176,7 @@ struct gm_tet {
     std::vector<uint8_t> fixed;            // 4N: constrained (ux, uy, uz, p)
     std::vector<double> fu;                // 3N nodal forces
     DBuf mask, dfu, Kinv, Sd, Cd, part;
-    DBuf w[15];
+    DBuf w[16];
     DBuf pcg_st, pcg_part;                  // device-resident PCG: state and reduction partials
     bool prec_ready = false;
     // fault: interface elements on the fault triangles
@@ -206,6 +215,65 @@ struct gm_tet {
     }
     int set_err(int code, const std::string& m) { err = m; return code; }
 };
+
+namespace {
+
+// Assemble the operators once mesh and materials are there (structure per mesh,
+// values per material).  Rows that would take more than half of the free device
+// memory, or an allocation that fails, leave csr_ready false: products then
+// walk the elements.
+void tet_assemble(gm_tet* t)
+{
+    t->csr_ready = false;
+    if (!t->has_mesh || !t->has_mat) return;
+    cudaSetDevice(t->device);
+    const int N = (int)t->N;
+    const unsigned wblocks = (unsigned)((N + 3) / 4);
+    DBuf count, rows;
+    auto give_up = [&]() {
+        (void)cudaGetLastError();
+        t->nnz = 0;
+        for (DBuf* b : {&t->crow, &t->ccol, &t->cK64, &t->cA64, &t->cSC64, &t->cK32, &t->cA32, &t->cSC32}) b->drop();
+    };
+    cudaDeviceSynchronize();      // products in flight may read the arrays that change below
+    if (t->nnz == 0) {
+        if (count.alloc((size_t)N * 4) != cudaSuccess) return give_up();
+        tcsr_neighbours<<<wblocks, 128>>>(N, t->rowptr.as<int>(), t->adj.as<int>(), t->tets.as<int>(), count.as<int>(),
+                                          nullptr, nullptr, nullptr);
+        std::vector<int> h(N + 1, 0);
+        if (cudaMemcpy(h.data() + 1, count.p, (size_t)N * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return give_up();
+        long long nnz = 0;
+        for (int n = 0; n < N; ++n) nnz += h[n + 1];
+        size_t free_b = 0, total_b = 0;
+        if (nnz >= (1LL << 31) - 1 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+            (double)nnz * (17 * 12 + 8) > 0.5 * (double)free_b)
+            return give_up();
+        for (int n = 0; n < N; ++n) h[n + 1] += h[n];
+        if (t->crow.put(h.data(), h.size() * 4) != cudaSuccess || t->ccol.alloc(nnz * 4) != cudaSuccess ||
+            t->cK64.alloc(nnz * 72) != cudaSuccess || t->cA64.alloc(nnz * 48) != cudaSuccess ||
+            t->cSC64.alloc(nnz * 16) != cudaSuccess || t->cK32.alloc(nnz * 36) != cudaSuccess ||
+            t->cA32.alloc(nnz * 24) != cudaSuccess || t->cSC32.alloc(nnz * 8) != cudaSuccess)
+            return give_up();
+        t->nnz = nnz;
+    }
+    const long long nnz = t->nnz;
+    if (rows.alloc(nnz * 4) != cudaSuccess) return give_up();
+    tcsr_neighbours<<<wblocks, 128>>>(N, t->rowptr.as<int>(), t->adj.as<int>(), t->tets.as<int>(), nullptr,
+                                      t->crow.as<int>(), t->ccol.as<int>(), rows.as<int>());
+    const double lam = t->E * t->nu / ((1 + t->nu) * (1 - 2 * t->nu)), mu = t->E / (2 * (1 + t->nu));
+    tcsr_values<<<(unsigned)((nnz + 127) / 128), 128>>>(nnz, t->rowptr.as<int>(), t->adj.as<int>(), t->tets.as<int>(),
+                                                        t->G64.as<double>(), t->V64.as<double>(), t->crow.as<int>(),
+                                                        t->ccol.as<int>(), rows.as<int>(), lam, mu, t->alpha,
+                                                        1.0 / t->Mb, t->k / t->mu_f, t->cK64.as<double>(),
+                                                        t->cA64.as<double>(), t->cSC64.as<double>());
+    tcsr_cast<<<608, 256>>>(9 * nnz, t->cK64.as<double>(), t->cK32.as<float>());
+    tcsr_cast<<<608, 256>>>(6 * nnz, t->cA64.as<double>(), t->cA32.as<float>());
+    tcsr_cast<<<608, 256>>>(2 * nnz, t->cSC64.as<double>(), t->cSC32.as<float>());
+    if (cudaDeviceSynchronize() != cudaSuccess) return give_up();
+    t->csr_ready = true;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -308,6 +376,8 @@ int gm_tet_mesh(gm_tet* t, const double* nodes, int64_t n_nodes, const int64_t* 
     t->has_fault = false;
     t->fault_ready = false;
     t->has_mesh = true;
+    t->nnz = 0;
+    tet_assemble(t);
     return GM_OK;
 }
 
@@ -320,6 +390,7 @@ int gm_tet_materials(gm_tet* t, double E, double nu, double alpha, double M, dou
     t->has_mat = true;
     t->prec_ready = false;
     t->fault_ready = false;
+    tet_assemble(t);
     return GM_OK;
 }
 
@@ -327,14 +398,46 @@ int gm_tet_materials(gm_tet* t, double E, double nu, double alpha, double M, dou
 
 namespace {
 
+template <typename T>
+TetCsr<T> csr(const gm_tet* t)
+{
+    if constexpr (sizeof(T) == 8)
+        return {t->crow.as<int>(), t->ccol.as<int>(), t->cK64.as<T>(), t->cA64.as<T>(), t->cSC64.as<T>()};
+    else
+        return {t->crow.as<int>(), t->ccol.as<int>(), t->cK32.as<T>(), t->cA32.as<T>(), t->cSC32.as<T>()};
+}
+
 template <typename T, int MODE>
 void launch(gm_tet* t, const TetCoef<T>& c, const T* xu, const T* xp, T* yu, T* yp, cudaStream_t s, const T* G,
             const T* V, const int* skip)
 {
     const int N = (int)t->N;
+    if (t->csr_ready) {
+        tcsr_apply<T, MODE, false><<<(unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s>>>(
+            N, csr<T>(t), c.cApu, c.cC, xu, xp, yu, yp, skip, TetDir<T>{});
+        return;
+    }
     const unsigned blocks = (unsigned)((32LL * N + 127) / 128);   // one warp per node
     gm_tet_apply_kernel<T, MODE><<<blocks, 128, 0, s>>>(N, t->rowptr.as<int>(), t->adj.as<int>(), t->tets.as<int>(), G,
                                                         V, c, xu, xp, yu, yp, skip);
+}
+
+// One PCG product by rows: p_new = z + beta p_old, q = K p_new with constrained
+// entries 0, and alpha; false (nothing launched) without the assembled rows.
+template <typename T>
+bool apply_k_dir(gm_tet* t, const TetDir<T>& d, T* q, cudaStream_t s)
+{
+    if (!t->csr_ready) return false;
+    const int N = (int)t->N;
+    tcsr_apply<T, TM_K, true><<<(unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s>>>(
+        N, csr<T>(t), T(1), T(0), nullptr, nullptr, q, nullptr, &d.st->done, d);
+    return true;
+}
+
+// partials of the PCG reductions: the vector kernels' blocks or the product's
+size_t pcg_part_bytes(const gm_tet* t)
+{
+    return 2 * sizeof(double) * (size_t)std::max<long long>(TPCG_BLOCKS, (8 * t->N + TPCG_NT - 1) / TPCG_NT);
 }
 
 // skip: if non-null, the kernel does nothing while *skip != 0
@@ -467,13 +570,17 @@ struct Stepper {
     void xpby(long long n, const double* x, double b, double* y) { tet_xpby<<<TET_RED_BLOCKS, 256, 0, s>>>(n, x, b, y); }
 
     // x = K^-1 b (x from 0), PCG with 3x3 nodal block Jacobi to ||r|| <= rtol ||b||,
-    // device-resident (scratch 0-3 and 14)
+    // device-resident (scratch 0-3, 14 and 15)
     int solve_k(const double* b, double* x, double rtol, int maxit, long long* its) {
         TetPcg<double> e{N, s, t->w[14].as<double>(), t->w[0].as<double>(), t->w[1].as<double>(),
                          t->w[2].as<double>(), t->w[3].as<double>(), t->pcg_st.as<TetPcgState>(),
                          t->pcg_part.as<double>(),
                          TetPrecT<double>{N, 0, t->Kinv.as<double>(), nullptr, nullptr, nullptr, nullptr},
                          t->mask.as<uint8_t>()};
+        if (t->csr_ready) {
+            e.p2 = t->w[15].as<double>();
+            e.step_by_rows = [t = t](const TetDir<double>& d, double* q, cudaStream_t cs) { apply_k_dir<double>(t, d, q, cs); };
+        }
         const int rc = e.solve(
             b, x, rtol, maxit, its,
             [&](const double* p, double* q, const int* skip, cudaStream_t cs) {
@@ -539,7 +646,7 @@ int tet_prepare(gm_tet* t)
         (ce = t->Cd.put(Cd.data(), N * 8)) != cudaSuccess || (ce = t->mask.put(mk.data(), N)) != cudaSuccess ||
         (ce = t->dfu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (ce = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
         (ce = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
-        (ce = t->pcg_part.alloc(2 * TPCG_BLOCKS * sizeof(double))) != cudaSuccess)
+        (ce = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
         return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(ce));
     for (auto& b : t->w)
         if ((ce = b.alloc(3 * N * 8)) != cudaSuccess)
@@ -1028,7 +1135,7 @@ int tetf_prepare(gm_tet* t)
         (ce = t->f_Pinv.alloc(36 * P * 8)) != cudaSuccess || (ce = t->f_Pinv32.alloc(36 * P * 4)) != cudaSuccess ||
         (ce = t->f_Kinv32.alloc(9 * N * 4)) != cudaSuccess || (ce = t->f_D32.alloc(6 * P * 4)) != cudaSuccess ||
         (ce = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
-        (ce = t->pcg_part.alloc(2 * TPCG_BLOCKS * sizeof(double))) != cudaSuccess)
+        (ce = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
         return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
     for (auto& b : t->fw)
         if ((ce = b.alloc(3 * N * 8)) != cudaSuccess)
