@@ -44,6 +44,27 @@ constexpr size_t gm_fx_smem()
                                                                      : sizeof(BulkTileSmem<double, MODE>);
 }
 
+// Output mode s of displacement field c of one element with modulus limbs E:
+// K_b row times the element's input modes, times E.
+template <int CLS>
+__device__ __forceinline__ void gm_fx_k_mode(const RefFx& F, const int (&xv)[24][3], int c, int s, const int (&E)[3],
+                                             int (&y)[3])
+{
+    constexpr ParPat PP = gm_make_parpat(CLS);
+    FxAcc acc{0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 24; ++j)
+        if (PP.k[c * 8 + s][j] >= 0 && (j & 7) != 0) {
+            const int* k = F.k[PP.k[c * 8 + s][j]];
+            gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+        }
+    int r[3];
+    gm_fx_carry(acc, r);
+    FxAcc ae{0, 0, 0};
+    gm_fx_mac(ae, r, E[2], E[1], E[0]);
+    gm_fx_carry(ae, y);
+}
+
 // The FP64 tile as a function of its own: it needs twice the registers, and
 // inlined its spills would reach into the fixed-point part.
 template <int CLS, int MODE>
@@ -218,17 +239,7 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
     auto out_mode = [&](const int (&xv)[NI * 8][3], int c, int s, const int (&E)[3], int (&y)[3]) {
         FxAcc acc{0, 0, 0};
         if constexpr (DO_K) {
-#pragma unroll
-            for (int j = 0; j < 24; ++j)
-                if (PP.k[c * 8 + s][j] >= 0 && (j & 7) != 0) {
-                    const int* k = F.k[PP.k[c * 8 + s][j]];
-                    gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
-                }
-            int r[3];
-            gm_fx_carry(acc, r);
-            FxAcc ae{0, 0, 0};
-            gm_fx_mac(ae, r, E[2], E[1], E[0]);
-            gm_fx_carry(ae, y);
+            gm_fx_k_mode<CLS>(F, xv, c, s, E, y);
         } else if constexpr (DO_APU) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)

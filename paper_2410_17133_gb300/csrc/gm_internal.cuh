@@ -392,6 +392,7 @@ struct MGLevel {
     double lmax = 0.0;       // largest eigenvalue estimate of M^-1 K_T
     int deg = 2;             // Chebyshev degree of the smoother (of the solve on the coarsest level)
     int coef_off = 0;        // first (c1, c2) pair of this level in mg_coef
+    int cluster32 = 0, cluster64 = 0;   // CTAs of the coarsest level's cluster kernel (0: not used)
 };
 
 struct gm_ctx {

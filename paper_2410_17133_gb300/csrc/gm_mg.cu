@@ -288,6 +288,12 @@ __global__ void __launch_bounds__(256) mg_cheb_kernel(long long N, const T* b, c
     }
 }
 
+}  // namespace
+
+#include "gm_mg_coarse.cuh"
+
+namespace {
+
 // Per-block partial sums of v.v (set-up only; summed on the host in block order).
 __global__ void __launch_bounds__(256) mg_norm2_kernel(long long n, const float* v, double* part)
 {
@@ -498,13 +504,80 @@ int smooth(gm_ctx* c, const MGLevel& L, int deg, bool xzero, const int* skip, cu
     return GM_OK;
 }
 
+// The coarsest level's polynomial as one cluster kernel where that is the faster
+// way: its rows fit the CTAs' shared memory, the smoother's pair threads add the
+// fault rows, and a CTA has few elements (FP32: 4,096, FP64: 1,024; beyond, a product spread over all
+// SMs wins).  Called at set-up: it sets kernel attributes, outside any capture.
+template <typename T, int CLS>
+int coarse_cluster(gm_ctx* x)
+{
+    using MT = typename MinvType<T>::type;
+    if (x->g.kf >= 0 && !x->pair_prec) return 0;
+    const int n = mgc_setup<T, MT, CLS>(x->device);
+    if (n == 0) return 0;
+    const int rows = (x->ny + n) / n;            // ceil((ny + 1) / n)
+    if (mgc_layout<T, MT>(x->g, rows, false).total > MGC_SMEM) return 0;
+    const long long rn = (long long)(x->nx + 1) * x->g.nplanes, faces = (long long)x->nx * x->nz;
+    if (rn * 3 * (rows + 2) >= 65536 || faces * 6 * rows >= 65536) return 0;     // quotients by multiplication
+    const long long work = 2LL * rows * faces;
+    return work <= (sizeof(T) == 8 ? 1024 : 4096) ? n : 0;
+}
+template <typename T>
+int coarse_cluster(gm_ctx* x)
+{
+    switch (x->cls) {
+    case GM_CLS_BOX: return coarse_cluster<T, GM_CLS_BOX>(x);
+    case GM_CLS_MONO: return coarse_cluster<T, GM_CLS_MONO>(x);
+    default: return coarse_cluster<T, GM_CLS_GEN>(x);
+    }
+}
+
+template <typename T, int CLS>
+int coarse_launch(gm_ctx* c, const MGLevel& L, int n, const int* skip, cudaStream_t s)
+{
+    using MT = typename MinvType<T>::type;
+    gm_ctx* x = L.cx;
+    const LV<T> v = lv<T>(L);
+    const int rows = (x->ny + n) / n;
+    const bool fixedin = mgc_layout<T, MT>(x->g, rows, true).total <= MGC_SMEM;
+    CoarseArgs<T, MT> a{x->g, sizeof(T) == 8 ? (const T*)x->dE64.p : (const T*)x->dE32.p, x->dmask.as<uint8_t>(), v.b, v.x,
+                        level_inv<T>(x), level_pairs<T>(x), level_fault<T>(x),
+                        c->mg_coef.as<double>() + 2 * L.coef_off, L.deg, rows, fixedin ? 1 : 0,
+                        mgc_magic((x->nx + 1) * x->g.nplanes), mgc_magic(x->nx + 1), mgc_magic(x->nx),
+                        mgc_magic(x->nx * x->nz), skip};
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = n;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(mgc_threads<T>());
+    cfg.dynamicSmemBytes = mgc_layout<T, MT>(x->g, rows, fixedin).total;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, mg_coarse_kernel<T, MT, CLS>, a, x->R32, x->Rfx);
+    if (e != cudaSuccess) return c->set_err(GM_ECUDA, std::string("multigrid: coarsest level: ") + cudaGetErrorString(e));
+    x->applies += L.deg - 1;
+    GM_LAUNCHED(c);
+    return GM_OK;
+}
+
 template <typename T>
 int vcycle(gm_ctx* c, size_t l, const int* skip, cudaStream_t s)
 {
     const MGLevel& L = c->mg[l];
     const LV<T> v = lv<T>(L);
     int rc;
-    if (l + 1 == c->mg.size()) return smooth<T>(c, L, L.deg, true, skip, s);
+    if (l + 1 == c->mg.size()) {
+        const int n = sizeof(T) == 8 ? L.cluster64 : L.cluster32;
+        if (n == 0) return smooth<T>(c, L, L.deg, true, skip, s);
+        switch (L.cx->cls) {
+        case GM_CLS_BOX: return coarse_launch<T, GM_CLS_BOX>(c, L, n, skip, s);
+        case GM_CLS_MONO: return coarse_launch<T, GM_CLS_MONO>(c, L, n, skip, s);
+        default: return coarse_launch<T, GM_CLS_GEN>(c, L, n, skip, s);
+        }
+    }
     if ((rc = smooth<T>(c, L, L.deg, true, skip, s))) return rc;
     if ((rc = apply_kt(L.cx, v.x, v.y, skip, s))) return rc;
     const MGLevel& C = c->mg[l + 1];
@@ -646,14 +719,17 @@ int build(gm_ctx* c)
         if ((rc = estimate_lmax(c, L))) { gm_mg_release(c); return rc; }
     c->mg[0].b = nullptr;
     c->mg[0].x = nullptr;
+    MGLevel& last = c->mg.back();
+    last.cluster32 = coarse_cluster<float>(last.cx);
+    last.cluster64 = coarse_cluster<double>(last.cx);
     int off = 1;
     for (size_t l = 0; l < c->mg.size(); ++l) {
         MGLevel& L = c->mg[l];
-        const bool last = l + 1 == c->mg.size();
-        L.deg = last ? mg_coarse_deg() : mg_smooth_deg();
+        const bool coarsest = l + 1 == c->mg.size();
+        L.deg = coarsest ? mg_coarse_deg() : mg_smooth_deg();
         L.coef_off = off;
         const double hi = 1.15 * L.lmax;
-        const double lo = (last ? mg_frac("GM_MG_COARSE_LO", 0.003) : mg_frac("GM_MG_SMOOTH_LO", 0.15)) * L.lmax;
+        const double lo = (coarsest ? mg_frac("GM_MG_COARSE_LO", 0.003) : mg_frac("GM_MG_SMOOTH_LO", 0.15)) * L.lmax;
         cheb_coefs(lo, hi, L.deg, coef);
         off += L.deg;
     }

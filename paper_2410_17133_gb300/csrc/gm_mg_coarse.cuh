@@ -1,0 +1,426 @@
+// The whole Chebyshev polynomial of the coarsest multigrid level in one launch.
+//
+// The coarsest grid (10 to 19 cells per direction) has a few thousand nodes and a
+// polynomial of degree 24: as 47 launches of a K_b product or an update it took
+// two thirds of the launches of a V-cycle, each one bound by its own latency
+// (about 4 us in FP32 and 15 us in FP64 at 12^3..16^3, where the work is a few
+// hundred nanoseconds of the chip).  Here one thread-block cluster runs all
+// steps.  A CTA owns node rows in y (all x and z, so that the fault pairs spread
+// over the CTAs and both lips of a pair are neighbours in one row), keeps their
+// iterate in shared memory, reads the rows beside its own from its neighbours'
+// shared memory, and meets the others once per step at the cluster barrier.
+//
+// What bounds it: latency, so the work of a row is cut into as many independent
+// items as there are: elements of the two layers around the row (FP64: and
+// output fields), then (node, component) twice.  FP32 multiplies in the parity
+// basis like gm_bulk32.cuh; FP64 in wide fixed point like gm_bulkfx.cuh with the
+// unit of the CTA's rows (a preconditioner needs no grading test; values that
+// are not finite give NaN).  The march direction is y here: a mode's bit 1
+// (s & 2) separates a layer's lower and upper rows.
+// Included by gm_mg.cu only.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "gm_bulkfx.cuh"
+
+namespace {
+
+template <typename T>
+__host__ __device__ constexpr int mgc_threads() { return sizeof(T) == 8 ? 384 : 512; }
+template <typename T>
+__host__ __device__ constexpr int mgc_limbs() { return sizeof(T) == 8 ? 3 : 1; }
+
+template <typename T, typename MT>
+struct CoarseArgs {
+    GridDesc g;
+    const T* E;
+    const uint8_t* mask;
+    const T* b;
+    T* x;                // result
+    const MT* mi;
+    PairPrec<T> pp;
+    FaultK<T> fk;
+    const double* coef;  // (c1, c2) per step
+    int deg, rows;       // rows of a CTA at most
+    int fixedin;         // b and the nodal inverses are copied to shared memory
+    unsigned m_rn, m_rowlen, m_nx, m_faces;   // ceil(2^32 / d): quotients by one multiplication
+    const int* skip;
+};
+
+// x / d for x < 2^16, d < 2^16 with m = ceil(2^32 / d): exact, since x (m d - 2^32) < 2^32
+__device__ inline int mgc_div(int x, unsigned m) { return (int)__umulhi((unsigned)x, m); }
+inline unsigned mgc_magic(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ull + d - 1) / d); }
+
+// first node row of CTA r of n: the first CTAs take one row more, so that
+// neighbouring rows are in neighbouring CTAs also where some have none
+__host__ __device__ inline int mgc_row(const GridDesc& g, int r, int n)
+{
+    const int q = (g.ny + 1) / n, rem = (g.ny + 1) % n;
+    return r * q + (r < rem ? r : rem);
+}
+
+// Shared memory of a CTA in bytes from the start: iterate (two buffers),
+// direction and residual of its rows, staged rows as words, what the layers
+// around a row give it, modulus and mask of the staged part; with `fixedin` also
+// b and the nodal inverses (the cluster barrier empties the L1 cache, so what is
+// read in every step would come from L2 each time).
+struct MgcLayout {
+    size_t x, d, r, st, out, E, mask, b, mi, total;
+};
+template <typename T, typename MT>
+__host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows, bool fixedin)
+{
+    const size_t rn = (size_t)(g.nx + 1) * g.nplanes, faces = (size_t)g.nx * g.nz, NL = mgc_limbs<T>();
+    MgcLayout L{};
+    size_t at = 0;
+    auto put = [&](size_t bytes) {
+        const size_t p = at;
+        at += (bytes + 15) & ~(size_t)15;
+        return p;
+    };
+    L.x = put(2 * rows * 3 * rn * sizeof(T));
+    L.d = put(rows * 3 * rn * sizeof(T));
+    L.r = put(rows * 3 * rn * sizeof(T));
+    L.st = put((rows + 2) * 3 * NL * rn * 4);
+    L.out = put(rows * 2 * 12 * NL * faces * 4);
+    L.E = put((rows + 1) * faces * sizeof(T));
+    L.mask = put((rows + 2) * rn);
+    if (fixedin) {
+        L.b = put(rows * 3 * rn * sizeof(T));
+        L.mi = put(rows * 6 * rn * sizeof(MT));
+    }
+    L.total = at;
+    return L;
+}
+
+template <typename T, typename MT, int CLS>
+__global__ void __launch_bounds__(mgc_threads<T>(), 1)
+mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_constant__ RefOps<float> R,
+                 const __grid_constant__ RefFx F)
+{
+    constexpr bool FX = sizeof(T) == 8;
+    constexpr int NL = mgc_limbs<T>(), NT = mgc_threads<T>();
+    using W = typename std::conditional<FX, int, float>::type;      // word of a staged value
+    constexpr ParPat PP = gm_make_parpat(CLS);
+    if (a.skip && *a.skip) return;                                  // the same for every CTA
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
+
+    extern __shared__ __align__(16) unsigned char mgc_raw[];
+    __shared__ int s_top[NT / 32];
+    const GridDesc& g = a.g;
+    const MgcLayout L = mgc_layout<T, MT>(g, a.rows, a.fixedin != 0);
+    const int rowlen = g.nx + 1, rn = rowlen * g.nplanes, faces = g.nx * g.nz;
+    const long long N = g.N;
+    const int tid = threadIdx.x;
+    T* sx = reinterpret_cast<T*>(mgc_raw + L.x);                    // [buffer][row][field][node]
+    T* sd = reinterpret_cast<T*>(mgc_raw + L.d);                    // [row][field][node]
+    T* sr = reinterpret_cast<T*>(mgc_raw + L.r);                    // [row][field][node]
+    T* sb = reinterpret_cast<T*>(mgc_raw + L.b);                    // [row][field][node]
+    MT* smi = reinterpret_cast<MT*>(mgc_raw + L.mi);                // [row][entry][node]
+    W* st = reinterpret_cast<W*>(mgc_raw + L.st);                   // [staged row][field][limb][node]
+    W* out = reinterpret_cast<W*>(mgc_raw + L.out);                 // [row][layer][field][corner][limb][face]
+    T* sE = reinterpret_cast<T*>(mgc_raw + L.E);                    // [layer][face]
+    uint8_t* sm = mgc_raw + L.mask;                                 // [staged row][node]
+    const int j0 = mgc_row(g, rank, ncta), j1 = mgc_row(g, rank + 1, ncta), own = j1 - j0;
+    const size_t buf = (size_t)a.rows * 3 * rn;
+
+    // node i + rowlen kk of row j
+    auto node = [&](int n, int j) -> long long {
+        const int kk = mgc_div(n, a.m_rowlen);
+        return (n - kk * rowlen) + (long long)rowlen * (j + (long long)(g.ny + 1) * kk);
+    };
+    if (own > 0) {
+        for (int q = tid; q < (own + 2) * rn; q += NT) {
+            const int sr_ = mgc_div(q, a.m_rn), n = q - sr_ * rn, j = j0 - 1 + sr_;
+            sm[q] = j >= 0 && j <= g.ny ? a.mask[node(n, j)] : (uint8_t)7;
+        }
+        for (int q = tid; q < (own + 1) * faces; q += NT) {
+            const int l = mgc_div(q, a.m_faces), f = q - l * faces, j = j0 - 1 + l;
+            const int ek = mgc_div(f, a.m_nx);
+            sE[q] = j >= 0 && j < g.ny ? a.E[(f - ek * g.nx) + (long long)g.nx * (j + (long long)g.ny * ek)] : T(0);
+        }
+    }
+    if (a.fixedin)
+        for (int row = 0; row < own; ++row)
+            for (int n = tid; n < rn; n += NT) {
+                const long long gn = node(n, j0 + row);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) sb[(size_t)(row * 3 + c) * rn + n] = a.b[c * N + gn];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) smi[(size_t)(row * 6 + k) * rn + n] = a.mi[k * N + gn];
+            }
+    __syncthreads();
+
+    for (int step = 0; step < a.deg; ++step) {
+        const T c1 = (T)a.coef[2 * step], c2 = (T)a.coef[2 * step + 1];
+        const T* xi = sx + (step & 1 ? 0 : buf);                    // written by the step before
+        T* xo = sx + (step & 1 ? buf : 0);
+        double scale = 0.0;
+        if (step > 0 && own > 0) {
+            // stage rows j0 - 1 .. j1: own rows, and the neighbours' nearest ones
+            int top = 0;
+            const T* from[2] = {xi, xi};
+            if (rank > 0 && j0 > 0) from[0] = cl.map_shared_rank(const_cast<T*>(xi), rank - 1) +
+                                              (size_t)(j0 - 1 - mgc_row(g, rank - 1, ncta)) * 3 * rn;
+            if (rank + 1 < ncta && j1 <= g.ny) from[1] = cl.map_shared_rank(const_cast<T*>(xi), rank + 1);
+            const int count = (own + 2) * rn;
+            auto value = [&](int q, int f) -> T {
+                const int r = mgc_div(q, a.m_rn), n = q - r * rn, j = j0 - 1 + r;
+                if (j < 0 || j > g.ny || ((sm[q] >> f) & 1u)) return T(0);
+                const T* p = r == 0 ? from[0] : r == own + 1 ? from[1] : xi + (size_t)(r - 1) * 3 * rn;
+                return p[(size_t)f * rn + n];
+            };
+            if constexpr (FX) {
+                constexpr int MAXQ = 8;                             // values kept between the two passes
+                T keep[MAXQ];
+#pragma unroll
+                for (int u = 0; u < MAXQ; ++u) {
+                    const int i = tid + u * NT;
+                    keep[u] = T(0);
+                    if (i < 3 * count) {
+                        const int f = (i >= count) + (i >= 2 * count);
+                        keep[u] = value(i - f * count, f);
+                        top = max(top, (__double2hiint(keep[u]) & 0x7fffffff) >> 20);
+                    }
+                }
+                for (int i = tid + MAXQ * NT; i < 3 * count; i += NT) {
+                    const int f = (i >= count) + (i >= 2 * count);
+                    top = max(top, (__double2hiint(value(i - f * count, f)) & 0x7fffffff) >> 20);
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+                if ((tid & 31) == 0) s_top[tid >> 5] = top;
+                __syncthreads();
+#pragma unroll
+                for (int w = 0; w < NT / 32; ++w) top = max(top, s_top[w]);
+                // a field of zeros or subnormals gives zero; not finite gives NaN
+                const int qe = (top - 1022 - GM_FX_IN) + F.eK + F.topE - 1022;
+                scale = top == 0x7ff || qe > 900 ? nan("")
+                      : qe < -1000 || top < 100 ? 0.0 : gm_fx_real((int64_t)(qe + 1023) << 52);
+                auto limbs = [&](int i, T v) {
+                    const int f = (i >= count) + (i >= 2 * count), q = i - f * count, r = mgc_div(q, a.m_rn), n = q - r * rn;
+                    int l[3];
+                    gm_fx_from_double(v, top, l);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) st[((size_t)(r * 3 + f) * 3 + k) * rn + n] = l[k];
+                };
+#pragma unroll
+                for (int u = 0; u < MAXQ; ++u)
+                    if (tid + u * NT < 3 * count) limbs(tid + u * NT, keep[u]);
+                for (int i = tid + MAXQ * NT; i < 3 * count; i += NT) {
+                    const int f = (i >= count) + (i >= 2 * count);
+                    limbs(i, value(i - f * count, f));
+                }
+            } else {
+                for (int q = tid; q < count; q += NT) {
+                    const int r = mgc_div(q, a.m_rn), n = q - r * rn;
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) st[(size_t)(r * 3 + f) * rn + n] = value(q, f);
+                }
+            }
+        }
+        __syncthreads();
+        if (step > 0) {
+            // layer 0: elements below the row (their upper part), layer 1: above it (lower part)
+            constexpr int NC = FX ? 3 : 1;                      // FP64: one output field per item
+            for (int it = tid; it < own * 2 * NC * faces; it += NT) {
+                const int blk = mgc_div(it, a.m_faces), f = it - blk * faces;   // (row, layer, field)
+                const int rl = NC == 1 ? blk : blk / NC, cc = blk - rl * NC;
+                const int row = rl >> 1, lay = rl & 1, j = j0 + row;
+                if (lay == 0 ? j == 0 : j == g.ny) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        if (NC == 1 || c == cc)
+#pragma unroll
+                            for (int q = 0; q < 4 * NL; ++q) out[(size_t)((rl * 3 + c) * 4 * NL + q) * faces + f] = W(0);
+                    continue;
+                }
+                const int ek = mgc_div(f, a.m_nx), fi = f - ek * g.nx;
+                const int nd = fi + rowlen * (ek + (g.kf >= 0 && ek >= g.kf ? 1 : 0));
+                W xv[24][NL];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int l = 0; l < NL; ++l) {
+                        W t[2][4];                              // [ay][sx + 2 sz]
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            const W* v = st + ((size_t)((row + lay + s) * 3 + c) * NL + l) * rn + nd;
+                            const W a0 = v[0] + v[1], a1 = v[0] - v[1];
+                            const W b0 = v[rowlen] + v[rowlen + 1], b1 = v[rowlen] - v[rowlen + 1];
+                            t[s][0] = a0 + b0;
+                            t[s][1] = a1 + b1;
+                            t[s][2] = a0 - b0;
+                            t[s][3] = a1 - b1;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int s0 = (q & 1) | ((q & 2) << 1);     // mode (sx, 0, sz)
+                            xv[c * 8 + s0][l] = t[0][q] + t[1][q];
+                            xv[c * 8 + (s0 | 2)][l] = t[0][q] - t[1][q];
+                        }
+                    }
+                const T Ee = sE[(size_t)(row + lay) * faces + f];
+                int El[3] = {0, 0, 0};
+                if constexpr (FX) gm_fx_coef(Ee, F.topE, El);
+                auto field = [&](auto c_) {
+                    constexpr int c = decltype(c_)::value;
+                    W o[4][NL];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        W lo[NL] = {}, hi[NL];
+                        auto mode = [&](int s, W (&y)[NL]) {
+                            if constexpr (FX) {
+                                gm_fx_k_mode<CLS>(F, xv, c, s, El, y);
+                            } else {
+                                float t = 0.f;
+#pragma unroll
+                                for (int i = 0; i < 24; ++i)
+                                    if (PP.k[c * 8 + s][i] >= 0 && (i & 7) != 0)
+                                        t = fmaf(R.K[PP.k[c * 8 + s][i]], xv[i][0], t);
+                                y[0] = Ee * t;
+                            }
+                        };
+                        const int s0 = (q & 1) | ((q & 2) << 1);
+                        if (s0 != 0) mode(s0, lo);              // the constant mode carries no force
+                        mode(s0 | 2, hi);
+#pragma unroll
+                        for (int l = 0; l < NL; ++l) o[q][l] = lay == 0 ? lo[l] - hi[l] : lo[l] + hi[l];
+                    }
+#pragma unroll
+                    for (int l = 0; l < NL; ++l) {
+                        const W p0 = o[0][l] + o[1][l], p1 = o[0][l] - o[1][l];
+                        const W q0 = o[2][l] + o[3][l], q1 = o[2][l] - o[3][l];
+                        W* w = out + (size_t)((rl * 3 + c) * 4 * NL + l) * faces + f;
+                        w[0] = p0 + q0;                         // corner ax + 2 az
+                        w[(size_t)NL * faces] = p1 + q1;
+                        w[(size_t)2 * NL * faces] = p0 - q0;
+                        w[(size_t)3 * NL * faces] = p1 - q1;
+                    }
+                };
+                if (NC == 1 || cc == 0) field(std::integral_constant<int, 0>{});
+                if (NC == 1 || cc == 1) field(std::integral_constant<int, 1>{});
+                if (NC == 1 || cc == 2) field(std::integral_constant<int, 2>{});
+            }
+            __syncthreads();
+        }
+        // residual r = b - K_T x
+        for (int it = tid; it < own * 3 * rn; it += NT) {
+            const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3, j = j0 + row;
+            const int kk = mgc_div(n, a.m_rowlen), i = n - kk * rowlen;
+            const bool fixed = (sm[(size_t)(row + 1) * rn + n] >> c) & 1u;
+            T r = a.fixedin ? sb[it] : a.b[c * N + i + (long long)rowlen * (j + (long long)(g.ny + 1) * kk)];
+            if (step > 0 && !fixed) {
+                W s[NL];
+#pragma unroll
+                for (int l = 0; l < NL; ++l) s[l] = W(0);
+#pragma unroll
+                for (int dz = 0; dz < 2; ++dz) {                // elements above and below in z
+                    const int kb = kk - dz;
+                    if (kb < 0 || kb + 1 >= g.nplanes || kb == g.kf) continue;
+                    const int ek = (g.kf >= 0 && kb > g.kf) ? kb - 1 : kb;
+#pragma unroll
+                    for (int dx = 0; dx < 2; ++dx) {
+                        const int fi = i - dx;
+                        if (fi < 0 || fi >= g.nx) continue;
+#pragma unroll
+                        for (int lay = 0; lay < 2; ++lay)
+#pragma unroll
+                            for (int l = 0; l < NL; ++l)
+                                s[l] += out[(size_t)((((row * 2 + lay) * 3 + c) * 4 + dx + 2 * dz) * NL + l) * faces + fi + g.nx * ek];
+                    }
+                }
+                if constexpr (FX) r -= scale * gm_fx_to_double(s[0], s[1], s[2]);
+                else r -= s[0];
+                if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) {
+                    // cohesive force +-A_i D [[x]]
+                    const int nl = i + rowlen * g.kf, nu = nl + rowlen;
+                    const int nqi = (i > 0) + (i < g.nx), nqj = (j > 0) + (j < g.ny);
+                    const T Ai = a.fk.Aq * T(0.25) * T(nqi * nqj);
+                    const long long P = g.nb, q = i + (long long)rowlen * j;
+                    T f = T(0);
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) {
+                        const T up = ((sm[(size_t)(row + 1) * rn + nu] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nu];
+                        const T um = ((sm[(size_t)(row + 1) * rn + nl] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nl];
+                        const int lo = c < e ? c : e, hi = c < e ? e : c;
+                        const int k = lo == 0 ? hi : lo + hi + 1;       // 00 01 02 11 12 22
+                        f = fma(a.fk.D[k * P + q], up - um, f);
+                    }
+                    r = kk == g.kf ? fma(Ai, f, r) : fma(-Ai, f, r);
+                }
+            }
+            sr[it] = r;
+        }
+        __syncthreads();
+        // z = M^-1 r, d = c1 d + c2 z, x = x + d
+        for (int it = tid; it < own * 3 * rn; it += NT) {
+            const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3, j = j0 + row;
+            const int kk = mgc_div(n, a.m_rowlen), i = n - kk * rowlen;
+            const long long gn = i + (long long)rowlen * (j + (long long)(g.ny + 1) * kk);
+            T z = T(0);
+            if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) {
+                const int nl = i + rowlen * g.kf, ra = (kk - g.kf) * 3 + c;
+                const long long q = i + (long long)rowlen * j;
+#pragma unroll
+                for (int e = 0; e < 6; ++e)
+                    z = fma(a.pp.inv[(ra * 6 + e) * a.pp.nb + q], sr[(size_t)(row * 3 + e % 3) * rn + nl + (e < 3 ? 0 : rowlen)], z);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    const int lo = c < e ? c : e, hi = c < e ? e : c;
+                    const int k = lo == 0 ? hi : lo + hi + 1;
+                    z = fma(mg_ld<T>(a.fixedin ? smi + (size_t)(row * 6 + k) * rn + n : a.mi + k * N + gn),
+                            sr[(size_t)(row * 3 + e) * rn + n], z);
+                }
+            }
+            const T dn = step > 0 ? fma(c1, sd[it], c2 * z) : c2 * z;
+            const T xn = step > 0 ? xi[it] + dn : dn;
+            sd[it] = dn;
+            if (step + 1 < a.deg) xo[it] = xn;
+            else a.x[c * N + gn] = xn;
+        }
+        // the step's rows are complete; in the last step: nobody reads this CTA's rows any more
+        cl.sync();
+    }
+}
+
+// Cluster size the kernel runs with on this device (0: not available).
+constexpr int MGC_SMEM = 226 * 1024;
+template <typename T, typename MT, int CLS>
+int mgc_setup(int dev)
+{
+    static int size[64] = {};
+    int& r = size[dev & 63];
+    if (r != 0) return r < 0 ? 0 : r;
+    const void* k = (const void*)mg_coarse_kernel<T, MT, CLS>;
+    r = -1;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MGC_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    for (int n : {16, 8}) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = n;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(n);
+        cfg.blockDim = dim3(mgc_threads<T>());
+        cfg.dynamicSmemBytes = MGC_SMEM;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int active = 0;
+        if (cudaOccupancyMaxActiveClusters(&active, k, &cfg) == cudaSuccess && active > 0) {
+            r = n;
+            break;
+        }
+        (void)cudaGetLastError();
+    }
+    return r < 0 ? 0 : r;
+}
+
+}  // namespace
