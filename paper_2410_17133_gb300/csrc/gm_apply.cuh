@@ -374,6 +374,8 @@ static int gm_fx_setup(int dev)
     if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_K, true>, gm_fx_smem<GM_M_K>());
     if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_APU, false>, gm_fx_smem<GM_M_APU>());
     if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_M_AUP, false>, gm_fx_smem<GM_M_AUP>());
+    if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_FX_FLOW, false>, gm_fx_smem<GM_FX_FLOW>());
+    if (!e) e = set((const void*)gm_bulk_fx_kernel<CLS, GM_FX_FLOW, true>, gm_fx_smem<GM_FX_FLOW>());
     if (!e) done[dev & 63] = true;
     return e;
 }
@@ -382,7 +384,8 @@ static int gm_fx_setup(int dev)
 // (two per SM: their registers) marches its planes plus a halo layer, and looks
 // over its inputs first, which costs about half a layer.
 template <int CLS, int MODE, bool DOT>
-static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accumulate, cudaStream_t s)
+static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accumulate, cudaStream_t s,
+                        const FlowFx& Q = FlowFx{})
 {
     const int gx = (c->nx + 1 + 14) / 15, gy = (c->ny + 1 + 14) / 15, np = c->g.nplanes;
     int zc = c->zchunk_override;
@@ -398,27 +401,30 @@ static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accu
     b.zchunk = zc;
     b.cfx = factor;
     b.accumulate = accumulate ? 1 : 0;
-    gm_bulk_fx_kernel<CLS, MODE, DOT><<<dim3(gx, gy, gz), 256, gm_fx_smem<MODE>(), s>>>(b, c->Rfx, c->R64);
+    gm_bulk_fx_kernel<CLS, MODE, DOT><<<dim3(gx, gy, gz), 256, gm_fx_smem<MODE>(), s>>>(b, c->Rfx, c->R64, Q);
     c->applies++;
     c->launches++;
     return gx * gy * gz;
 }
 
-// New search direction p = z + beta p_old of a K_T solve, constrained entries 0
-// (the fixed-point product needs the whole direction before it can scale it).
+// New search direction p = z + beta p_old of a K_T (NC 3) or A22 (NC 1) solve,
+// constrained entries and tied upper-lip pressures 0 (the fixed-point product
+// needs the whole direction before it can scale it).
+template <int NC>
 static __global__ void __launch_bounds__(256)
-gm_pcg_dir_kernel(long long N, const double* z, const double* p_old, double* p, const uint8_t* mask,
+gm_pcg_dir_kernel(GridDesc g, const double* z, const double* p_old, double* p, const uint8_t* mask,
                   const PcgScalars* sc)
 {
     if (sc->done) return;
     const double beta = sc->beta;
+    const long long N = g.N, s0 = (NC == 1 && g.tied) ? g.nb * (g.kf + 1) : -1;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
          n += (long long)gridDim.x * blockDim.x) {
-        const unsigned m = mask[n];
+        const unsigned m = mask[n] | (s0 >= 0 && n >= s0 && n < s0 + g.nb ? 8u : 0u);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < NC; ++c) {
             const long long k = c * N + n;
-            p[k] = ((m >> c) & 1u) ? 0.0 : fma(beta, p_old[k], z[k]);
+            p[k] = ((m >> (NC == 3 ? c : 3)) & 1u) ? 0.0 : fma(beta, p_old[k], z[k]);
         }
     }
 }
@@ -436,16 +442,22 @@ static void gm_apply_launch_t(gm_ctx* c, const RefOps<T>& R, double cK, double c
     b.skip = skip;
     constexpr int BULK = MODE & (GM_M_K | GM_M_APU | GM_M_AUP | GM_M_S | GM_M_C);
     if constexpr (std::is_same<T, double>::value) {
-        // block by block: K_b, A_pu and A_up in fixed point, S and C in FP64
+        // block by block in fixed point
         constexpr int FLOW = BULK & (GM_M_S | GM_M_C);
         if constexpr ((BULK & GM_M_K) != 0) gm_fx_launch<CLS, GM_M_K, false>(c, b, cK, false, s);
         if constexpr ((BULK & GM_M_APU) != 0) gm_fx_launch<CLS, GM_M_APU, false>(c, b, cApu, (BULK & GM_M_K) != 0, s);
         if constexpr (FLOW != 0) {
-            b.zchunk = zchunk;
-            b.accumulate = 0;
-            gm_bulk_apply_kernel<T, CLS, FLOW, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
-            c->applies++;
-            c->launches++;
+            // cS or cC is 0 where the mode has one of the two only
+            const FlowFx Q = gm_flow_fx(c, cS, cC);
+            if (Q.grade >= 0) {
+                gm_fx_launch<CLS, GM_FX_FLOW, false>(c, b, 1.0, false, s, Q);
+            } else {
+                b.zchunk = zchunk;
+                b.accumulate = 0;
+                gm_bulk_apply_kernel<T, CLS, GM_FX_FLOW, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+                c->applies++;
+                c->launches++;
+            }
         }
         if constexpr ((BULK & GM_M_AUP) != 0) gm_fx_launch<CLS, GM_M_AUP, false>(c, b, cAup, FLOW != 0, s);
     } else {
@@ -516,14 +528,24 @@ static void gm_pcg_apply_t(gm_ctx* c, const RefOps<T>& R, const T* z, const T* p
         c->launches++;
     } else if constexpr (U) {
         const int nblk = (int)std::min<long long>((c->N + 255) / 256, GM_RED_BLOCKS);
-        gm_pcg_dir_kernel<<<nblk, 256, 0, s>>>(c->N, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
+        gm_pcg_dir_kernel<3><<<nblk, 256, 0, s>>>(c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
         c->launches++;
         b.xu = p_new;
         nbulk = gm_fx_launch<CLS, GM_M_K, true>(c, b, 1.0, false, s);
     } else {
-        gm_bulk_apply_kernel<T, CLS, BULK, true><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
-        c->applies++;
-        c->launches++;
+        // the per-element storage of the fixed-stress operator has no fixed-point form
+        const FlowFx Q = fs == nullptr ? gm_flow_fx(c, cS, cC) : FlowFx{};
+        if (fs == nullptr && Q.grade >= 0) {
+            const int nblk = (int)std::min<long long>((c->N + 255) / 256, GM_RED_BLOCKS);
+            gm_pcg_dir_kernel<1><<<nblk, 256, 0, s>>>(c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
+            c->launches++;
+            b.xp = p_new;
+            nbulk = gm_fx_launch<CLS, GM_FX_FLOW, true>(c, b, 1.0, false, s, Q);
+        } else {
+            gm_bulk_apply_kernel<T, CLS, BULK, true><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+            c->applies++;
+            c->launches++;
+        }
     }
     if (c->g.kf >= 0) {
         FaultArgs<T> f = gm_fault_args<T>(c, cK, 0, 0, cS, cC, U);

@@ -1,12 +1,13 @@
 // FP64 bulk products in wide fixed point (gm_fixed.cuh): K_b (u -> u), A_pu
-// (p -> u) and A_up (u -> p) of gm_bulk.cuh, same operator, tiling and march.
+// (p -> u), A_up (u -> p) and S + dt C (p -> p) of gm_bulk.cuh, same operator, tiling and march.
 //
 // Why: the FP64 kernel is bound by the FP64 pipe (2 lanes per clock and SM).
 // In the parity basis a K_b element takes about 210 FP64 instructions, 64
 // issue slots each; the same element takes about 2200 integer instructions here
 // (560 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
-// per product: K_T on 128^3 dipping cells 1254 -> 403; K_T + A_pu + A_up on
-// 61x127x46 cells sheared both ways 683 -> 229; J on 8^3 cells 89 -> 62.
+// per product: K_T on 128^3 dipping cells 1254 -> 403; K_T + A_pu + A_up + A22 on
+// 61x127x46 cells sheared both ways 804 -> 274 (A22 121 -> 46); J on 8^3 cells
+// 89 -> 47.
 //
 // Each CTA first looks over its inputs: the largest exponent sets the tile's
 // unit, and the smallest of the elements' largest exponents says how far the
@@ -29,13 +30,16 @@
 #include "gm_bulk.cuh"
 #include "gm_fixed.cuh"
 
+constexpr int GM_FX_FLOW = GM_M_S | GM_M_C;
 template <int MODE>
 struct FxSmem {
-    static constexpr int NI = MODE == GM_M_APU ? 1 : 3, NO = MODE == GM_M_AUP ? 1 : 3;
+    static constexpr int NI = MODE == GM_M_APU || MODE == GM_FX_FLOW ? 1 : 3;
+    static constexpr int NO = MODE == GM_M_AUP || MODE == GM_FX_FLOW ? 1 : 3;
+    static constexpr int NL = MODE == GM_FX_FLOW ? 4 : 3;   // limbs of a result
     static constexpr bool CARRY = MODE == GM_M_K;      // K_b: the carried tuples live here, not in registers
     int plane[3][NI][3][17 * 17];                      // ring of node planes, limb by limb
-    int face[2][NO][3][256];                           // upper node row of the faces, by plane parity
-    int carry[CARRY ? NO * 12 : 1][CARRY ? 256 : 1];
+    int face[2][NO][NL][256];                          // upper node row of the faces, by plane parity
+    int carry[CARRY ? NO * 4 * NL : 1][CARRY ? 256 : 1];
 };
 template <int MODE>
 constexpr size_t gm_fx_smem()
@@ -75,15 +79,19 @@ __device__ __noinline__ void gm_fx_fp64_tile(const BulkArgs<double>& a, const Re
 
 template <int CLS, int MODE, bool DOT>
 __global__ void __launch_bounds__(256, 2)
-gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_constant__ RefFx F, const __grid_constant__ RefOps<double> R)
+gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_constant__ RefFx F,
+                  const __grid_constant__ RefOps<double> R, const __grid_constant__ FlowFx Q)
 {
     constexpr bool DO_K = MODE == GM_M_K;
     constexpr bool DO_APU = MODE == GM_M_APU;
     constexpr bool DO_AUP = MODE == GM_M_AUP;
-    static_assert(DO_K || DO_APU || DO_AUP, "one block at a time");
-    static_assert(!DOT || DO_K, "the dot product belongs to K_b");
-    constexpr int NI = DO_APU ? 1 : 3;
-    constexpr int NO = DO_AUP ? 1 : 3;
+    constexpr bool DO_Q = MODE == GM_FX_FLOW;
+    static_assert(DO_K || DO_APU || DO_AUP || DO_Q, "one block at a time");
+    static_assert(!DOT || DO_K || DO_Q, "the dot product belongs to K_b and S + dt C");
+    constexpr bool IN_P = DO_APU || DO_Q, OUT_P = DO_AUP || DO_Q;
+    constexpr int NI = IN_P ? 1 : 3;
+    constexpr int NO = OUT_P ? 1 : 3;
+    constexpr int NL = FxSmem<MODE>::NL;
     constexpr int TN = 17, PL = TN * TN;
     constexpr ParPat PP = gm_make_parpat(CLS);
     extern __shared__ __align__(16) unsigned char raw[];
@@ -101,11 +109,11 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
     const int z0 = blockIdx.z * a.zchunk;
     const int z1 = min(z0 + a.zchunk, g.nplanes);
     const int N = (int)g.N, nb = (int)g.nb, rowlen = g.nx + 1;
-    const double* xin = DO_APU ? a.xp : a.xu;
+    const double* xin = IN_P ? a.xp : a.xu;
     auto layer_exists = [&](int kb) -> bool { return kb >= 0 && kb + 1 < g.nplanes && kb != g.kf; };
     auto layer_index = [&](int kb) -> int { return (g.kf >= 0 && kb > g.kf) ? kb - 1 : kb; };
     // node whose value plane kk's node takes: a tied upper lip reads the pressure of the lower lip
-    auto src_plane = [&](int kk) -> int { return (DO_APU && g.tied && kk == g.kf + 1) ? kk - 1 : kk; };
+    auto src_plane = [&](int kk) -> int { return (IN_P && g.tied && kk == g.kf + 1) ? kk - 1 : kk; };
 
     // ---- the tile's unit and grading -------------------------------------
     const int kbeg = layer_exists(z0 - 1) ? z0 - 1 : z0;
@@ -124,7 +132,7 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
 #pragma unroll
                     for (int f = 0; f < NI; ++f) {
                         const int hi = __ldg(reinterpret_cast<const int*>(xin + (long long)f * N + node) + 1) & 0x7fffffff;
-                        if (!((m >> (DO_APU ? 3 : f)) & 1u)) m4 = max(m4, hi);
+                        if (!((m >> (IN_P ? 3 : f)) & 1u)) m4 = max(m4, hi);
                     }
                 }
                 if (layer_exists(kk - 1) && kk > kbeg) {
@@ -145,9 +153,9 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
     mx >>= 20;
     mn = min(mn >> 20, mx);
     const int top = mx == 0 ? 1023 : mx;
-    const int qe = (top - 1022 - GM_FX_IN) + (DO_K ? F.eK + F.topE - 1022 : F.eA);
+    const int qe = (top - 1022 - GM_FX_IN) + (DO_K ? F.eK + F.topE - 1022 : DO_Q ? Q.eU : F.eA);
     const bool fixed_ok = top < 0x7ff && top >= 100 && qe >= -1000 && qe <= 900 &&
-                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : F.gradeA));
+                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : DO_Q ? Q.grade : F.gradeA));
     if (!fixed_ok) {
         // uniform over the CTA
         gm_fx_fp64_tile<CLS, MODE>(a, R, raw);
@@ -159,9 +167,11 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
                 for (int kk = z0; kk < z1; ++kk) {
                     if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) continue;
                     const int node = kk * nb + gj * rowlen + gi;
+                    if constexpr (DO_Q) dot = fma(a.xp[node], a.yp[node], dot);
+                    else
 #pragma unroll
-                    for (int f = 0; f < 3; ++f)
-                        dot = fma(a.xu[(long long)f * N + node], a.yu[(long long)f * N + node], dot);
+                        for (int f = 0; f < 3; ++f)
+                            dot = fma(a.xu[(long long)f * N + node], a.yu[(long long)f * N + node], dot);
                 }
             gm_cta_dot(dot, s_dot, a.part);
         }
@@ -192,7 +202,7 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
             const unsigned m = a.mask[node];
 #pragma unroll
             for (int f = 0; f < NI; ++f)
-                if (!((m >> (DO_APU ? 3 : f)) & 1u)) pf[sl][f] = xin[(long long)f * N + node];
+                if (!((m >> (IN_P ? 3 : f)) & 1u)) pf[sl][f] = xin[(long long)f * N + node];
         }
     };
     auto store = [&](int buf) {
@@ -224,19 +234,19 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
 
     // top contributions of the layer below, per output field and tuple
     constexpr bool SC = FxSmem<MODE>::CARRY;
-    int rcarry[SC ? 1 : NO][4][3];
+    int rcarry[SC ? 1 : NO][4][NL];
 #pragma unroll
     for (int f = 0; f < NO; ++f)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                if constexpr (SC) S.carry[(f * 4 + q) * 3 + i][tid] = 0;
+            for (int i = 0; i < NL; ++i) {
+                if constexpr (SC) S.carry[(f * 4 + q) * NL + i][tid] = 0;
                 else rcarry[f][q][i] = 0;
             }
 
     // Output mode `s` of field c from the element's input modes xv.
-    auto out_mode = [&](const int (&xv)[NI * 8][3], int c, int s, const int (&E)[3], int (&y)[3]) {
+    auto out_mode = [&](const int (&xv)[NI * 8][3], int c, int s, const int (&E)[3], int (&y)[NL]) {
         FxAcc acc{0, 0, 0};
         if constexpr (DO_K) {
             gm_fx_k_mode<CLS>(F, xv, c, s, E, y);
@@ -248,6 +258,25 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
                     gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
                 }
             gm_fx_carry(acc, y);
+        } else if constexpr (DO_Q) {
+            // E holds the limbs of the element's dt k/mu; mode 0 has no flow.  The
+            // results keep a fourth limb: elements of low permeability lie far
+            // below the unit that the most permeable one sets
+            FxAcc4 sum{0, 0, 0, 0};
+            if (s != 0 && a.cC != 0.0) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (PP.l[s][j] >= 0) {
+                        const int* k = Q.l[PP.l[s][j]];
+                        gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+                    }
+                int r[3];
+                gm_fx_carry(acc, r);
+                gm_fx_mac4(sum, r, E[2], E[1], E[0]);
+            }
+            const int* m = Q.m[s];
+            gm_fx_mac4(sum, xv[s], m[2], m[1], m[0]);
+            gm_fx_carry4_signed(sum, y);
         } else {
 #pragma unroll
             for (int j = 0; j < 24; ++j)
@@ -262,13 +291,14 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
     // Layer kb between planes kb and kb + 1 of the ring.  With `plane`, field by
     // field: complete the face tuples of plane kb, transform them back and
     // exchange; in any case the layer's top contributions become the carry.
-    int low[NO][3];
+    int low[NO][NL];
     auto layer = [&](int kb, bool exists, bool plane) {
         const bool work = exists && fval;
         int xv[NI * 8][3];
         int E[3] = {0, 0, 0};
         if (work) {
             double Ed = 0.0;
+            if constexpr (DO_Q) Ed = a.cC * a.kap[fi + (long long)g.nx * (fj + (long long)g.ny * layer_index(kb))];
             if constexpr (DO_K) Ed = a.E[fi + (long long)g.nx * (fj + (long long)g.ny * layer_index(kb))];
             const int sb = (kb - kbeg) % 3, st = (kb + 1 - kbeg) % 3;
 #pragma unroll
@@ -285,21 +315,22 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
                     }
             }
             if constexpr (DO_K) gm_fx_coef(Ed, F.topE, E);
+            if constexpr (DO_Q) gm_fx_coef(Ed, Q.topW, E);
         }
 #pragma unroll
         for (int c = 0; c < NO; ++c) {
-            int o[4][3];
+            int o[4][NL];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+                int lo[NL] = {}, hi[NL] = {};
                 if (work) {
-                    if (DO_AUP || q != 0) out_mode(xv, c, q, E, lo);   // mode 0 of u carries no force
+                    if (OUT_P || q != 0) out_mode(xv, c, q, E, lo);   // mode 0 of u carries no force
                     out_mode(xv, c, q + 4, E, hi);
                 }
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
+                for (int i = 0; i < NL; ++i) {
                     if constexpr (SC) {
-                        int& cy = S.carry[(c * 4 + q) * 3 + i][tid];
+                        int& cy = S.carry[(c * 4 + q) * NL + i][tid];
                         o[q][i] = cy + lo[i] + hi[i];
                         cy = lo[i] - hi[i];
                     } else {
@@ -310,7 +341,7 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
             }
             if (plane) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
+                for (int i = 0; i < NL; ++i) {
                     const int c0 = o[0][i] + o[1][i], c1 = o[0][i] - o[1][i];
                     const int d0 = o[2][i] + o[3][i], d1 = o[2][i] - o[3][i];
                     const int p10 = __shfl_up_sync(0xffffffffu, c1 + d1, 1, 16);
@@ -331,21 +362,25 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
         const unsigned m = a.mask[node];
         const bool lip = g.kf >= 0 && (kk == g.kf || kk == g.kf + 1);
         // raw value on a tied slave lip: the fault kernel folds it
-        const bool slave = DO_AUP && g.tied && kk == g.kf + 1;
+        const bool slave = OUT_P && g.tied && kk == g.kf + 1;
 #pragma unroll
         for (int f = 0; f < NO; ++f) {
-            const int(&up)[3][256] = S.face[kk & 1][f];
-            const double v = scale * gm_fx_to_double(low[f][0] + up[0][tid - 16], low[f][1] + up[1][tid - 16],
-                                                     low[f][2] + up[2][tid - 16]);
-            double* y = DO_AUP ? a.yp + node : a.yu + (long long)f * N + node;
-            const bool fixed = !slave && ((m >> (DO_AUP ? 3 : f)) & 1u);
+            const int(&up)[NL][256] = S.face[kk & 1][f];
+            int l[NL];
+#pragma unroll
+            for (int i = 0; i < NL; ++i) l[i] = low[f][i] + up[i][tid - 16];
+            double v;
+            if constexpr (DO_Q) v = scale * gm_fx_to_double4(l[0], l[1], l[2], l[3]);
+            else v = scale * gm_fx_to_double(l[0], l[1], l[2]);
+            double* y = OUT_P ? a.yp + node : a.yu + (long long)f * N + node;
+            const bool fixed = !slave && ((m >> (OUT_P ? 3 : f)) & 1u);
             if (a.accumulate) {
                 if (!fixed) *y += v;
             } else {
                 *y = fixed ? 0.0 : v;
             }
             if constexpr (DOT)
-                if (!lip && !fixed) dot = fma(a.xu[(long long)f * N + node], v, dot);
+                if (!lip && !fixed) dot = fma(DO_Q ? a.xp[node] : a.xu[(long long)f * N + node], v, dot);
         }
     };
 

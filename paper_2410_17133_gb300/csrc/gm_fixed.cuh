@@ -111,6 +111,34 @@ __host__ __device__ inline void gm_fx_carry_signed(const FxAcc& s, int (&l)[3])
     l[2] = (int)(t1 >> GM_FX_RADIX);
 }
 
+// Product sums with one limb more below (weight 2^-26), for results whose terms
+// carry coefficients far apart: l[0] is that limb, l[1..3] those above.
+struct FxAcc4 {
+    int64_t a2, a1, a0, am;
+};
+__host__ __device__ inline void gm_fx_mac4(FxAcc4& s, const int (&x)[3], int c2, int c1, int c0)
+{
+    s.a2 += (int64_t)x[2] * c2;
+    s.a1 += (int64_t)x[1] * c2;
+    s.a1 += (int64_t)x[2] * c1;
+    s.a0 += (int64_t)x[0] * c2;
+    s.a0 += (int64_t)x[1] * c1;
+    s.a0 += (int64_t)x[2] * c0;
+    s.am += (int64_t)x[0] * c1;
+    s.am += (int64_t)x[1] * c0;
+}
+__host__ __device__ inline void gm_fx_carry4_signed(const FxAcc4& s, int (&l)[4])
+{
+    constexpr int H = 1 << (GM_FX_RADIX - 1);
+    const int64_t tm = s.a0 + (s.am >> GM_FX_RADIX) + H;
+    l[0] = ((int)tm & GM_FX_MASK) - H;
+    const int64_t t0 = s.a1 + (tm >> GM_FX_RADIX) + H;
+    l[1] = ((int)t0 & GM_FX_MASK) - H;
+    const int64_t t1 = s.a2 + (t0 >> GM_FX_RADIX) + H;
+    l[2] = ((int)t1 & GM_FX_MASK) - H;
+    l[3] = (int)(t1 >> GM_FX_RADIX);
+}
+
 // nearest double of l2 2^52 + l1 2^26 + l0 (one rounding): the bits below 2^52
 // and the rest are exact doubles, joined by one fused multiply-add
 __host__ __device__ inline double gm_fx_to_double(int l0, int l1, int l2)
@@ -120,4 +148,18 @@ __host__ __device__ inline double gm_fx_to_double(int l0, int l1, int l2)
     const double lo = gm_fx_real((t & 0xfffffffffffffll) | 0x4330000000000000ll) - 4503599627370496.0;
     const double dh = gm_fx_real((int64_t)(0x4330000000000000ull | (uint32_t)(hi ^ 0x80000000))) - 4503601774854144.0;
     return fma(dh, 4503599627370496.0, lo);
+}
+
+// double of l3 2^52 + l2 2^26 + l1 + l0 2^-26, within one unit of its last place:
+// the middle part is kept in [-2^51, 2^51), so that values of either sign below
+// one unit keep their lowest limb
+__host__ __device__ inline double gm_fx_to_double4(int l0, int l1, int l2, int l3)
+{
+    const int64_t t = (int64_t)l2 * (1 << GM_FX_RADIX) + l1;
+    const int64_t up = (t + (1ll << 51)) >> 52;
+    const int hi = l3 + (int)up;
+    const double mid = gm_fx_real((int64_t)(0x4338000000000000ull + (uint64_t)(t - up * (1ll << 52)))) - 6755399441055744.0;
+    const double dl = gm_fx_real((int64_t)(0x4330000000000000ull | (uint32_t)(l0 ^ 0x80000000))) - 4503601774854144.0;
+    const double dh = gm_fx_real((int64_t)(0x4330000000000000ull | (uint32_t)(hi ^ 0x80000000))) - 4503601774854144.0;
+    return fma(dh, 4503599627370496.0, fma(dl, 1.4901161193847656e-08, mid));
 }

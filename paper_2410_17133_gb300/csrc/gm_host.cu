@@ -180,7 +180,7 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
 // does not belong to the class, or the pattern rule does not hold).
 template <int CLS>
 bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8],
-              const double L[8][8], RefOps<double>& R, RefFx& F, double alpha, double Emin, double Emax)
+              const double L[8][8], RefOps<double>& R, RefFx& F, double alpha, double Emin, double Emax, double& Lsum)
 {
     constexpr ParPat PP = gm_make_parpat(CLS);
     static double Kt[24][24], At[24][8], Mt[8][8], Lt[8][8];   // index (c*8+s)
@@ -241,6 +241,13 @@ bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8
             else if (std::fabs(Lt[i][j]) > tol * lmax) return false;
         }
     make_fx(Kt, At, PP, alpha, Emin, Emax, F);
+    Lsum = 0.0;
+    for (int i = 0; i < 8; ++i) {
+        double t = 0.0;
+        for (int j = 0; j < 8; ++j)
+            if (PP.l[i][j] >= 0) t += std::fabs(Lt[i][j]);
+        Lsum = std::max(Lsum, t);
+    }
     return true;
 }
 
@@ -257,6 +264,58 @@ int bind_impl(gm_ctx* c);
 
 }  // namespace
 
+// range of k/mu for the fixed-point scale of the flow block
+static void note_kap_range(gm_ctx* c, const std::vector<double>& kap)
+{
+    double lo = 0.0, hi = 0.0;
+    c->kap_zero = false;
+    for (double k : kap) {
+        hi = std::max(hi, k);
+        if (!(k > 0.0)) c->kap_zero = true;
+        if (k > 0.0 && (lo == 0.0 || k < lo)) lo = k;
+    }
+    // captured A22 iterations hold the scale that follows from the range
+    if (lo != c->kap_lo || hi != c->kap_hi) c->drop_graphs();
+    c->kap_lo = lo;
+    c->kap_hi = hi;
+}
+
+// Flow block S cS / M + cC C in fixed point (cS as given to the launchers).
+FlowFx gm_flow_fx(const gm_ctx* c, double cS, double cC)
+{
+    FlowFx Q;
+    std::memset(&Q, 0, sizeof(Q));
+    double ms = 0.0;
+    for (double m : c->R64.M) ms = std::max(ms, std::fabs(m));
+    const double storage = std::fabs(cS) / c->M * ms;
+    // the smallest coefficient an element can have (one without flow: its storage)
+    const double hi = std::max(storage, cC * c->kap_hi * c->Lsum), flow = cC * c->kap_lo * c->Lsum;
+    const double lo = storage > 0.0 ? (c->kap_zero ? storage : std::max(storage, flow)) : flow;
+    if (!(cC >= 0.0) || !std::isfinite(hi) || !(hi < 1e250) || (hi > 0.0 && !(hi > 1e-250))) {
+        Q.grade = -1;
+        return Q;
+    }
+    if (!(hi > 0.0)) {                 // the block is zero
+        Q.topW = 1022;
+        Q.grade = GM_FX_GRADE;
+        return Q;
+    }
+    const int eL = c->Lsum > 0.0 ? std::ilogb(c->Lsum) + 1 : 0;
+    Q.eU = std::ilogb(hi) + 1 + 2;
+    // dt k/mu 2^eL / 2^eU; a factor of two for its row sum below 2^eL
+    Q.eU = std::max(Q.eU, (c->kap_hi > 0.0 && cC > 0.0 ? std::ilogb(cC * c->kap_hi) + 1 : -2000) + eL + 2);
+    Q.topW = 1022 + Q.eU - eL;
+    for (int i = 0; i < GM_PP_MAXL; ++i) fx_limbs(c->R64.L[i], 0.0, eL, Q.l[i]);
+    for (int i = 0; i < 8; ++i) {
+        const double f = cS / c->M, v = f * c->R64.M[i];
+        fx_limbs(v, std::fma(f, c->R64.M[i], -v), Q.eU, Q.m[i]);
+    }
+    // the fourth limb of the results covers coefficients 2^24 apart; the inputs'
+    // own grading is judged by the kernel as for the other blocks
+    Q.grade = std::ilogb(hi) - std::ilogb(lo) <= 24 ? GM_FX_GRADE - 2 : -1;
+    return Q;
+}
+
 // per-element k/mu arrays (FP64, FP32) and the diagonals that depend on them
 int gm_upload_permeability(gm_ctx* c)
 {
@@ -267,6 +326,7 @@ int gm_upload_permeability(gm_ctx* c)
         kap[e] = c->kperm[e] / c->mu_f;
         f32[e] = (float)kap[e];
     }
+    note_kap_range(c, kap);
     GM_CUDA_TRY(c, cudaMemcpy(c->dK64.p, kap.data(), nel * 8, cudaMemcpyHostToDevice));
     GM_CUDA_TRY(c, cudaMemcpy(c->dK32.p, f32.data(), nel * 4, cudaMemcpyHostToDevice));
     int rc = gm_launch_diag(c, 0);
@@ -878,9 +938,9 @@ int bind_impl(gm_ctx* c)
     if (!ref_cell(c->h, c->shear, c->nu, K, A, M, L)) return c->set_err(GM_EINVAL, "bind: degenerate cell");
     const auto Er = std::minmax_element(c->E.begin(), c->E.end());
     const double E0 = *Er.first, E1 = *Er.second;
-    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1)
-            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1)
-                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1);
+    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum)
+            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum)
+                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum);
     if (!ok) return c->set_err(GM_EINVAL, "bind: cell operators break the expected parity pattern");
     cast_ref(c->R64, c->R32);
     for (int i = 0; i < GM_PP_MAXK; ++i) c->R32p.K[i] = make_float2(c->R32.K[i], c->R32.K[i]);
@@ -1007,6 +1067,7 @@ int bind_impl(gm_ctx* c)
     {
         std::vector<double> kap(nel);
         for (long long e = 0; e < nel; ++e) kap[e] = c->kperm[e] / c->mu_f;
+        note_kap_range(c, kap);
         GM_CUDA_TRY(c, cudaMemcpy(c->dK64.p, kap.data(), nel * 8, cudaMemcpyHostToDevice));
         for (long long e = 0; e < nel; ++e) f32[e] = (float)kap[e];
         GM_CUDA_TRY(c, cudaMemcpy(c->dK32.p, f32.data(), nel * 4, cudaMemcpyHostToDevice));

@@ -172,6 +172,17 @@ struct RefFx {
     int eK, eA, topE, gradeK, gradeA;
 };
 
+// The flow block of one launch in the same form: Darcy entries (row sums at most
+// 1), storage per mode, and the scale 2^eU that bounds both (a quarter each, so
+// that 36 results of their sum meet in a node); topW is the biased exponent of
+// the largest dt k/mu that the scale admits.  grade < 0: coefficients too far
+// apart for the fixed-point unit, use FP64.
+struct FlowFx {
+    int l[GM_PP_MAXL][3];
+    int m[8][3];
+    int topW, eU, grade;
+};
+
 // Per-node mask bits: 1,2,4 = ux,uy,uz fixed, 8 = p fixed.
 // Tied upper-lip pressures are slaves (handled by index, not by this mask).
 
@@ -419,6 +430,9 @@ struct gm_ctx {
     RefOps<float> R32{};
     RefPairs32 R32p{};
     RefFx Rfx{};
+    double Lsum = 0.0;            // largest absolute row sum of the Darcy operator in the parity basis (k/mu = 1)
+    double kap_lo = 0.0, kap_hi = 0.0;   // smallest positive and largest k/mu of an element (0: none)
+    bool kap_zero = false;        // some element has k = 0
     double Kblk_ref[8][9] = {};   // nodal 3x3 diagonal blocks of K_ref (E = 1)
     double Mdiag_ref[8] = {}, Ldiag_ref[8] = {};
     double Aq = 0, nrm[3] = {0, 0, 1}, t1[3] = {1, 0, 0}, t2[3] = {0, 1, 0};
@@ -531,6 +545,7 @@ int gm_launch_block_jacobi(gm_ctx* c, cudaStream_t s);    // K_T 3x3 inverse blo
 // multigrid preconditioner of the FP32 K_T solves (gm_mg.cu)
 int gm_prepare_bulk32(gm_ctx* c);                     // kernel attributes, at bind
 int gm_prepare_fx(gm_ctx* c);
+FlowFx gm_flow_fx(const gm_ctx* c, double cS, double cC);   // gm_host.cu
 int gm_launch_bulk_k_f32(gm_ctx* c, const float* x, float* y, cudaStream_t s, const int* skip);
 int gm_launch_bulk_k_f64(gm_ctx* c, const double* x, double* y, cudaStream_t s, const int* skip);
 int gm_mg_prepare(gm_ctx* c, int prec, cudaStream_t s);   // GM_EINVAL: grid not coarsenable (caller falls back)

@@ -93,6 +93,61 @@ def test_products_within_fp64_rounding_row_by_row(name, kind):
         assert np.all(y[~out] == 0.0)
 
 
+CONTRAST = {"even": lambda r, n: np.full(n, 1e-15), "lognormal": lambda r, n: 10.0 ** r.normal(-15.0, 0.5, n),
+            "layers": lambda r, n: r.choice([0.0, 1e-19, 1e-12], n), "extreme": lambda r, n: 10.0 ** r.uniform(-40, 0, n),
+            "none": lambda r, n: np.zeros(n)}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dt", [2.0, 1e-9, 1e9])
+@pytest.mark.parametrize("kind", ["noise", "decay", "steep", "spike", "zero", "antisymmetric"])
+@pytest.mark.parametrize("contrast", list(CONTRAST))
+def test_flow_products_within_fp64_rounding_row_by_row(contrast, kind, dt):
+    from gpu_common import cuda, need_gpu, solver_for
+    need_gpu()
+    prob = problem("dip_ragged")
+    prob.k = CONTRAST[contrast](np.random.default_rng(9), prob.n_el)
+    model = fem.Model(prob)
+    s = solver_for(prob)
+    s.timestep(dt)
+    free = prob.fixed[3] == 0
+    p = field(kind, prob, 5)[3] * free
+    # element by element: what its own coefficients make of its largest input
+    from oracle.fem import element_matrices
+    X = model.mesh.coords()[model.conn]
+    cond = np.asarray(prob.k) / prob.mu_f
+    _, _, S, C = element_matrices(X, prob.E, prob.nu, prob.alpha, 1.0 / prob.M, cond)
+    big = np.abs(p)[model.conn].max(1)
+    rows = (np.abs(S) + dt * np.abs(C)).sum(2) * big[:, None]
+    scale = np.zeros(prob.n_nodes)
+    np.add.at(scale, model.conn.ravel(), rows.ravel())
+    ref = model.S @ p + dt * (model.C @ p)
+    y = s.apply("A22", cuda(p)).cpu().numpy()
+    assert np.all(np.abs(y - ref)[free] <= (34 + 34) * EPS * scale[free])
+    assert np.all(y[~free] == 0.0)
+
+
+@pytest.mark.gpu
+def test_flow_solves_follow_a_new_permeability():
+    from gpu_common import cuda, need_gpu, solver_for
+    need_gpu()
+    prob = problem("box_16")
+    rng = np.random.default_rng(4)
+    b = cuda(rng.normal(size=prob.n_nodes) * 1e-12 * (prob.fixed[3] == 0))
+    s = solver_for(prob)
+    s.timestep(3.0)
+    for scale in (1.0, 1e5, 1e-6):
+        k = prob.k * scale
+        s.set_permeability(k)
+        x, _ = s.pcg("A22", b, rtol=1e-12)
+        fresh = problem("box_16")
+        fresh.k = k
+        f = solver_for(fresh)
+        f.timestep(3.0)
+        y, _ = f.pcg("A22", b, rtol=1e-12)
+        assert bool((x == y).all())
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
 def test_values_that_are_not_finite_reach_their_rows(bad):
@@ -124,6 +179,15 @@ extern "C" {
 void from_double(double x, int top, int* l) { int v[3]; gm_fx_from_double(x, top, v); for (int i = 0; i < 3; ++i) l[i] = v[i]; }
 void coef(double x, int top, int* l) { int v[3]; gm_fx_coef(x, top, v); for (int i = 0; i < 3; ++i) l[i] = v[i]; }
 double to_double(int a, int b, int c) { return gm_fx_to_double(a, b, c); }
+double to_double4(int a, int b, int c, int d) { return gm_fx_to_double4(a, b, c, d); }
+void product4(const int* x, const int* k, int n, int* l)
+{
+    FxAcc4 s{0, 0, 0, 0};
+    for (int i = 0; i < n; ++i) { int v[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]}; gm_fx_mac4(s, v, k[3 * i + 2], k[3 * i + 1], k[3 * i]); }
+    int r[4];
+    gm_fx_carry4_signed(s, r);
+    for (int i = 0; i < 4; ++i) l[i] = r[i];
+}
 void product(const int* x, const int* k, int n, int sgn, int* l)
 {
     FxAcc s{0, 0, 0};
@@ -146,7 +210,7 @@ def host(tmp_path_factory):
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-ffp-contract=off", "-I",
                     os.path.join(ROOT, "paper_2410_17133_gb300", "csrc"), "-o", so, str(d / "h.cpp")], check=True)
     lib = ctypes.CDLL(so)
-    lib.to_double.restype = ctypes.c_double
+    lib.to_double.restype = lib.to_double4.restype = ctypes.c_double
     lib.from_double.argtypes = lib.coef.argtypes = [ctypes.c_double, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     return lib
 
@@ -170,6 +234,30 @@ def test_limbs_and_back(host):
         a, b = (int(v) for v in rng.integers(-2 ** 31 + 1, 2 ** 31, 2) >> rng.integers(0, 31, 2))
         c = int(rng.integers(-2 ** 30, 2 ** 30)) >> int(rng.integers(0, 31))
         assert host.to_double(a, b, c) == float((c << 52) + (b << 26) + a)   # int -> float rounds to nearest even
+
+
+def test_four_limbs_and_back(host):
+    from fractions import Fraction
+    rng = np.random.default_rng(7)
+    for t in range(2000):
+        a, b, c = (int(v) for v in rng.integers(-2 ** 30, 2 ** 30, 3) >> rng.integers(0, 31, 3))
+        d = int(rng.integers(-2 ** 29, 2 ** 29)) >> int(rng.integers(0, 30))
+        if t % 3 == 0:
+            d = 0 if t % 2 else -1                     # cancelling parts of either sign
+        v = Fraction((d << 52) + (c << 26) + b) + Fraction(a, 2 ** 26)
+        y = host.to_double4(a, b, c, d)
+        assert abs(Fraction(y) - v) <= abs(v) * Fraction(1, 2 ** 52)
+    out = (ctypes.c_int * 4)()
+    P = ctypes.POINTER(ctypes.c_int)
+    for _ in range(300):
+        n = int(rng.integers(1, 4))
+        x = np.ascontiguousarray(rng.integers(-2 ** 29, 2 ** 29, (n, 3)) // [1, 1, 8], dtype=np.int32)
+        k = np.ascontiguousarray(rng.integers(-2 ** 24, 2 ** 24, (n, 3)), dtype=np.int32)
+        host.product4(x.ctypes.data_as(P), k.ctypes.data_as(P), n, out)
+        exact = sum(value(x[i]) * value(k[i]) for i in range(n))
+        got = (value(out[1:]) << 26) + int(out[0])     # units of 2^-26
+        assert abs(got * 2 ** 52 - exact) <= (2 + 4 * n) * 2 ** 52
+        assert all(-2 ** 25 <= out[i] < 2 ** 25 for i in range(3))
 
 
 @pytest.mark.parametrize("signed", [0, 1])
