@@ -37,20 +37,15 @@ __device__ inline void gm_pcg_alpha_from(PcgScalars* sc, double pq)
     }
 }
 
-// Sum n partials in a fixed order with one block (thread-strided, then a tree).
+// Sum n partials in a fixed order with one block of 256 threads (thread-strided,
+// then a tree); the result is on thread 0.
 __device__ inline double gm_block_sum_fixed(const double* part, int n)
 {
-    __shared__ double sh[32];
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) acc += ((volatile const double*)part)[b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    double tot = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += sh[w];
-    return tot;
+    __shared__ double sh[16];
+    double acc[1] = {0.0};
+    for (int b = threadIdx.x; b < n; b += blockDim.x) acc[0] += ((volatile const double*)part)[b];
+    gm_block_sum256<1>(acc, sh);
+    return acc[0];
 }
 
 template <typename T, int MODE, bool PCG>
@@ -132,12 +127,12 @@ gm_fault_apply_kernel(const FaultArgs<T> a)
                 if (!((mp >> c) & 1u)) {
                     const T y = a.yu[c * N + np] + f[c];
                     a.yu[c * N + np] = y;
-                    if constexpr (PCG) dot += (double)a.xu[c * N + np] * (double)y;
+                    if constexpr (PCG) dot = fma(gm_widen(a.xu[c * N + np]), gm_widen(y), dot);
                 }
                 if (!((mm >> c) & 1u)) {
                     const T y = a.yu[c * N + nm] - f[c];
                     a.yu[c * N + nm] = y;
-                    if constexpr (PCG) dot += (double)a.xu[c * N + nm] * (double)y;
+                    if constexpr (PCG) dot = fma(gm_widen(a.xu[c * N + nm]), gm_widen(y), dot);
                 }
             }
         }
@@ -169,35 +164,30 @@ gm_fault_apply_kernel(const FaultArgs<T> a)
                 const T y = ((mm >> 3) & 1u) ? T(0) : v;
                 a.yp[nm] = y;
                 a.yp[np] = T(0);
-                if constexpr (PCG) dot += (double)pval(nm) * (double)y;
+                if constexpr (PCG) dot = fma(gm_widen(pval(nm)), gm_widen(y), dot);
             } else {
                 const T vp = T(0.5) * dav + dtr, vm = T(0.5) * dav - dtr;
                 if (!((mp >> 3) & 1u)) {
                     const T y = a.yp[np] + vp;
                     a.yp[np] = y;
-                    if constexpr (PCG) dot += (double)a.xp[np] * (double)y;
+                    if constexpr (PCG) dot = fma(gm_widen(a.xp[np]), gm_widen(y), dot);
                 }
                 if (!((mm >> 3) & 1u)) {
                     const T y = a.yp[nm] + vm;
                     a.yp[nm] = y;
-                    if constexpr (PCG) dot += (double)a.xp[nm] * (double)y;
+                    if constexpr (PCG) dot = fma(gm_widen(a.xp[nm]), gm_widen(y), dot);
                 }
             }
         }
     }
 
     if constexpr (PCG) {
-        __shared__ double sh[8];
+        __shared__ double sh[16];
         __shared__ bool last;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, o);
-        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dot;
-        __syncthreads();
+        double sum[1] = {dot};
+        gm_block_sum256<1>(sum, sh);
         if (threadIdx.x == 0) {
-            double s = 0.0;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) s += sh[w];
-            a.part[a.nbulk + blockIdx.x] = s;
+            a.part[a.nbulk + blockIdx.x] = sum[0];
             __threadfence();
             last = (atomicAdd(a.counter, 1u) == gridDim.x - 1);
         }

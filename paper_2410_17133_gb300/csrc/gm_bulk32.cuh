@@ -366,7 +366,7 @@ gm_bulk32_kernel(const BulkArgs<float> a, const __grid_constant__ gm32::Ref32 R)
                 if constexpr (PCG) {
                     const float p = slave ? 0.f : pown[f].x;
                     pnew[f * N + node0] = p;
-                    if (!lip) dot += (double)p * (double)y;
+                    if (!lip) dot = fma(gm_widen(p), gm_widen(y), dot);
                 }
             }
             if (ok1) {
@@ -376,7 +376,7 @@ gm_bulk32_kernel(const BulkArgs<float> a, const __grid_constant__ gm32::Ref32 R)
                 if constexpr (PCG) {
                     const float p = slave ? 0.f : pown[f].y;
                     pnew[f * N + node0 + rowlen] = p;
-                    if (!lip) dot += (double)p * (double)y;
+                    if (!lip) dot = fma(gm_widen(p), gm_widen(y), dot);
                 }
             }
         }

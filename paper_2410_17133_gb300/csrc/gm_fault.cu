@@ -4,37 +4,14 @@
 // ---------------------------------------------------------------------------
 // Deterministic block reductions (fixed grid, last block sums the partials)
 // ---------------------------------------------------------------------------
-template <int NV>
-__device__ void gm_block_sum(double (&v)[NV], double* sh /* NV * 32 */)
-{
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) sh[k * 32 + w] = v[k];
-    __syncthreads();
-    if (w == 0) {
-        const int nw = blockDim.x >> 5;
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            v[k] = lane < nw ? sh[k * 32 + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        }
-    }
-}
-
 // Writes this block's partials; returns true in the (single) last block, whose
 // thread 0 then holds the grand totals in v (summed in block order).
 template <int NV>
 __device__ bool gm_grid_sum(double (&v)[NV], double* part, unsigned* counter)
 {
-    __shared__ double sh[NV * 32];
+    __shared__ double sh[16];
     __shared__ bool last;
-    gm_block_sum<NV>(v, sh);
+    gm_block_sum256<NV>(v, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) part[k * gridDim.x + blockIdx.x] = v[k];
@@ -52,8 +29,7 @@ __device__ bool gm_grid_sum(double (&v)[NV], double* part, unsigned* counter)
         for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
             acc[k] += ((volatile double*)part)[k * gridDim.x + b];
     }
-    __syncthreads();
-    gm_block_sum<NV>(acc, sh);
+    gm_block_sum256<NV>(acc, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) v[k] = acc[k];
@@ -249,7 +225,7 @@ int gm_launch_residual(gm_ctx* c, const double* y1u, const double* y1p, const do
     a.part = c->dpart.as<double>();
     a.counter = c->dcount.as<unsigned>();
     a.out = out2;
-    gm_residual_kernel<<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(a);
+    gm_residual_kernel<<<gm_red_blocks(c->N), GM_RED_THREADS, 0, s>>>(a);
     GM_LAUNCHED(c);
     return GM_OK;
 }

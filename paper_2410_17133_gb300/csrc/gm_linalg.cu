@@ -12,34 +12,11 @@
 #include "gm_pcgvec.cuh"
 
 template <int NV>
-__device__ void gm_block_sum_l(double (&v)[NV], double* sh)
-{
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) sh[k * 32 + w] = v[k];
-    __syncthreads();
-    if (w == 0) {
-        const int nw = blockDim.x >> 5;
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            v[k] = lane < nw ? sh[k * 32 + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        }
-    }
-}
-
-template <int NV>
 __device__ bool gm_grid_sum_l(double (&v)[NV], double* part, unsigned* counter)
 {
-    __shared__ double sh[NV * 32];
+    __shared__ double sh[16];
     __shared__ bool last;
-    gm_block_sum_l<NV>(v, sh);
+    gm_block_sum256<NV>(v, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) part[k * gridDim.x + blockIdx.x] = v[k];
@@ -57,8 +34,7 @@ __device__ bool gm_grid_sum_l(double (&v)[NV], double* part, unsigned* counter)
         for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
             acc[k] += ((volatile double*)part)[k * gridDim.x + b];
     }
-    __syncthreads();
-    gm_block_sum_l<NV>(acc, sh);
+    gm_block_sum256<NV>(acc, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) v[k] = acc[k];
@@ -233,20 +209,20 @@ int gm_launch_pcg_init(gm_ctx* c, int which, int prec, const void* b, const void
     RedCtx rc = redctx(c);
     if (prec == GM_F64) {
         if (which == 0)
-            gm_pcg_init_kernel<double, 0><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_init_kernel<double, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (const double*)b, (const double*)q, (double*)r, (double*)z, (double*)p,
                 prec_ptr<double>(c, 0), rtol, sc, rc, pairprec<double>(c, 0));
         else
-            gm_pcg_init_kernel<double, 1><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_init_kernel<double, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (const double*)b, (const double*)q, (double*)r, (double*)z, (double*)p,
                 prec_ptr<double>(c, which), rtol, sc, rc, pairprec<double>(c, which));
     } else {
         if (which == 0)
-            gm_pcg_init_kernel<float, 0><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_init_kernel<float, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (const float*)b, (const float*)q, (float*)r, (float*)z, (float*)p,
                 prec_ptr<float>(c, 0), rtol, sc, rc, pairprec<float>(c, 0));
         else
-            gm_pcg_init_kernel<float, 1><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_init_kernel<float, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (const float*)b, (const float*)q, (float*)r, (float*)z, (float*)p,
                 prec_ptr<float>(c, which), rtol, sc, rc, pairprec<float>(c, which));
     }
@@ -261,20 +237,20 @@ int gm_launch_pcg_update(gm_ctx* c, int which, int prec, void* x, void* r, void*
     RedCtx rc = redctx(c);
     if (prec == GM_F64) {
         if (which == 0)
-            gm_pcg_update_kernel<double, 0><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_update_kernel<double, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (double*)x, (double*)r, (double*)z, (const double*)p, (const double*)q,
                 prec_ptr<double>(c, 0), sc, maxit, rc, pairprec<double>(c, 0));
         else
-            gm_pcg_update_kernel<double, 1><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_update_kernel<double, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (double*)x, (double*)r, (double*)z, (const double*)p, (const double*)q,
                 prec_ptr<double>(c, which), sc, maxit, rc, pairprec<double>(c, which));
     } else {
         if (which == 0)
-            gm_pcg_update_kernel<float, 0><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_update_kernel<float, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (float*)x, (float*)r, (float*)z, (const float*)p, (const float*)q,
                 prec_ptr<float>(c, 0), sc, maxit, rc, pairprec<float>(c, 0));
         else
-            gm_pcg_update_kernel<float, 1><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+            gm_pcg_update_kernel<float, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
                 N, (float*)x, (float*)r, (float*)z, (const float*)p, (const float*)q,
                 prec_ptr<float>(c, which), sc, maxit, rc, pairprec<float>(c, which));
     }
@@ -295,7 +271,7 @@ __global__ void gm_axpby_kernel(long long n, double a, const double* x, double b
 int gm_launch_axpby(gm_ctx* c, long long n, double a, const double* x, double b, double* y,
                     cudaStream_t s)
 {
-    gm_axpby_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, a, x, b, y);
+    gm_axpby_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, a, x, b, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
@@ -346,33 +322,33 @@ int gm_launch_cast_scaled_d2f(gm_ctx* c, long long n, const double* x, float* y,
 {
     int rc = gm_launch_dot(c, n, x, x, nullptr, nullptr, sc, s);
     if (rc) return rc;
-    gm_d2f_scaled_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, x, y, sc);
+    gm_d2f_scaled_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y, sc);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_axpy_scaled_f2d(gm_ctx* c, long long n, const double* sc, const float* x, double* y,
                               cudaStream_t s)
 {
-    gm_axpy_f2d_scaled_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, sc, x, y);
+    gm_axpy_f2d_scaled_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, sc, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 
 int gm_launch_copy_cast_d2f(gm_ctx* c, long long n, const double* x, float* y, cudaStream_t s)
 {
-    gm_d2f_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, x, y);
+    gm_d2f_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_copy_cast_f2d(gm_ctx* c, long long n, const float* x, double* y, cudaStream_t s)
 {
-    gm_f2d_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, x, y);
+    gm_f2d_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_axpy_f2d(gm_ctx* c, long long n, double a, const float* x, double* y, cudaStream_t s)
 {
-    gm_axpy_f2d_kernel<<<GM_RED_BLOCKS, 256, 0, s>>>(n, a, x, y);
+    gm_axpy_f2d_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, a, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
@@ -396,7 +372,7 @@ gm_dot_kernel(long long n, const double* x, const double* y, const double* x2, c
 int gm_launch_dot(gm_ctx* c, long long n, const double* x, const double* y, const double* x2,
                   const double* y2, double* out, cudaStream_t s)
 {
-    gm_dot_kernel<<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(n, x, y, x2, y2, out, redctx(c));
+    gm_dot_kernel<<<gm_red_blocks(n), GM_RED_THREADS, 0, s>>>(n, x, y, x2, y2, out, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;
 }
@@ -419,7 +395,10 @@ gm_pcg_update_noz_kernel(long long n, T* x, T* r, const T* p, const T* q, PcgSca
         x[i] = fma(alpha, p[i], x[i]);
         const T ri = fma(-alpha, q[i], r[i]);
         r[i] = ri;
-        v[0] += (double)ri * (double)ri;
+        {
+            const double w = gm_widen(ri);
+            v[0] = fma(w, w, v[0]);
+        }
     }
     if (gm_grid_sum_l<1>(v, rc.part, rc.counter)) {
         sc->it += 1;
@@ -444,7 +423,7 @@ gm_pcg_rz_kernel(long long n, const T* r, const T* z, PcgScalars* sc, int init, 
     double v[1] = {0.0};
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
-        v[0] += (double)r[i] * (double)z[i];
+        v[0] = fma(gm_widen(r[i]), gm_widen(z[i]), v[0]);
     if (gm_grid_sum_l<1>(v, rc.part, rc.counter)) {
         if (!isfinite(v[0]) || !(v[0] > 0.0)) {
             sc->status = isfinite(v[0]) ? GM_ENOCONV : GM_ENAN;
@@ -462,10 +441,10 @@ int gm_launch_pcg_update_noz(gm_ctx* c, int prec, void* x, void* r, const void* 
                              PcgScalars* sc, int maxit, cudaStream_t s)
 {
     if (prec == GM_F64)
-        gm_pcg_update_noz_kernel<double><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+        gm_pcg_update_noz_kernel<double><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(
             3 * c->N, (double*)x, (double*)r, (const double*)p, (const double*)q, sc, maxit, redctx(c));
     else
-        gm_pcg_update_noz_kernel<float><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(
+        gm_pcg_update_noz_kernel<float><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(
             3 * c->N, (float*)x, (float*)r, (const float*)p, (const float*)q, sc, maxit, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;
@@ -475,10 +454,10 @@ int gm_launch_pcg_rz(gm_ctx* c, int prec, const void* r, const void* z, PcgScala
                      cudaStream_t s)
 {
     if (prec == GM_F64)
-        gm_pcg_rz_kernel<double><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(3 * c->N, (const double*)r,
+        gm_pcg_rz_kernel<double><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(3 * c->N, (const double*)r,
                                                                         (const double*)z, sc, init, redctx(c));
     else
-        gm_pcg_rz_kernel<float><<<GM_RED_BLOCKS, GM_RED_THREADS, 0, s>>>(3 * c->N, (const float*)r,
+        gm_pcg_rz_kernel<float><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(3 * c->N, (const float*)r,
                                                                        (const float*)z, sc, init, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;

@@ -44,13 +44,14 @@ __device__ inline void gm_dot_node(const T (&r)[NC], const T (&z)[NC], double (&
             a = fma(r[c], z[c], a);
             b = fma(r[c], r[c], b);
         }
-        v[0] += (double)a;
-        v[1] += (double)b;
+        v[0] += gm_widen(a);
+        v[1] += gm_widen(b);
     } else {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            v[0] += (double)r[c] * (double)z[c];
-            v[1] += (double)r[c] * (double)r[c];
+            const double rd = gm_widen(r[c]);
+            v[0] = fma(rd, gm_widen(z[c]), v[0]);
+            v[1] = fma(rd, rd, v[1]);
         }
     }
 }
