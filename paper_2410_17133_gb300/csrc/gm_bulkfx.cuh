@@ -4,8 +4,8 @@
 // Why: the FP64 kernel is bound by the FP64 pipe (2 lanes per clock and SM).
 // In the parity basis a K_b element takes about 210 FP64 instructions, 64
 // issue slots each; the same element takes about 2200 integer instructions here
-// (560 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
-// per product: K_T on 128^3 dipping cells 1254 -> 403; K_T + A_pu + A_up + A22 on
+// (490 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
+// per product: K_T on 128^3 dipping cells 1254 -> 376; K_T + A_pu + A_up + A22 on
 // 61x127x46 cells sheared both ways 804 -> 274 (A22 121 -> 46); J on 8^3 cells
 // 89 -> 47.
 //
@@ -49,7 +49,7 @@ constexpr size_t gm_fx_smem()
 }
 
 // Output mode s of displacement field c of one element with modulus limbs E:
-// K_b row times the element's input modes, times E.
+// K_b row times the element's input modes, times E (limbs of gm_fx_coef22).
 template <int CLS>
 __device__ __forceinline__ void gm_fx_k_mode(const RefFx& F, const int (&xv)[24][3], int c, int s, const int (&E)[3],
                                              int (&y)[3])
@@ -60,7 +60,7 @@ __device__ __forceinline__ void gm_fx_k_mode(const RefFx& F, const int (&xv)[24]
     for (int j = 0; j < 24; ++j)
         if (PP.k[c * 8 + s][j] >= 0 && (j & 7) != 0) {
             const int* k = F.k[PP.k[c * 8 + s][j]];
-            gm_fx_mac(acc, xv[j], k[2], k[1], k[0]);
+            gm_fx_mac2(acc, xv[j], k[1], k[0]);
         }
     int r[3];
     gm_fx_carry(acc, r);
@@ -314,7 +314,7 @@ gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_const
                         xv[f * 8 + q + 4][i] = b[q][i] - t[q][i];
                     }
             }
-            if constexpr (DO_K) gm_fx_coef(Ed, F.topE, E);
+            if constexpr (DO_K) gm_fx_coef22(Ed, F.topE, E);
             if constexpr (DO_Q) gm_fx_coef(Ed, Q.topW, E);
         }
 #pragma unroll

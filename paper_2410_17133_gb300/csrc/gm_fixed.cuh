@@ -11,7 +11,8 @@
 //     of two at or above the largest input of the tile;
 //   - 8-point transforms and sums of up to 28 (signed limbs: 36) results fit the words;
 //   - coefficients: |c| < 1 as c2 2^-26 + c1 2^-52 + c0 2^-78, exact for the
-//     53 bits of a double within 2^25 of the largest;
+//     53 bits of a double within 2^25 of the largest (moduli: within 2^21; the
+//     entries of K_b as two limbs, to 2^-57 of a row's sum);
 //   - a product sum loses at most about 2^3 units of the last place (the limb
 //     pairs below it), a node of the operators about 2^6, so results are exact
 //     to 2^-69 of the tile's largest term, 16 bits below FP64's rounding.
@@ -78,6 +79,21 @@ __host__ __device__ inline void gm_fx_coef(double c, int top, int (&l)[3])
     l[0] = (s0 >= 0 ? (int)(M >> s0) : (int)(M << -s0)) & GM_FX_MASK;
 }
 
+// limbs of a coefficient 0 <= c < 1 as l2 2^-22 + l1 2^-48 + l0 2^-74
+__host__ __device__ inline void gm_fx_coef22(double c, int top, int (&l)[3])
+{
+    const int64_t b = gm_fx_bits(c);
+    const int e = (int)((uint64_t)b >> 52) & 0x7ff;
+    const uint64_t m = e ? (((uint64_t)b & 0xfffffffffffffull) | 0x10000000000000ull) : 0ull;
+    int d = top - e;                               // c = m 2^(74 - 53 - d) units of 2^-74
+    const uint64_t M = d < 74 ? m << 11 : 0;       // 74 bits: M 2^(10 - d)
+    if (d > 73) d = 73;
+    const int s2 = 42 + d, s1 = 16 + d, s0 = d - 10;
+    l[2] = s2 < 64 ? (int)(M >> s2) : 0;
+    l[1] = s1 < 64 ? (int)(M >> s1) & GM_FX_MASK : 0;
+    l[0] = (s0 >= 0 ? (int)(M >> s0) : (int)(M << -s0)) & GM_FX_MASK;
+}
+
 // sums of limb products of one result, by weight
 struct FxAcc {
     int64_t a2, a1, a0;
@@ -91,6 +107,19 @@ __host__ __device__ inline void gm_fx_mac(FxAcc& s, const int (&x)[3], int c2, i
     s.a0 += (int64_t)x[1] * c1;
     s.a0 += (int64_t)x[2] * c0;
 }
+// The same with a coefficient of two limbs, c2 2^-30 + c1 2^-56 (|c2| <= 2^30):
+// five multiplications instead of six.  Sums and carried limbs then weigh 2^4
+// less: (2^48, 2^22, 2^-4); multiplied by a coefficient whose top limb has 22 bits
+// (gm_fx_coef22) they are back at (2^52, 2^26, 1).
+__host__ __device__ inline void gm_fx_mac2(FxAcc& s, const int (&x)[3], int c2, int c1)
+{
+    s.a2 += (int64_t)x[2] * c2;
+    s.a1 += (int64_t)x[1] * c2;
+    s.a1 += (int64_t)x[2] * c1;
+    s.a0 += (int64_t)x[0] * c2;
+    s.a0 += (int64_t)x[1] * c1;
+}
+
 // carried limbs: l0, l1 in [0, 2^26), l2 signed
 __host__ __device__ inline void gm_fx_carry(const FxAcc& s, int (&l)[3])
 {

@@ -161,14 +161,20 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
     F.eA = (as > 0.0 ? std::ilogb(as) + 1 : 0) + 1;
     for (int i = 0; i < 24; ++i) {
         for (int j = 0; j < 24; ++j)
-            if (PP.k[i][j] >= 0) fx_limbs(Kt[i][j], 0.0, F.eK, F.k[PP.k[i][j]]);
+            if (PP.k[i][j] >= 0) {
+                // c2 2^-30 + c1 2^-56, c1 in [-2^25, 2^25]
+                const int64_t n = (int64_t)std::nearbyint(std::ldexp(Kt[i][j], 56 - F.eK));
+                const int64_t hi = (n + (1ll << 25)) >> 26;
+                F.k[PP.k[i][j]][1] = (int)hi;
+                F.k[PP.k[i][j]][0] = (int)(n - hi * (1ll << 26));
+            }
         for (int j = 0; j < 8; ++j)
             if (PP.a[i][j] >= 0) {
                 const double hi = alpha * At[i][j];
                 fx_limbs(hi, std::fma(alpha, At[i][j], -hi), F.eA, F.a[PP.a[i][j]]);
             }
     }
-    // moduli: limbs are exact while the smallest is within 2^25 of the largest;
+    // moduli: limbs are exact while the smallest is within 2^21 of the largest;
     // what a low modulus loses against the tile's unit comes off the grading
     F.topE = std::ilogb(Emax) + 1023;
     F.gradeK = GM_FX_GRADE - (std::ilogb(Emax) - std::ilogb(Emin));

@@ -264,7 +264,7 @@ mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_const
                     }
                 const T Ee = sE[(size_t)(row + lay) * faces + f];
                 int El[3] = {0, 0, 0};
-                if constexpr (FX) gm_fx_coef(Ee, F.topE, El);
+                if constexpr (FX) gm_fx_coef22(Ee, F.topE, El);
                 auto field = [&](auto c_) {
                     constexpr int c = decltype(c_)::value;
                     W o[4][NL];

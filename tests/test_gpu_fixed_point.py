@@ -178,6 +178,15 @@ HOST = r"""
 extern "C" {
 void from_double(double x, int top, int* l) { int v[3]; gm_fx_from_double(x, top, v); for (int i = 0; i < 3; ++i) l[i] = v[i]; }
 void coef(double x, int top, int* l) { int v[3]; gm_fx_coef(x, top, v); for (int i = 0; i < 3; ++i) l[i] = v[i]; }
+void coef22(double x, int top, int* l) { int v[3]; gm_fx_coef22(x, top, v); for (int i = 0; i < 3; ++i) l[i] = v[i]; }
+void product2(const int* x, const int* k, int n, int* l)
+{
+    FxAcc s{0, 0, 0};
+    for (int i = 0; i < n; ++i) { int v[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]}; gm_fx_mac2(s, v, k[2 * i + 1], k[2 * i]); }
+    int r[3];
+    gm_fx_carry(s, r);
+    for (int i = 0; i < 3; ++i) l[i] = r[i];
+}
 double to_double(int a, int b, int c) { return gm_fx_to_double(a, b, c); }
 double to_double4(int a, int b, int c, int d) { return gm_fx_to_double4(a, b, c, d); }
 void product4(const int* x, const int* k, int n, int* l)
@@ -211,7 +220,7 @@ def host(tmp_path_factory):
                     os.path.join(ROOT, "paper_2410_17133_gb300", "csrc"), "-o", so, str(d / "h.cpp")], check=True)
     lib = ctypes.CDLL(so)
     lib.to_double.restype = lib.to_double4.restype = ctypes.c_double
-    lib.from_double.argtypes = lib.coef.argtypes = [ctypes.c_double, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    lib.from_double.argtypes = lib.coef.argtypes = lib.coef22.argtypes = [ctypes.c_double, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     return lib
 
 
@@ -234,6 +243,32 @@ def test_limbs_and_back(host):
         a, b = (int(v) for v in rng.integers(-2 ** 31 + 1, 2 ** 31, 2) >> rng.integers(0, 31, 2))
         c = int(rng.integers(-2 ** 30, 2 ** 30)) >> int(rng.integers(0, 31))
         assert host.to_double(a, b, c) == float((c << 52) + (b << 26) + a)   # int -> float rounds to nearest even
+
+
+def test_two_limb_coefficients(host):
+    rng = np.random.default_rng(8)
+    l = (ctypes.c_int * 3)()
+    P = ctypes.POINTER(ctypes.c_int)
+    for t in range(300):
+        c = float(rng.uniform(0, 1)) * 2.0 ** -int(rng.integers(0, 90))
+        host.coef22(c, 1022, l)
+        m, e = c.as_integer_ratio()
+        assert (int(l[2]) << 52) + (int(l[1]) << 26) + int(l[0]) == (m << 74) // e
+        # a row of entries whose absolute sum is 1, at the largest inputs, on one sign or mixed
+        n = int(rng.integers(1, 25))
+        w = rng.dirichlet(np.ones(n)) if t % 2 else np.eye(n)[0]
+        s = np.ones(n, int) if t % 4 < 2 else rng.choice([-1, 1], n)
+        k = np.zeros((n, 2), np.int32)
+        x = np.zeros((n, 3), np.int32)
+        for i in range(n):
+            v = int(w[i] * 2 ** 56) * int(s[i])
+            hi = (v + 2 ** 25) >> 26
+            k[i] = [v - (hi << 26), hi]
+            x[i] = int(s[i]) * np.array([2 ** 29 - 8, 2 ** 29 - 8, 2 ** 26 - 8])
+        host.product2(x.ctypes.data_as(P), k.ctypes.data_as(P), n, l)
+        exact = sum(value(x[i]) * ((int(k[i][1]) << 26) + int(k[i][0])) for i in range(n))
+        # limbs weigh 2^48, 2^22, 2^-4; the pair left out is below 2^54 2^-56
+        assert abs(value(l) * 2 ** 52 - exact) <= (2 + 16 * n) * 2 ** 52
 
 
 def test_four_limbs_and_back(host):
