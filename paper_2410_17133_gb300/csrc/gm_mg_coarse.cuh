@@ -43,7 +43,6 @@ struct CoarseArgs {
     FaultK<T> fk;
     const double* coef;  // (c1, c2) per step
     int deg, rows;       // rows of a CTA at most
-    int fixedin;         // b and the nodal inverses are copied to shared memory
     unsigned m_rn, m_rowlen, m_nx, m_faces;   // ceil(2^32 / d): quotients by one multiplication
     const int* skip;
 };
@@ -60,16 +59,17 @@ __host__ __device__ inline int mgc_row(const GridDesc& g, int r, int n)
     return r * q + (r < rem ? r : rem);
 }
 
-// Shared memory of a CTA in bytes from the start: iterate (two buffers),
-// direction and residual of its rows, staged rows as words, what the layers
-// around a row give it, modulus and mask of the staged part; with `fixedin` also
-// b and the nodal inverses (the cluster barrier empties the L1 cache, so what is
-// read in every step would come from L2 each time).
+// Shared memory of a CTA in bytes from the start: iterate (two buffers), right
+// side, direction and residual of its rows, staged rows as words, what the layers around a row give
+// it, modulus and mask of the staged part, nodal and pair inverses, tangents, and
+// what each (node, component) item reads (the
+// cluster barrier empties the L1 cache: what is read in every step would come
+// from L2 each time).
 struct MgcLayout {
-    size_t x, d, r, st, out, E, mask, b, mi, total;
+    size_t x, b, d, r, st, out, E, mask, mi, item, P, D, total;
 };
 template <typename T, typename MT>
-__host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows, bool fixedin)
+__host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows)
 {
     const size_t rn = (size_t)(g.nx + 1) * g.nplanes, faces = (size_t)g.nx * g.nz, NL = mgc_limbs<T>();
     MgcLayout L{};
@@ -80,15 +80,18 @@ __host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows, boo
         return p;
     };
     L.x = put(2 * rows * 3 * rn * sizeof(T));
+    L.b = put(rows * 3 * rn * sizeof(T));
     L.d = put(rows * 3 * rn * sizeof(T));
     L.r = put(rows * 3 * rn * sizeof(T));
     L.st = put((rows + 2) * 3 * NL * rn * 4);
     L.out = put(rows * 2 * 12 * NL * faces * 4);
     L.E = put((rows + 1) * faces * sizeof(T));
     L.mask = put((rows + 2) * rn);
-    if (fixedin) {
-        L.b = put(rows * 3 * rn * sizeof(T));
-        L.mi = put(rows * 6 * rn * sizeof(MT));
+    L.mi = put(rows * 6 * rn * sizeof(MT));
+    L.item = put(rows * 3 * rn * sizeof(int2));
+    if (g.kf >= 0) {
+        L.P = put((size_t)rows * 36 * (g.nx + 1) * sizeof(T));
+        L.D = put((size_t)rows * 6 * (g.nx + 1) * sizeof(T));
     }
     L.total = at;
     return L;
@@ -111,15 +114,18 @@ mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_const
     extern __shared__ __align__(16) unsigned char mgc_raw[];
     __shared__ int s_top[NT / 32];
     const GridDesc& g = a.g;
-    const MgcLayout L = mgc_layout<T, MT>(g, a.rows, a.fixedin != 0);
+    const MgcLayout L = mgc_layout<T, MT>(g, a.rows);
     const int rowlen = g.nx + 1, rn = rowlen * g.nplanes, faces = g.nx * g.nz;
     const long long N = g.N;
     const int tid = threadIdx.x;
     T* sx = reinterpret_cast<T*>(mgc_raw + L.x);                    // [buffer][row][field][node]
+    T* sb = reinterpret_cast<T*>(mgc_raw + L.b);                    // [row][field][node]
     T* sd = reinterpret_cast<T*>(mgc_raw + L.d);                    // [row][field][node]
     T* sr = reinterpret_cast<T*>(mgc_raw + L.r);                    // [row][field][node]
-    T* sb = reinterpret_cast<T*>(mgc_raw + L.b);                    // [row][field][node]
     MT* smi = reinterpret_cast<MT*>(mgc_raw + L.mi);                // [row][entry][node]
+    int2* sit = reinterpret_cast<int2*>(mgc_raw + L.item);          // first word of its layers' results; flags
+    T* sP = reinterpret_cast<T*>(mgc_raw + L.P);                    // [row][entry][pair of the row]
+    T* sD = reinterpret_cast<T*>(mgc_raw + L.D);                    // [row][entry][pair of the row]
     W* st = reinterpret_cast<W*>(mgc_raw + L.st);                   // [staged row][field][limb][node]
     W* out = reinterpret_cast<W*>(mgc_raw + L.out);                 // [row][layer][field][corner][limb][face]
     T* sE = reinterpret_cast<T*>(mgc_raw + L.E);                    // [layer][face]
@@ -143,15 +149,32 @@ mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_const
             sE[q] = j >= 0 && j < g.ny ? a.E[(f - ek * g.nx) + (long long)g.nx * (j + (long long)g.ny * ek)] : T(0);
         }
     }
-    if (a.fixedin)
-        for (int row = 0; row < own; ++row)
-            for (int n = tid; n < rn; n += NT) {
-                const long long gn = node(n, j0 + row);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) sb[(size_t)(row * 3 + c) * rn + n] = a.b[c * N + gn];
-#pragma unroll
-                for (int k = 0; k < 6; ++k) smi[(size_t)(row * 6 + k) * rn + n] = a.mi[k * N + gn];
-            }
+    if (g.kf >= 0)
+        for (int q = tid; q < own * 42 * rowlen; q += NT) {
+            const int row = q / (42 * rowlen), e = (q - row * 42 * rowlen) / rowlen, i = q % rowlen;
+            const long long pair = i + (long long)rowlen * (j0 + row);
+            if (e < 36) sP[(size_t)(row * 36 + e) * rowlen + i] = a.pp.inv[e * a.pp.nb + pair];
+            else sD[(size_t)(row * 6 + e - 36) * rowlen + i] = a.fk.D[(e - 36) * g.nb + pair];
+        }
+    // the (node, component) items
+    constexpr int FIXED = 16, LIP = 32, UPPER = 64;
+    for (int it = tid; it < own * 3 * rn; it += NT) {
+        const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3;
+        const int kk = mgc_div(n, a.m_rowlen), i = n - kk * rowlen;
+        const long long gn = node(n, j0 + row);
+        const bool above = kk + 1 < g.nplanes && kk != g.kf, below = kk > 0 && kk - 1 != g.kf;
+        // bit dx + 2 dz: the element to the left (dx) and below in z (dz) of the node exists
+        int fl = 0;
+        if (above && i < g.nx) fl |= 1;
+        if (above && i > 0) fl |= 2;
+        if (below && i < g.nx) fl |= 4;
+        if (below && i > 0) fl |= 8;
+        if ((sm[(size_t)(row + 1) * rn + n] >> c) & 1u) fl |= FIXED;
+        if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) fl |= LIP | (kk > g.kf ? UPPER : 0);
+        sit[it] = make_int2((row * 6 + c) * 4 * NL * faces + i + g.nx * (kk - (g.kf >= 0 && kk > g.kf ? 1 : 0)), fl);
+        sb[it] = a.b[c * N + gn];
+        for (int k = c; k < 6; k += 3) smi[(size_t)(row * 6 + k) * rn + n] = a.mi[k * N + gn];
+    }
     __syncthreads();
 
     for (int step = 0; step < a.deg; ++step) {
@@ -308,48 +331,40 @@ mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_const
         }
         // residual r = b - K_T x
         for (int it = tid; it < own * 3 * rn; it += NT) {
-            const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3, j = j0 + row;
-            const int kk = mgc_div(n, a.m_rowlen), i = n - kk * rowlen;
-            const bool fixed = (sm[(size_t)(row + 1) * rn + n] >> c) & 1u;
-            T r = a.fixedin ? sb[it] : a.b[c * N + i + (long long)rowlen * (j + (long long)(g.ny + 1) * kk)];
-            if (step > 0 && !fixed) {
+            const int2 item = sit[it];
+            const int fl = item.y;
+            T r = sb[it];
+            if (step > 0 && !(fl & FIXED)) {
                 W s[NL];
 #pragma unroll
                 for (int l = 0; l < NL; ++l) s[l] = W(0);
 #pragma unroll
-                for (int dz = 0; dz < 2; ++dz) {                // elements above and below in z
-                    const int kb = kk - dz;
-                    if (kb < 0 || kb + 1 >= g.nplanes || kb == g.kf) continue;
-                    const int ek = (g.kf >= 0 && kb > g.kf) ? kb - 1 : kb;
+                for (int q = 0; q < 4; ++q) {
+                    const int dx = q & 1, dz = q >> 1;
+                    const W* w = out + item.x + q * NL * faces - dx - dz * g.nx;
+                    if (fl & (1 << q))
 #pragma unroll
-                    for (int dx = 0; dx < 2; ++dx) {
-                        const int fi = i - dx;
-                        if (fi < 0 || fi >= g.nx) continue;
-#pragma unroll
-                        for (int lay = 0; lay < 2; ++lay)
-#pragma unroll
-                            for (int l = 0; l < NL; ++l)
-                                s[l] += out[(size_t)((((row * 2 + lay) * 3 + c) * 4 + dx + 2 * dz) * NL + l) * faces + fi + g.nx * ek];
-                    }
+                        for (int l = 0; l < NL; ++l) s[l] += w[l * faces] + w[(12 * NL + l) * faces];
                 }
                 if constexpr (FX) r -= scale * gm_fx_to_double(s[0], s[1], s[2]);
                 else r -= s[0];
-                if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) {
+                if (fl & LIP) {
                     // cohesive force +-A_i D [[x]]
-                    const int nl = i + rowlen * g.kf, nu = nl + rowlen;
-                    const int nqi = (i > 0) + (i < g.nx), nqj = (j > 0) + (j < g.ny);
+                    const int blk = mgc_div(it, a.m_rn), row = blk / 3, c = blk - row * 3, j = j0 + row;
+                    const int i = mgc_div(it - blk * rn, a.m_rowlen), p = it - blk * rn - i * rowlen;
+                    const int nl = p + rowlen * g.kf, nu = nl + rowlen;
+                    const int nqi = (p > 0) + (p < g.nx), nqj = (j > 0) + (j < g.ny);
                     const T Ai = a.fk.Aq * T(0.25) * T(nqi * nqj);
-                    const long long P = g.nb, q = i + (long long)rowlen * j;
+                    const uint8_t* mk = sm + (size_t)(row + 1) * rn;
                     T f = T(0);
 #pragma unroll
                     for (int e = 0; e < 3; ++e) {
-                        const T up = ((sm[(size_t)(row + 1) * rn + nu] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nu];
-                        const T um = ((sm[(size_t)(row + 1) * rn + nl] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nl];
+                        const T up = ((mk[nu] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nu];
+                        const T um = ((mk[nl] >> e) & 1u) ? T(0) : xi[(size_t)(row * 3 + e) * rn + nl];
                         const int lo = c < e ? c : e, hi = c < e ? e : c;
-                        const int k = lo == 0 ? hi : lo + hi + 1;       // 00 01 02 11 12 22
-                        f = fma(a.fk.D[k * P + q], up - um, f);
+                        f = fma(sD[(size_t)(row * 6 + (lo == 0 ? hi : lo + hi + 1)) * rowlen + p], up - um, f);
                     }
-                    r = kk == g.kf ? fma(Ai, f, r) : fma(-Ai, f, r);
+                    r = (fl & UPPER) ? fma(-Ai, f, r) : fma(Ai, f, r);
                 }
             }
             sr[it] = r;
@@ -357,30 +372,27 @@ mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_const
         __syncthreads();
         // z = M^-1 r, d = c1 d + c2 z, x = x + d
         for (int it = tid; it < own * 3 * rn; it += NT) {
-            const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3, j = j0 + row;
-            const int kk = mgc_div(n, a.m_rowlen), i = n - kk * rowlen;
-            const long long gn = i + (long long)rowlen * (j + (long long)(g.ny + 1) * kk);
+            const int fl = sit[it].y;
+            const int blk = mgc_div(it, a.m_rn), n = it - blk * rn, row = blk / 3, c = blk - row * 3;
+            const T* rr = sr + (size_t)row * 3 * rn;
             T z = T(0);
-            if (g.kf >= 0 && (kk == g.kf || kk == g.kf + 1)) {
-                const int nl = i + rowlen * g.kf, ra = (kk - g.kf) * 3 + c;
-                const long long q = i + (long long)rowlen * j;
+            if (fl & LIP) {
+                const int p = n - mgc_div(n, a.m_rowlen) * rowlen, nl = p + rowlen * g.kf;
+                const T* P = sP + (size_t)(row * 36 + ((fl & UPPER ? 3 : 0) + c) * 6) * rowlen + p;
 #pragma unroll
-                for (int e = 0; e < 6; ++e)
-                    z = fma(a.pp.inv[(ra * 6 + e) * a.pp.nb + q], sr[(size_t)(row * 3 + e % 3) * rn + nl + (e < 3 ? 0 : rowlen)], z);
+                for (int e = 0; e < 6; ++e) z = fma(P[(size_t)e * rowlen], rr[(size_t)(e % 3) * rn + nl + (e < 3 ? 0 : rowlen)], z);
             } else {
 #pragma unroll
                 for (int e = 0; e < 3; ++e) {
                     const int lo = c < e ? c : e, hi = c < e ? e : c;
-                    const int k = lo == 0 ? hi : lo + hi + 1;
-                    z = fma(mg_ld<T>(a.fixedin ? smi + (size_t)(row * 6 + k) * rn + n : a.mi + k * N + gn),
-                            sr[(size_t)(row * 3 + e) * rn + n], z);
+                    z = fma(mg_ld<T>(smi + (size_t)(row * 6 + (lo == 0 ? hi : lo + hi + 1)) * rn + n), rr[(size_t)e * rn + n], z);
                 }
             }
             const T dn = step > 0 ? fma(c1, sd[it], c2 * z) : c2 * z;
             const T xn = step > 0 ? xi[it] + dn : dn;
             sd[it] = dn;
             if (step + 1 < a.deg) xo[it] = xn;
-            else a.x[c * N + gn] = xn;
+            else a.x[c * N + node(n, j0 + row)] = xn;
         }
         // the step's rows are complete; in the last step: nobody reads this CTA's rows any more
         cl.sync();
