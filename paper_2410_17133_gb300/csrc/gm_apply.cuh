@@ -50,8 +50,9 @@ __device__ inline double gm_block_sum_fixed(const double* part, int n)
 
 template <typename T, int MODE, bool PCG>
 __global__ void __launch_bounds__(256)
-gm_fault_apply_kernel(const FaultArgs<T> a)
+gm_fault_apply_kernel(int chained, const FaultArgs<T> a)
 {
+    gm_chain(chained);
     constexpr bool DO_KF = (MODE & GM_M_KF) != 0;
     constexpr bool DO_APU = (MODE & GM_M_APU) != 0;
     constexpr bool DO_AUP = (MODE & GM_M_AUP) != 0;
@@ -204,8 +205,9 @@ gm_fault_apply_kernel(const FaultArgs<T> a)
 
 // Without a fault, one block closes the p.Ap reduction of the bulk partials.
 static __global__ void __launch_bounds__(256)
-gm_pcg_alpha_finalize_kernel(const double* part, int n, PcgScalars* sc)
+gm_pcg_alpha_finalize_kernel(int chained, const double* part, int n, PcgScalars* sc)
 {
+    gm_chain(chained);
     if (sc->done) return;
     const double pq = gm_block_sum_fixed(part, n);
     if (threadIdx.x == 0) gm_pcg_alpha_from(sc, pq);
@@ -283,9 +285,9 @@ static int gm_bulk32_launch(gm_ctx* c, BulkArgs<float>& b, cudaStream_t s)
     const int gz = (c->g.nplanes + zc - 1) / zc;
     b.zchunk = zc;
 #if GM32_PACKED_PRODUCTS
-    gm_bulk32_kernel<CLS, MODE, PCG><<<dim3(gx, gy, gz), gm32::NT, SMEM, s>>>(b, c->R32p);
+    gm_launch_chained(gm_bulk32_kernel<CLS, MODE, PCG>, dim3(gx, gy, gz), gm32::NT, SMEM, s, b, c->R32p);
 #else
-    gm_bulk32_kernel<CLS, MODE, PCG><<<dim3(gx, gy, gz), gm32::NT, SMEM, s>>>(b, c->R32);
+    gm_launch_chained(gm_bulk32_kernel<CLS, MODE, PCG>, dim3(gx, gy, gz), gm32::NT, SMEM, s, b, c->R32);
 #endif
     return gx * gy * gz;
 }
@@ -391,7 +393,7 @@ static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accu
     b.zchunk = zc;
     b.cfx = factor;
     b.accumulate = accumulate ? 1 : 0;
-    gm_bulk_fx_kernel<CLS, MODE, DOT><<<dim3(gx, gy, gz), 256, gm_fx_smem<MODE>(), s>>>(b, c->Rfx, c->R64, Q);
+    gm_launch_chained(gm_bulk_fx_kernel<CLS, MODE, DOT>, dim3(gx, gy, gz), 256, gm_fx_smem<MODE>(), s, b, c->Rfx, c->R64, Q);
     c->applies++;
     c->launches++;
     return gx * gy * gz;
@@ -402,9 +404,10 @@ static int gm_fx_launch(gm_ctx* c, BulkArgs<double>& b, double factor, bool accu
 // needs the whole direction before it can scale it).
 template <int NC>
 static __global__ void __launch_bounds__(256)
-gm_pcg_dir_kernel(GridDesc g, const double* z, const double* p_old, double* p, const uint8_t* mask,
+gm_pcg_dir_kernel(int chained, GridDesc g, const double* z, const double* p_old, double* p, const uint8_t* mask,
                   const PcgScalars* sc)
 {
+    gm_chain(chained);
     if (sc->done) return;
     const double beta = sc->beta;
     const long long N = g.N, s0 = (NC == 1 && g.tied) ? g.nb * (g.kf + 1) : -1;
@@ -444,7 +447,7 @@ static void gm_apply_launch_t(gm_ctx* c, const RefOps<T>& R, double cK, double c
             } else {
                 b.zchunk = zchunk;
                 b.accumulate = 0;
-                gm_bulk_apply_kernel<T, CLS, GM_FX_FLOW, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+                gm_launch_chained(gm_bulk_apply_kernel<T, CLS, GM_FX_FLOW, false>, dim3(gx, gy, gz), 256, 0, s, b, R);
                 c->applies++;
                 c->launches++;
             }
@@ -454,7 +457,7 @@ static void gm_apply_launch_t(gm_ctx* c, const RefOps<T>& R, double cK, double c
         if constexpr (BULK == GM_M_K || BULK == (GM_M_S | GM_M_C))
             gm_bulk32_launch<CLS, BULK, false>(c, b, s);
         else
-            gm_bulk_apply_kernel<T, CLS, BULK, false><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+            gm_launch_chained(gm_bulk_apply_kernel<T, CLS, BULK, false>, dim3(gx, gy, gz), 256, 0, s, b, R);
         c->applies++;
         c->launches++;
     }
@@ -466,7 +469,7 @@ static void gm_apply_launch_t(gm_ctx* c, const RefOps<T>& R, double cK, double c
         f.D = D;
         f.skip = skip;
         const int nblk = (int)((c->g.nb + 255) / 256);
-        gm_fault_apply_kernel<T, MODE, false><<<nblk, 256, 0, s>>>(f);
+        gm_launch_chained(gm_fault_apply_kernel<T, MODE, false>, nblk, 256, 0, s, f);
         c->launches++;
     }
 }
@@ -518,7 +521,7 @@ static void gm_pcg_apply_t(gm_ctx* c, const RefOps<T>& R, const T* z, const T* p
         c->launches++;
     } else if constexpr (U) {
         const int nblk = (int)std::min<long long>((c->N + 255) / 256, GM_RED_BLOCKS);
-        gm_pcg_dir_kernel<3><<<nblk, 256, 0, s>>>(c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
+        gm_launch_chained(gm_pcg_dir_kernel<3>, nblk, 256, 0, s, c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
         c->launches++;
         b.xu = p_new;
         nbulk = gm_fx_launch<CLS, GM_M_K, true>(c, b, 1.0, false, s);
@@ -527,12 +530,12 @@ static void gm_pcg_apply_t(gm_ctx* c, const RefOps<T>& R, const T* z, const T* p
         const FlowFx Q = fs == nullptr ? gm_flow_fx(c, cS, cC) : FlowFx{};
         if (fs == nullptr && Q.grade >= 0) {
             const int nblk = (int)std::min<long long>((c->N + 255) / 256, GM_RED_BLOCKS);
-            gm_pcg_dir_kernel<1><<<nblk, 256, 0, s>>>(c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
+            gm_launch_chained(gm_pcg_dir_kernel<1>, nblk, 256, 0, s, c->g, z, p_old, p_new, c->dmask.as<uint8_t>(), sc);
             c->launches++;
             b.xp = p_new;
             nbulk = gm_fx_launch<CLS, GM_FX_FLOW, true>(c, b, 1.0, false, s, Q);
         } else {
-            gm_bulk_apply_kernel<T, CLS, BULK, true><<<dim3(gx, gy, gz), 256, 0, s>>>(b, R);
+            gm_launch_chained(gm_bulk_apply_kernel<T, CLS, BULK, true>, dim3(gx, gy, gz), 256, 0, s, b, R);
             c->applies++;
             c->launches++;
         }
@@ -548,10 +551,10 @@ static void gm_pcg_apply_t(gm_ctx* c, const RefOps<T>& R, const T* z, const T* p
         f.counter = c->dcount.as<unsigned>();
         f.sc = sc;
         const int nblk = (int)((c->g.nb + 255) / 256);
-        gm_fault_apply_kernel<T, MODE, true><<<nblk, 256, 0, s>>>(f);
+        gm_launch_chained(gm_fault_apply_kernel<T, MODE, true>, nblk, 256, 0, s, f);
         c->launches++;
     } else {
-        gm_pcg_alpha_finalize_kernel<<<1, 256, 0, s>>>(part, nbulk, sc);
+        gm_launch_chained(gm_pcg_alpha_finalize_kernel, 1, 256, 0, s, part, nbulk, sc);
         c->launches++;
     }
 }

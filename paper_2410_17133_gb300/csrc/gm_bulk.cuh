@@ -396,8 +396,9 @@ __device__ __forceinline__ void gm_bulk_tile(const BulkArgs<T>& a, const RefOps<
 
 template <typename T, int CLS, int MODE, bool PCG>
 __global__ void __launch_bounds__(256, gm_bulk_min_blocks<T, CLS, MODE>())
-gm_bulk_apply_kernel(const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
+gm_bulk_apply_kernel(int chained, const BulkArgs<T> a, const __grid_constant__ RefOps<T> R)
 {
+    gm_chain(chained);
     if (a.skip != nullptr && *a.skip != 0) return;
     __shared__ BulkTileSmem<T, MODE> sm;
     gm_bulk_tile<T, CLS, MODE, PCG>(a, R, sm);

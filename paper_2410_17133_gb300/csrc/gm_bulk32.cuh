@@ -128,8 +128,9 @@ constexpr int gm32_min_blocks() { return MODE == GM_M_K ? (PCG ? 2 : 3) : 4; }
 
 template <int CLS, int MODE, bool PCG>
 __global__ void __launch_bounds__(gm32::NT, gm32_min_blocks<MODE, PCG>())
-gm_bulk32_kernel(const BulkArgs<float> a, const __grid_constant__ gm32::Ref32 R)
+gm_bulk32_kernel(int chained, const BulkArgs<float> a, const __grid_constant__ gm32::Ref32 R)
 {
+    gm_chain(chained);
     using namespace gm32;
     constexpr bool DO_K = MODE == GM_M_K;
     static_assert(MODE == GM_M_K || MODE == (GM_M_S | GM_M_C), "K or S + dt C");

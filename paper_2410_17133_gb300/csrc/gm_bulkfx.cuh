@@ -6,8 +6,8 @@
 // issue slots each; the same element takes about 2200 integer instructions here
 // (490 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
 // per product: K_T on 128^3 dipping cells 1254 -> 376; K_T + A_pu + A_up + A22 on
-// 61x127x46 cells sheared both ways 804 -> 274 (A22 121 -> 46); J on 8^3 cells
-// 89 -> 47.
+// 61x127x46 cells sheared both ways 804 -> 271 (A22 121 -> 46); J on 8^3 cells
+// 89 -> 42.
 //
 // Each CTA first looks over its inputs: the largest exponent sets the tile's
 // unit, and the smallest of the elements' largest exponents says how far the
@@ -79,9 +79,10 @@ __device__ __noinline__ void gm_fx_fp64_tile(const BulkArgs<double>& a, const Re
 
 template <int CLS, int MODE, bool DOT>
 __global__ void __launch_bounds__(256, 2)
-gm_bulk_fx_kernel(const __grid_constant__ BulkArgs<double> a, const __grid_constant__ RefFx F,
+gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const __grid_constant__ RefFx F,
                   const __grid_constant__ RefOps<double> R, const __grid_constant__ FlowFx Q)
 {
+    gm_chain(chained);
     constexpr bool DO_K = MODE == GM_M_K;
     constexpr bool DO_APU = MODE == GM_M_APU;
     constexpr bool DO_AUP = MODE == GM_M_AUP;

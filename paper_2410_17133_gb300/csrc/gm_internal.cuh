@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/gm.h"
+#include "gm_launch.cuh"
 
 // ---------------------------------------------------------------------------
 // Operator block selection for the matrix-free applies
@@ -608,7 +609,7 @@ constexpr int GM_RED_THREADS = 256;
 inline int gm_red_blocks(long long n)
 {
     const long long one = (n + 255) / 256, four = (n + 1023) / 1024;
-    const long long b = one < 152 ? one : (four < 152 ? 152 : four);
+    const long long b = one < 152 ? one : (four + 151) / 152 * 152;     // whole waves of one block per SM
     return (int)(b < 1 ? 1 : b < GM_RED_BLOCKS ? b : GM_RED_BLOCKS);
 }
 

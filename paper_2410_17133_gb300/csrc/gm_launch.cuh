@@ -1,0 +1,53 @@
+// Launches that overlap with the tail of the kernel before them.
+//
+// The solvers' inner loops are chains of kernels of a few microseconds, each
+// reading what the one before wrote.  With programmatic stream serialisation the
+// next kernel is launched once every CTA of its predecessor has started, takes
+// its place on the SMs and waits in gm_chain until the predecessor has
+// completed and its writes are visible; the launch itself costs no time then.
+// A kernel launched this way takes `chained` first and calls gm_chain(chained)
+// before it touches global memory, in every thread and on every path, so
+// completion is transitive along the chain: a kernel cannot complete before its
+// predecessors have.  Kernels in between that are launched normally wait for
+// completion as usual.  In a captured graph the programmatic edges measured
+// slower than plain ones, so there the launches are plain and gm_chain returns
+// at once.  A time step at 32^3 with its gradient: 55 -> 45 ms together with the
+// coarsest level's shared-memory items; FP32 step at 64^3 84 -> 75 ms.
+#pragma once
+
+#include <cuda_runtime.h>
+
+__device__ __forceinline__ void gm_chain(int chained)
+{
+    if (!chained) return;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+inline bool gm_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();      // the legacy stream while another one captures
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t gm_launch_chained(void (*kernel)(int, Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                     Args&&... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    const int chained = gm_capturing(s) ? 0 : 1;
+    cfg.numAttrs = chained;
+    return cudaLaunchKernelEx(&cfg, kernel, chained, static_cast<Args&&>(args)...);
+}

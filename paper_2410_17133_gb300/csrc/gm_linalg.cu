@@ -50,9 +50,10 @@ struct RedCtx {
 
 template <typename T, int WHICH>
 __global__ void __launch_bounds__(256)
-gm_pcg_init_kernel(long long N, const T* b, const T* q, T* r, T* z, T* p, const T* mi, double rtol,
+gm_pcg_init_kernel(int chained, long long N, const T* b, const T* q, T* r, T* z, T* p, const T* mi, double rtol,
                    PcgScalars* sc, RedCtx rc, PairPrec<T> pp)
 {
+    gm_chain(chained);
     constexpr int NC = Prec<T, WHICH>::NC;
     double v[2] = {0.0, 0.0};
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
@@ -111,9 +112,10 @@ gm_pcg_init_kernel(long long N, const T* b, const T* q, T* r, T* z, T* p, const 
 
 template <typename T, int WHICH>
 __global__ void __launch_bounds__(256)
-gm_pcg_update_kernel(long long N, T* x, T* r, T* z, const T* p, const T* q, const T* mi,
+gm_pcg_update_kernel(int chained, long long N, T* x, T* r, T* z, const T* p, const T* q, const T* mi,
                      PcgScalars* sc, int maxit, RedCtx rc, PairPrec<T> pp)
 {
+    gm_chain(chained);
     constexpr int NC = Prec<T, WHICH>::NC;
     if (sc->done) return;
     const T alpha = (T)sc->alpha;
@@ -209,20 +211,20 @@ int gm_launch_pcg_init(gm_ctx* c, int which, int prec, const void* b, const void
     RedCtx rc = redctx(c);
     if (prec == GM_F64) {
         if (which == 0)
-            gm_pcg_init_kernel<double, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_init_kernel<double, 0>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (const double*)b, (const double*)q, (double*)r, (double*)z, (double*)p,
                 prec_ptr<double>(c, 0), rtol, sc, rc, pairprec<double>(c, 0));
         else
-            gm_pcg_init_kernel<double, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_init_kernel<double, 1>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (const double*)b, (const double*)q, (double*)r, (double*)z, (double*)p,
                 prec_ptr<double>(c, which), rtol, sc, rc, pairprec<double>(c, which));
     } else {
         if (which == 0)
-            gm_pcg_init_kernel<float, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_init_kernel<float, 0>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (const float*)b, (const float*)q, (float*)r, (float*)z, (float*)p,
                 prec_ptr<float>(c, 0), rtol, sc, rc, pairprec<float>(c, 0));
         else
-            gm_pcg_init_kernel<float, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_init_kernel<float, 1>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (const float*)b, (const float*)q, (float*)r, (float*)z, (float*)p,
                 prec_ptr<float>(c, which), rtol, sc, rc, pairprec<float>(c, which));
     }
@@ -237,20 +239,20 @@ int gm_launch_pcg_update(gm_ctx* c, int which, int prec, void* x, void* r, void*
     RedCtx rc = redctx(c);
     if (prec == GM_F64) {
         if (which == 0)
-            gm_pcg_update_kernel<double, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_update_kernel<double, 0>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (double*)x, (double*)r, (double*)z, (const double*)p, (const double*)q,
                 prec_ptr<double>(c, 0), sc, maxit, rc, pairprec<double>(c, 0));
         else
-            gm_pcg_update_kernel<double, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_update_kernel<double, 1>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (double*)x, (double*)r, (double*)z, (const double*)p, (const double*)q,
                 prec_ptr<double>(c, which), sc, maxit, rc, pairprec<double>(c, which));
     } else {
         if (which == 0)
-            gm_pcg_update_kernel<float, 0><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_update_kernel<float, 0>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (float*)x, (float*)r, (float*)z, (const float*)p, (const float*)q,
                 prec_ptr<float>(c, 0), sc, maxit, rc, pairprec<float>(c, 0));
         else
-            gm_pcg_update_kernel<float, 1><<<gm_red_blocks(N), GM_RED_THREADS, 0, s>>>(
+            gm_launch_chained(gm_pcg_update_kernel<float, 1>, gm_red_blocks(N), GM_RED_THREADS, 0, s,
                 N, (float*)x, (float*)r, (float*)z, (const float*)p, (const float*)q,
                 prec_ptr<float>(c, which), sc, maxit, rc, pairprec<float>(c, which));
     }
@@ -261,8 +263,9 @@ int gm_launch_pcg_update(gm_ctx* c, int which, int prec, void* x, void* r, void*
 // ---------------------------------------------------------------------------
 // Generic vector kernels
 // ---------------------------------------------------------------------------
-__global__ void gm_axpby_kernel(long long n, double a, const double* x, double b, double* y)
+__global__ void gm_axpby_kernel(int chained, long long n, double a, const double* x, double b, double* y)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         y[i] = a * x[i] + (b == 0.0 ? 0.0 : b * y[i]);
@@ -271,25 +274,28 @@ __global__ void gm_axpby_kernel(long long n, double a, const double* x, double b
 int gm_launch_axpby(gm_ctx* c, long long n, double a, const double* x, double b, double* y,
                     cudaStream_t s)
 {
-    gm_axpby_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, a, x, b, y);
+    gm_launch_chained(gm_axpby_kernel, gm_red_blocks(n), 256, 0, s, n, a, x, b, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 
-__global__ void gm_d2f_kernel(long long n, const double* x, float* y)
+__global__ void gm_d2f_kernel(int chained, long long n, const double* x, float* y)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         y[i] = (float)x[i];
 }
-__global__ void gm_f2d_kernel(long long n, const float* x, double* y)
+__global__ void gm_f2d_kernel(int chained, long long n, const float* x, double* y)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         y[i] = (double)x[i];
 }
-__global__ void gm_axpy_f2d_kernel(long long n, double a, const float* x, double* y)
+__global__ void gm_axpy_f2d_kernel(int chained, long long n, double a, const float* x, double* y)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         y[i] += a * (double)x[i];
@@ -299,8 +305,9 @@ __global__ void gm_axpy_f2d_kernel(long long n, double a, const float* x, double
 // from sc[0] = x.x (e = 0 when x is zero or not finite); sc[1] = 2^e.  The FP32
 // correction solves then work on values of order one however small the Newton
 // residual has become, away from FP32 subnormals; the scale is exact.
-__global__ void gm_d2f_scaled_kernel(long long n, const double* x, float* y, double* sc)
+__global__ void gm_d2f_scaled_kernel(int chained, long long n, const double* x, float* y, double* sc)
 {
+    gm_chain(chained);
     const double ms = sc[0] / (double)n;
     const int e = (ms > 0.0 && isfinite(ms)) ? ilogb(sqrt(ms)) : 0;
     const double inv = ldexp(1.0, -e);
@@ -309,8 +316,9 @@ __global__ void gm_d2f_scaled_kernel(long long n, const double* x, float* y, dou
          i += (long long)gridDim.x * blockDim.x)
         y[i] = (float)(x[i] * inv);
 }
-__global__ void gm_axpy_f2d_scaled_kernel(long long n, const double* sc, const float* x, double* y)
+__global__ void gm_axpy_f2d_scaled_kernel(int chained, long long n, const double* sc, const float* x, double* y)
 {
+    gm_chain(chained);
     const double a = sc[1];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
@@ -322,41 +330,42 @@ int gm_launch_cast_scaled_d2f(gm_ctx* c, long long n, const double* x, float* y,
 {
     int rc = gm_launch_dot(c, n, x, x, nullptr, nullptr, sc, s);
     if (rc) return rc;
-    gm_d2f_scaled_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y, sc);
+    gm_launch_chained(gm_d2f_scaled_kernel, gm_red_blocks(n), 256, 0, s, n, x, y, sc);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_axpy_scaled_f2d(gm_ctx* c, long long n, const double* sc, const float* x, double* y,
                               cudaStream_t s)
 {
-    gm_axpy_f2d_scaled_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, sc, x, y);
+    gm_launch_chained(gm_axpy_f2d_scaled_kernel, gm_red_blocks(n), 256, 0, s, n, sc, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 
 int gm_launch_copy_cast_d2f(gm_ctx* c, long long n, const double* x, float* y, cudaStream_t s)
 {
-    gm_d2f_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y);
+    gm_launch_chained(gm_d2f_kernel, gm_red_blocks(n), 256, 0, s, n, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_copy_cast_f2d(gm_ctx* c, long long n, const float* x, double* y, cudaStream_t s)
 {
-    gm_f2d_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, x, y);
+    gm_launch_chained(gm_f2d_kernel, gm_red_blocks(n), 256, 0, s, n, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 int gm_launch_axpy_f2d(gm_ctx* c, long long n, double a, const float* x, double* y, cudaStream_t s)
 {
-    gm_axpy_f2d_kernel<<<gm_red_blocks(n), 256, 0, s>>>(n, a, x, y);
+    gm_launch_chained(gm_axpy_f2d_kernel, gm_red_blocks(n), 256, 0, s, n, a, x, y);
     GM_LAUNCHED(c);
     return GM_OK;
 }
 
 __global__ void __launch_bounds__(256)
-gm_dot_kernel(long long n, const double* x, const double* y, const double* x2, const double* y2,
+gm_dot_kernel(int chained, long long n, const double* x, const double* y, const double* x2, const double* y2,
               double* out, RedCtx rc)
 {
+    gm_chain(chained);
     double v[2] = {0.0, 0.0};
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
@@ -372,7 +381,7 @@ gm_dot_kernel(long long n, const double* x, const double* y, const double* x2, c
 int gm_launch_dot(gm_ctx* c, long long n, const double* x, const double* y, const double* x2,
                   const double* y2, double* out, cudaStream_t s)
 {
-    gm_dot_kernel<<<gm_red_blocks(n), GM_RED_THREADS, 0, s>>>(n, x, y, x2, y2, out, redctx(c));
+    gm_launch_chained(gm_dot_kernel, gm_red_blocks(n), GM_RED_THREADS, 0, s, n, x, y, x2, y2, out, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;
 }
@@ -384,9 +393,10 @@ int gm_launch_dot(gm_ctx* c, long long n, const double* x, const double* y, cons
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
-gm_pcg_update_noz_kernel(long long n, T* x, T* r, const T* p, const T* q, PcgScalars* sc, int maxit,
+gm_pcg_update_noz_kernel(int chained, long long n, T* x, T* r, const T* p, const T* q, PcgScalars* sc, int maxit,
                          RedCtx rc)
 {
+    gm_chain(chained);
     if (sc->done) return;
     const T alpha = (T)sc->alpha;
     double v[1] = {0.0};
@@ -417,8 +427,9 @@ gm_pcg_update_noz_kernel(long long n, T* x, T* r, const T* p, const T* q, PcgSca
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-gm_pcg_rz_kernel(long long n, const T* r, const T* z, PcgScalars* sc, int init, RedCtx rc)
+gm_pcg_rz_kernel(int chained, long long n, const T* r, const T* z, PcgScalars* sc, int init, RedCtx rc)
 {
+    gm_chain(chained);
     if (sc->done) return;
     double v[1] = {0.0};
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -441,10 +452,10 @@ int gm_launch_pcg_update_noz(gm_ctx* c, int prec, void* x, void* r, const void* 
                              PcgScalars* sc, int maxit, cudaStream_t s)
 {
     if (prec == GM_F64)
-        gm_pcg_update_noz_kernel<double><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(
+        gm_launch_chained(gm_pcg_update_noz_kernel<double>, gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s,
             3 * c->N, (double*)x, (double*)r, (const double*)p, (const double*)q, sc, maxit, redctx(c));
     else
-        gm_pcg_update_noz_kernel<float><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(
+        gm_launch_chained(gm_pcg_update_noz_kernel<float>, gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s,
             3 * c->N, (float*)x, (float*)r, (const float*)p, (const float*)q, sc, maxit, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;
@@ -454,10 +465,10 @@ int gm_launch_pcg_rz(gm_ctx* c, int prec, const void* r, const void* z, PcgScala
                      cudaStream_t s)
 {
     if (prec == GM_F64)
-        gm_pcg_rz_kernel<double><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(3 * c->N, (const double*)r,
+        gm_launch_chained(gm_pcg_rz_kernel<double>, gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s, 3 * c->N, (const double*)r,
                                                                         (const double*)z, sc, init, redctx(c));
     else
-        gm_pcg_rz_kernel<float><<<gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s>>>(3 * c->N, (const float*)r,
+        gm_launch_chained(gm_pcg_rz_kernel<float>, gm_red_blocks(3 * c->N), GM_RED_THREADS, 0, s, 3 * c->N, (const float*)r,
                                                                        (const float*)z, sc, init, redctx(c));
     GM_LAUNCHED(c);
     return GM_OK;

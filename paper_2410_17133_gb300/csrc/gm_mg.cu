@@ -90,9 +90,10 @@ __device__ inline int mg_ext(const GridDesc& g, int o, int up) { return (g.kf >=
 // One thread per coarse component (blockIdx.y): 27 weighted loads each, and three
 // times the threads of one per node on the small levels (24^3 to 12^3, FP64: 15.3 -> 8.2 us).
 template <typename T>
-__global__ void mg_restrict_kernel(GridDesc F, GridDesc Cg, const T* bf, const T* yf, T* bc,
+__global__ void mg_restrict_kernel(int chained, GridDesc F, GridDesc Cg, const T* bf, const T* yf, T* bc,
                                    const uint8_t* maskc, const int* skip)
 {
+    gm_chain(chained);
     if (skip && *skip) return;
     const long long nc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (nc >= Cg.N) return;
@@ -132,9 +133,10 @@ __global__ void mg_restrict_kernel(GridDesc F, GridDesc Cg, const T* bf, const T
 // x_f += P x_c: trilinear interpolation inside each block; constrained fine
 // components unchanged.
 template <typename T>
-__global__ void mg_prolong_kernel(GridDesc F, GridDesc Cg, const T* xc, T* xf, const uint8_t* maskf,
+__global__ void mg_prolong_kernel(int chained, GridDesc F, GridDesc Cg, const T* xc, T* xf, const uint8_t* maskf,
                                   const int* skip)
 {
+    gm_chain(chained);
     if (skip && *skip) return;
     const long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= F.N) return;
@@ -208,10 +210,11 @@ __device__ inline T mg_ld(const MT* p)
     else return (T)*p;
 }
 template <typename T, typename MT>
-__global__ void __launch_bounds__(256) mg_cheb_kernel(long long N, const T* b, const T* y, T* x, T* d,
+__global__ void __launch_bounds__(256) mg_cheb_kernel(int chained, long long N, const T* b, const T* y, T* x, T* d,
                                                       const MT* mi, PairPrec<T> pp, const double* coef, int mode,
                                                       const int* skip, FaultK<T> fk)
 {
+    gm_chain(chained);
     if (skip && *skip) return;
     const T c1 = (T)coef[0], c2 = (T)coef[1];
     const bool xzero = (mode & CHEB_XZERO) != 0, dfx = (mode & CHEB_D_FROM_X) != 0, keepd = (mode & CHEB_NO_D) == 0;
@@ -476,7 +479,7 @@ int cheb_step(gm_ctx* c, const MGLevel& L, int k, int mode, bool fused, const in
     FaultK<T> fk = level_fault<T>(x);
     if (!fused) fk.D = nullptr;
     const bool xzero = (mode & CHEB_XZERO) != 0;
-    mg_cheb_kernel<T><<<mg_blocks(x->N), 256, 0, s>>>(x->N, v.b, xzero ? nullptr : v.y, v.x, v.d, level_inv<T>(x),
+    gm_launch_chained(mg_cheb_kernel<T, typename MinvType<T>::type>, mg_blocks(x->N), 256, 0, s, x->N, v.b, xzero ? nullptr : v.y, v.x, v.d, level_inv<T>(x),
                                                     level_pairs<T>(x), cf, mode, skip, fk);
     GM_LAUNCHED(c);
     return GM_OK;
@@ -545,17 +548,20 @@ int coarse_launch(gm_ctx* c, const MGLevel& L, int n, const int* skip, cudaStrea
                         mgc_magic((x->nx + 1) * x->g.nplanes), mgc_magic(x->nx + 1), mgc_magic(x->nx),
                         mgc_magic(x->nx * x->nz), skip};
     cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = n;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(n);
     cfg.blockDim = dim3(mgc_threads<T>());
     cfg.dynamicSmemBytes = mgc_layout<T, MT>(x->g, rows).total;
     cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, mg_coarse_kernel<T, MT, CLS>, a, x->R32, x->Rfx);
+    cfg.attrs = at;
+    const int chained = gm_capturing(s) ? 0 : 1;
+    cfg.numAttrs = 1 + chained;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, mg_coarse_kernel<T, MT, CLS>, chained, a, x->R32, x->Rfx);
     if (e != cudaSuccess) return c->set_err(GM_ECUDA, std::string("multigrid: coarsest level: ") + cudaGetErrorString(e));
     x->applies += L.deg - 1;
     GM_LAUNCHED(c);
@@ -581,11 +587,11 @@ int vcycle(gm_ctx* c, size_t l, const int* skip, cudaStream_t s)
     if ((rc = apply_kt(L.cx, v.x, v.y, skip, s))) return rc;
     const MGLevel& C = c->mg[l + 1];
     const LV<T> w = lv<T>(C);
-    mg_restrict_kernel<T><<<dim3((unsigned)((C.cx->N + 127) / 128), 3), 128, 0, s>>>(L.cx->g, C.cx->g, v.b, v.y, w.b,
+    gm_launch_chained(mg_restrict_kernel<T>, dim3((unsigned)((C.cx->N + 127) / 128), 3), 128, 0, s, L.cx->g, C.cx->g, v.b, v.y, w.b,
                                                                         C.cx->dmask.as<uint8_t>(), skip);
     GM_LAUNCHED(c);
     if ((rc = vcycle<T>(c, l + 1, skip, s))) return rc;
-    mg_prolong_kernel<T><<<(int)((L.cx->N + 255) / 256), 256, 0, s>>>(L.cx->g, C.cx->g, w.x, v.x,
+    gm_launch_chained(mg_prolong_kernel<T>, (int)((L.cx->N + 255) / 256), 256, 0, s, L.cx->g, C.cx->g, w.x, v.x,
                                                                        L.cx->dmask.as<uint8_t>(), skip);
     GM_LAUNCHED(c);
     return smooth<T>(c, L, L.deg, false, skip, s);
@@ -640,7 +646,7 @@ int estimate_lmax(gm_ctx* c, MGLevel& L)
         if ((rc = apply_kt(x, v, L.y, nullptr, 0))) return rc;
         FaultK<float> nofk = level_fault<float>(x);
         nofk.D = nullptr;
-        mg_cheb_kernel<float><<<GM_RED_BLOCKS, 256>>>(x->N, L.y, nullptr, L.x, L.d, level_inv<float>(x),
+        mg_cheb_kernel<float><<<GM_RED_BLOCKS, 256>>>(0, x->N, L.y, nullptr, L.x, L.d, level_inv<float>(x),
                                                       level_pairs<float>(x), unit, CHEB_XZERO | CHEB_NO_D, nullptr,
                                                       nofk);
         GM_LAUNCHED(c);

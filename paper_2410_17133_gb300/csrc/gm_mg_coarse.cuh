@@ -99,9 +99,10 @@ __host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows)
 
 template <typename T, typename MT, int CLS>
 __global__ void __launch_bounds__(mgc_threads<T>(), 1)
-mg_coarse_kernel(const __grid_constant__ CoarseArgs<T, MT> a, const __grid_constant__ RefOps<float> R,
+mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const __grid_constant__ RefOps<float> R,
                  const __grid_constant__ RefFx F)
 {
+    gm_chain(chained);
     constexpr bool FX = sizeof(T) == 8;
     constexpr int NL = mgc_limbs<T>(), NT = mgc_threads<T>();
     using W = typename std::conditional<FX, int, float>::type;      // word of a staged value

@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/gm_tet.h"
+#include "gm_launch.cuh"
 
 namespace {
 
@@ -413,7 +414,7 @@ void launch(gm_tet* t, const TetCoef<T>& c, const T* xu, const T* xp, T* yu, T* 
 {
     const int N = (int)t->N;
     if (t->csr_ready) {
-        tcsr_apply<T, MODE, false><<<(unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s>>>(
+        gm_launch_chained(tcsr_apply<T, MODE, false>, (unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s,
             N, csr<T>(t), c.cApu, c.cC, xu, xp, yu, yp, skip, TetDir<T>{});
         return;
     }
@@ -429,7 +430,7 @@ bool apply_k_dir(gm_tet* t, const TetDir<T>& d, T* q, cudaStream_t s)
 {
     if (!t->csr_ready) return false;
     const int N = (int)t->N;
-    tcsr_apply<T, TM_K, true><<<(unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s>>>(
+    gm_launch_chained(tcsr_apply<T, TM_K, true>, (unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s,
         N, csr<T>(t), T(1), T(0), nullptr, nullptr, q, nullptr, &d.st->done, d);
     return true;
 }

@@ -11,7 +11,7 @@
 // half of them idle on 15 entries and the FP64 adds of the shuffle tree cost
 // as much as the products, with 1 the small meshes leave most SMs without work.
 // Measured (36 k nodes, 197 k tetrahedra, FP64; K, A_pu, A_up, A22 and J in
-// turn): 652 us walking the elements, 103 us by rows.  What bounds it: the FP64
+// turn): 652 us walking the elements, 94 us by rows.  What bounds it: the FP64
 // pipe (K: 12 instructions per entry and 9 for the lanes' sums), then the rows'
 // 140 B per entry from L2.
 //
@@ -130,9 +130,10 @@ struct TetCsr {
 // entries of y are set to 0, p.q is summed over the grid and the last block
 // forms alpha.
 template <typename T, int MODE, bool PCG>
-__global__ void __launch_bounds__(TPCG_NT) tcsr_apply(int N, const TetCsr<T> A, T cApu, T cC, const T* xu, const T* xp,
+__global__ void __launch_bounds__(TPCG_NT) tcsr_apply(int chained, int N, const TetCsr<T> A, T cApu, T cC, const T* xu, const T* xp,
                                                       T* yu, T* yp, const int* skip, const TetDir<T> dir)
 {
+    gm_chain(chained);
     if (skip != nullptr && *skip != 0) return;
     constexpr bool IN_U = (MODE & (TM_K | TM_AUP)) != 0;
     constexpr bool IN_P = (MODE & (TM_APU | TM_S | TM_C)) != 0;

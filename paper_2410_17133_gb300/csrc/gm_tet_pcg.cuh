@@ -111,9 +111,10 @@ __device__ inline bool tpcg_reduce2(double a, double b, double* part, unsigned* 
 
 // r = b (cast to T), x = 0; state reset
 template <typename T>
-__global__ void __launch_bounds__(TPCG_NT) tpcg_start(long long n, const double* b, T* r, T* x, TetPcgState* st,
+__global__ void __launch_bounds__(TPCG_NT) tpcg_start(int chained, long long n, const double* b, T* r, T* x, TetPcgState* st,
                                                       double tol2, int maxit)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         r[i] = (T)b[i];
         x[i] = T(0);
@@ -144,9 +145,10 @@ __device__ inline void tpcg_prec_pair(const TetPrecT<T>& M, int i, const T (&r6)
 // x += alpha p, r -= alpha q, z = M^-1 r, then r.z and r.r; the last block
 // sets beta = (r.z)_new / (r.z)_old and the stopping state.
 template <typename T, bool START>
-__global__ void __launch_bounds__(TPCG_NT) tpcg_step(TetPrecT<T> M, T* x, T* r, T* z, const T* p, const T* q,
+__global__ void __launch_bounds__(TPCG_NT) tpcg_step(int chained, TetPrecT<T> M, T* x, T* r, T* z, const T* p, const T* q,
                                                      TetPcgState* st, double* part)
 {
+    gm_chain(chained);
     if (!START && st->done) return;
     const int N = M.N;
     const T al = START ? T(0) : (T)st->alpha;
@@ -224,9 +226,10 @@ __global__ void __launch_bounds__(TPCG_NT) tpcg_step(TetPrecT<T> M, T* x, T* r, 
 
 // constrained entries of q set to 0, then p.q; the last block sets alpha
 template <typename T>
-__global__ void __launch_bounds__(TPCG_NT) tpcg_pq(int N, const uint8_t* mask, const T* p, T* q, TetPcgState* st,
+__global__ void __launch_bounds__(TPCG_NT) tpcg_pq(int chained, int N, const uint8_t* mask, const T* p, T* q, TetPcgState* st,
                                                    double* part)
 {
+    gm_chain(chained);
     if (st->done) return;
     double acc = 0.0;
     for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
@@ -251,8 +254,9 @@ __global__ void __launch_bounds__(TPCG_NT) tpcg_pq(int N, const uint8_t* mask, c
 
 // p = z + beta p (START: p = z)
 template <typename T, bool START>
-__global__ void __launch_bounds__(TPCG_NT) tpcg_dir(long long n, const T* z, T* p, const TetPcgState* st)
+__global__ void __launch_bounds__(TPCG_NT) tpcg_dir(int chained, long long n, const T* z, T* p, const TetPcgState* st)
 {
+    gm_chain(chained);
     if (st->done) return;
     const T b = START ? T(0) : (T)st->beta;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -260,8 +264,9 @@ __global__ void __launch_bounds__(TPCG_NT) tpcg_dir(long long n, const T* z, T* 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(TPCG_NT) tpcg_out(long long n, const T* x, double* y)
+__global__ void __launch_bounds__(TPCG_NT) tpcg_out(int chained, long long n, const T* x, double* y)
 {
+    gm_chain(chained);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = (double)x[i];
 }
@@ -364,13 +369,13 @@ struct TetPcg {
                 // between two buffers (GRAPH_ITS is even)
                 T* pn = i & 1 ? p : p2;
                 step_by_rows(TetDir<T>{z, i & 1 ? p2 : p, pn, mask, st, part}, q, cs);
-                tpcg_step<T, false><<<tpcg_blocks(N), TPCG_NT, 0, cs>>>(M, x, r, z, pn, q, st, part);
+                gm_launch_chained(tpcg_step<T, false>, tpcg_blocks(N), TPCG_NT, 0, cs, M, x, r, z, pn, q, st, part);
                 continue;
             }
             op(p, q, &st->done, cs);
-            tpcg_pq<T><<<tpcg_blocks(N), TPCG_NT, 0, cs>>>(N, mask, p, q, st, part);
-            tpcg_step<T, false><<<tpcg_blocks(N), TPCG_NT, 0, cs>>>(M, x, r, z, p, q, st, part);
-            tpcg_dir<T, false><<<tpcg_blocks(n), TPCG_NT, 0, cs>>>(n, z, p, st);
+            gm_launch_chained(tpcg_pq<T>, tpcg_blocks(N), TPCG_NT, 0, cs, N, mask, p, q, st, part);
+            gm_launch_chained(tpcg_step<T, false>, tpcg_blocks(N), TPCG_NT, 0, cs, M, x, r, z, p, q, st, part);
+            gm_launch_chained(tpcg_dir<T, false>, tpcg_blocks(n), TPCG_NT, 0, cs, n, z, p, st);
         }
     }
 
@@ -402,9 +407,9 @@ struct TetPcg {
                 return -1;
             }
         }
-        tpcg_start<T><<<tpcg_blocks(n), TPCG_NT, 0, s>>>(n, b, r, x, st, rtol * rtol, maxit);
-        tpcg_step<T, true><<<tpcg_blocks(N), TPCG_NT, 0, s>>>(M, x, r, z, p, q, st, part);
-        tpcg_dir<T, true><<<tpcg_blocks(n), TPCG_NT, 0, s>>>(n, z, p, st);
+        gm_launch_chained(tpcg_start<T>, tpcg_blocks(n), TPCG_NT, 0, s, n, b, r, x, st, rtol * rtol, maxit);
+        gm_launch_chained(tpcg_step<T, true>, tpcg_blocks(N), TPCG_NT, 0, s, M, x, r, z, p, q, st, part);
+        gm_launch_chained(tpcg_dir<T, true>, tpcg_blocks(n), TPCG_NT, 0, s, n, z, p, st);
         int reps = 1;
         int hs[2] = {0, 0};
         for (;;) {
@@ -422,7 +427,7 @@ struct TetPcg {
         }
         *its += hs[1];
         if (hs[0] == 2 || hs[0] == 3) return hs[0];
-        tpcg_out<T><<<tpcg_blocks(n), TPCG_NT, 0, s>>>(n, x, x_out);
+        gm_launch_chained(tpcg_out<T>, tpcg_blocks(n), TPCG_NT, 0, s, n, x, x_out);
         return 0;
     }
 };
