@@ -516,6 +516,9 @@ int coarse_cluster(gm_ctx* x)
 {
     using MT = typename MinvType<T>::type;
     if (x->g.kf >= 0 && !x->pair_prec) return 0;
+    // FP64: the moduli's limbs are exact up to a contrast of 2^21; beyond it the
+    // level keeps its launches, whose FP64 tiles hold any contrast
+    if (sizeof(T) == 8 && x->Rfx.gradeK < GM_FX_GRADE - 21) return 0;
     const int n = mgc_setup<T, MT, CLS>(x->device);
     if (n == 0) return 0;
     const int rows = (x->ny + n) / n;            // ceil((ny + 1) / n)
