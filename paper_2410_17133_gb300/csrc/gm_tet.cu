@@ -151,6 +151,7 @@ struct DBuf {
 }  // namespace
 
 #include "gm_tet_pcg.cuh"
+#include "gm_tet_pcg_grid.cuh"
 #include "gm_tet_csr.cuh"
 
 // Largest node, tetrahedron or fault-triangle count: all device index arithmetic
@@ -169,6 +170,9 @@ struct gm_tet {
     // assembled rows (gm_tet_csr.cuh); false where they do not fit the device
     bool csr_ready = false;
     long long nnz = 0;
+    int grid_rows = 0, grid_ctas = 0;       // one-launch PCG (gm_tet_pcg_grid.cuh): rows per CTA, 0: not used
+    size_t grid_smem = 0;
+    DBuf grid_box;
     DBuf crow, ccol, cK64, cA64, cSC64, cK32, cA32, cSC32;
     // time stepping
     std::vector<double> hG, hV;            // element gradients and volumes (host copy)
@@ -255,6 +259,7 @@ void tet_assemble(gm_tet* t)
             t->cSC64.alloc(nnz * 16) != cudaSuccess || t->cK32.alloc(nnz * 36) != cudaSuccess ||
             t->cA32.alloc(nnz * 24) != cudaSuccess || t->cSC32.alloc(nnz * 8) != cudaSuccess)
             return give_up();
+        t->grid_rows = tgrid_plan(t->device, N, h, t->grid_smem, t->grid_ctas);
         t->nnz = nnz;
     }
     const long long nnz = t->nnz;
@@ -573,6 +578,21 @@ struct Stepper {
     // x = K^-1 b (x from 0), PCG with 3x3 nodal block Jacobi to ||r|| <= rtol ||b||,
     // device-resident (scratch 0-3, 14 and 15)
     int solve_k(const double* b, double* x, double rtol, int maxit, long long* its) {
+        const int rc = t->csr_ready && t->grid_rows ? solve_k_grid(b, x, rtol, maxit, its) : solve_k_loop(b, x, rtol, maxit, its);
+        if (rc == 2) return t->set_err(GM_ENAN, "tet step: K not positive on a direction");
+        if (rc == 3) return t->set_err(GM_ENOCONV, "tet step: K solve did not converge");
+        if (rc == 5) return t->set_err(GM_ECUDA, "tet step: the solve's blocks waited for one another too long");
+        if (rc < 0) return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(cudaGetLastError()));
+        return GM_OK;
+    }
+    int solve_k_grid(const double* b, double* x, double rtol, int maxit, long long* its) {
+        return tgrid_solve(TetGridArgs{N, t->grid_rows, maxit, rtol * rtol, t->crow.as<int>(), t->ccol.as<int>(),
+                                       t->cK64.as<double>(), t->Kinv.as<double>(), t->mask.as<uint8_t>(), b, x,
+                                       t->w[2].as<double>(), t->grid_box.as<ulonglong2>(),
+                                       t->pcg_st.as<TetPcgState>()},
+                           t->grid_ctas, t->grid_smem, s, its);
+    }
+    int solve_k_loop(const double* b, double* x, double rtol, int maxit, long long* its) {
         TetPcg<double> e{N, s, t->w[14].as<double>(), t->w[0].as<double>(), t->w[1].as<double>(),
                          t->w[2].as<double>(), t->w[3].as<double>(), t->pcg_st.as<TetPcgState>(),
                          t->pcg_part.as<double>(),
@@ -582,16 +602,12 @@ struct Stepper {
             e.p2 = t->w[15].as<double>();
             e.step_by_rows = [t = t](const TetDir<double>& d, double* q, cudaStream_t cs) { apply_k_dir<double>(t, d, q, cs); };
         }
-        const int rc = e.solve(
+        return e.solve(
             b, x, rtol, maxit, its,
             [&](const double* p, double* q, const int* skip, cudaStream_t cs) {
                 apply_t<double>(t, GM_OP_KB, p, q, 0.0, cs, skip);
             },
             t->use_graphs ? &t->pcg_graph[0] : nullptr, &t->cap_stream);
-        if (rc == 2) return t->set_err(GM_ENAN, "tet step: K not positive on a direction");
-        if (rc == 3) return t->set_err(GM_ENOCONV, "tet step: K solve did not converge");
-        if (rc < 0) return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(cudaGetLastError()));
-        return GM_OK;
     }
 };
 
@@ -646,6 +662,7 @@ int tet_prepare(gm_tet* t)
     if ((ce = t->Kinv.put(Kinv.data(), Kinv.size() * 8)) != cudaSuccess || (ce = t->Sd.put(Sd.data(), N * 8)) != cudaSuccess ||
         (ce = t->Cd.put(Cd.data(), N * 8)) != cudaSuccess || (ce = t->mask.put(mk.data(), N)) != cudaSuccess ||
         (ce = t->dfu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (ce = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
+        (t->grid_rows && (ce = t->grid_box.alloc(tgrid_box_bytes(t->grid_ctas))) != cudaSuccess) ||
         (ce = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
         (ce = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
         return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(ce));
