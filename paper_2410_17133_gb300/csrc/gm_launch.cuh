@@ -9,10 +9,11 @@
 // before it touches global memory, in every thread and on every path, so
 // completion is transitive along the chain: a kernel cannot complete before its
 // predecessors have.  Kernels in between that are launched normally wait for
-// completion as usual.  In a captured graph the programmatic edges measured
-// slower than plain ones, so there the launches are plain and gm_chain returns
-// at once.  A time step at 32^3 with its gradient: 55 -> 45 ms together with the
-// coarsest level's shared-memory items; FP32 step at 64^3 84 -> 75 ms.
+// completion as usual.  Measured, chained against plain launches: outside graphs
+// J on 8^3 cells 46.8 -> 43 us, five tetrahedral products 103 -> 94.5 us, the
+// FP32 products at 160^3 551 -> 533 us; in captured graphs it loses (FP32 step at
+// 64^3 84 -> 89 ms, FP64 K_T solve at 48^3 60.5 -> 66.8 ms), so there the launches
+// are plain and gm_chain returns at once.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -4,8 +4,8 @@
 // On these meshes an iteration is bound by latency: as two launches (product
 // with direction and alpha, then the vector step) it took 18.8 us on 4.9 k nodes,
 // of which the FP64 pipes worked about 4; this way it takes 13 (a time step of
-// 30 such solves: 98 -> 68 ms), half of it in the two sums.  Here a CTA owns a range of nodes for
-// the whole solve.  Its rows of K, the direction at each of its entries (so p is
+// 30 such solves: 98 -> 68 ms), more than half of it in the two sums.  Here a CTA
+// owns a range of nodes for the whole solve.  Its rows of K, the direction at each of its entries (so p is
 // never exchanged), its preconditioner blocks and vectors stay in shared memory
 // and registers; only z travels, once per iteration.  The two sums of an
 // iteration double as the grid's barriers: each CTA sends its partials to every
