@@ -347,7 +347,9 @@ def run_gm(args, rank, world, local_rank):
     apply["J_fp64_GBs_80B_per_node"] = 80.0 * N / t_app[("J", "fp64")] / 1e9
     apply["KB_fp64_alu_frac_nominal"] = flops / t_app[("KB", "fp64")] / 1e12 / FP64_PEAK_TFLOPS
     apply["notes"] = ("KB: bulk kernel alone (one launch); KT adds the fault kernel; J: the coupled "
-                      "Jacobian (4 DoF per node; FP32 and FP64 run the generic coupled bulk kernel); "
+                      "Jacobian (4 DoF per node; FP32 runs the generic coupled bulk kernel, FP64 one launch per block); "
+                      "FP64 products run in fixed point on the integer pipes, so their fraction of the FP64 "
+                      "peak counts the operator's FP64 operations and may exceed 1; "
                       "GDoF/s = field DoF of the product / launch time")
     peaks = {}
     if os.path.exists(PEAKS_FILE):
