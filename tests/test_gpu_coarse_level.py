@@ -52,3 +52,24 @@ def test_solves_converge_as_multigrid_does(nx, ny, nz, cell, fault, precision):
             ref = st if kind == 1 else ref
             assert np.linalg.norm(st["u"] - ref["u"]) <= 1e-6 * np.linalg.norm(ref["u"])
     assert 3 * its[1] <= its[0], its
+
+
+@pytest.mark.parametrize("bits", [12, 21, 23, 40])
+def test_modulus_contrast_on_both_sides_of_the_rule(bits):
+    """Soft lower half, 2^bits below the upper one: the FP64 cluster kernel serves a contrast
+    up to 2^21, the launches the rest.  The residual bound is that of the solves above."""
+    need_gpu()
+    nx, ny, nz = 8, 20, 16
+    prob = W.tiny_faulted(nx, ny, nz, seed=11, h=(0.5, 0.5, 0.5))
+    prob.kf = prob.fault = None
+    prob.fixed = np.zeros((4, prob.n_nodes), np.uint8)
+    prob.fixed[0:3, : (nx + 1) * (ny + 1)] = 1
+    prob.fu, prob.fp = np.zeros((3, prob.n_nodes)), np.zeros(prob.n_nodes)
+    prob.E = np.full_like(prob.E, 2.0 ** 34)
+    prob.E[: prob.E.size // 2] *= 2.0 ** -bits
+    u = np.random.default_rng(3).normal(size=(3, prob.n_nodes)) * 1e-6 * (prob.fixed[:3] == 0)
+    s = solver_for(prob)
+    s.set_preconditioner(1)
+    b = s.apply("KT", cuda(u))
+    x, rep = s.pcg("KT", b, rtol=1e-12)
+    assert torch.linalg.norm(b - s.apply("KT", x)) <= 1e-11 * torch.linalg.norm(b), rep
