@@ -516,6 +516,8 @@ int coarse_cluster(gm_ctx* x)
 {
     using MT = typename MinvType<T>::type;
     if (x->g.kf >= 0 && !x->pair_prec) return 0;
+    // one cell in x (GM_MG_MIN_CELLS=1): mgc_div has no multiplier for the divisor 1
+    if (x->nx < 2) return 0;
     // FP64: the moduli's limbs are exact up to a contrast of 2^21; beyond it the
     // level keeps its launches, whose FP64 tiles hold any contrast
     if (sizeof(T) == 8 && x->Rfx.gradeK < GM_FX_GRADE - 21) return 0;

@@ -47,9 +47,10 @@ struct CoarseArgs {
     const int* skip;
 };
 
-// x / d for x < 2^16, d < 2^16 with m = ceil(2^32 / d): exact, since x (m d - 2^32) < 2^32
+// x / d for x < 2^16, 2 <= d < 2^16 with m = ceil(2^32 / d): exact, since x (m d - 2^32) < 2^32
+// (d = 1 would need 33 bits; every divisor is at least nx, so levels of one cell in x keep their launches)
 __device__ inline int mgc_div(int x, unsigned m) { return (int)__umulhi((unsigned)x, m); }
-inline unsigned mgc_magic(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ull + d - 1) / d); }
+inline unsigned mgc_magic(unsigned d) { return (unsigned)((0x100000000ull + d - 1) / d); }
 
 // first node row of CTA r of n: the first CTAs take one row more, so that
 // neighbouring rows are in neighbouring CTAs also where some have none
