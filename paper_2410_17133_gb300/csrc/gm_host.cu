@@ -1122,8 +1122,7 @@ int bind_impl(gm_ctx* c)
     }
     c->bound = true;   // loads upload below needs the grid
     int rc = gm_prepare_bulk32(c);
-    if (rc) return rc;
-    rc = gm_prepare_fx(c);
+    if (!rc) rc = gm_prepare_fx(c);
     if (rc) { c->bound = false; return rc; }
     rc = upload_loads(c);
     if (rc) { c->bound = false; return rc; }
