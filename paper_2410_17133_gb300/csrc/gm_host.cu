@@ -274,16 +274,18 @@ int bind_impl(gm_ctx* c);
 static void note_kap_range(gm_ctx* c, const std::vector<double>& kap)
 {
     double lo = 0.0, hi = 0.0;
-    c->kap_zero = false;
+    bool zero = false;
     for (double k : kap) {
         hi = std::max(hi, k);
-        if (!(k > 0.0)) c->kap_zero = true;
+        if (!(k > 0.0)) zero = true;
         if (k > 0.0 && (lo == 0.0 || k < lo)) lo = k;
     }
-    // captured A22 iterations hold the scale that follows from the range
-    if (lo != c->kap_lo || hi != c->kap_hi) c->drop_graphs();
+    // captured A22 iterations hold the scale, and the choice of kernel, that
+    // follow from the range and from elements without flow
+    if (lo != c->kap_lo || hi != c->kap_hi || zero != c->kap_zero) c->drop_graphs();
     c->kap_lo = lo;
     c->kap_hi = hi;
+    c->kap_zero = zero;
 }
 
 // Flow block S cS / M + cC C in fixed point (cS as given to the launchers).

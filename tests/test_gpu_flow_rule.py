@@ -1,0 +1,44 @@
+"""Which kernel a flow product takes follows the permeabilities of the moment."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+from gpu_common import cuda, need_gpu, solver_for
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(k=None):
+    prob = W.tiny_faulted(16, 14, 9, seed=3, h=(0.4, 0.3, 0.5))
+    prob.kf = prob.fault = None
+    N = prob.n_nodes
+    prob.fixed = np.zeros((4, N), np.uint8)
+    prob.fixed[3, -2:] = 1
+    prob.fu, prob.fp = np.zeros((3, N)), np.zeros(N)
+    if k is not None:
+        prob.k = k
+    return prob
+
+
+@pytest.mark.parametrize("dt", [3.0, 1e10])
+def test_solves_follow_elements_that_lose_or_gain_flow(dt):
+    """Same smallest positive and largest k before and after: a solver that was given the new
+    array later returns what a fresh one does, bit for bit."""
+    need_gpu()
+    prob = problem()
+    rng = np.random.default_rng(4)
+    full = 10.0 ** rng.uniform(-15.0, -14.0, prob.n_el)
+    holes = full.copy()
+    inner = rng.permutation(prob.n_el)[:20]
+    holes[[e for e in inner if full[e] not in (full.min(), full.max())]] = 0.0
+    b = cuda(rng.normal(size=prob.n_nodes) * 1e-12 * (prob.fixed[3] == 0))
+    s = solver_for(problem(full))
+    s.timestep(dt)
+    for k in (full, holes, full):
+        s.set_permeability(k)
+        x, _ = s.pcg("A22", b, rtol=1e-8)
+        f = solver_for(problem(k))
+        f.timestep(dt)
+        y, _ = f.pcg("A22", b, rtol=1e-8)
+        assert bool((x == y).all())
