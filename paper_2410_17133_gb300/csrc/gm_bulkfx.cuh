@@ -276,7 +276,8 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
                 gm_fx_mac4(sum, r, E[2], E[1], E[0]);
             }
             const int* m = Q.m[s];
-            gm_fx_mac4(sum, xv[s], m[2], m[1], m[0]);
+            gm_fx_mac4(sum, xv[s], m[3], m[2], m[1]);
+            sum.am += (int64_t)xv[s][2] * m[0];
             gm_fx_carry4_signed(sum, y);
         } else {
 #pragma unroll

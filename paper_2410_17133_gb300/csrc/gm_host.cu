@@ -124,15 +124,16 @@ bool ref_cell(const double h[3], const double sh[2], double nu, double K[24][24]
 
 inline double hsgn(int s, int a) { return (gm_popc3(s & a) & 1) ? -1.0 : 1.0; }
 
-// signed limbs of v 2^-e (|v| < 2^e), v = hi + lo, to 78 bits
-void fx_limbs(double hi, double lo, int e, int (&l)[3])
+// signed limbs of v 2^-e (|v| < 2^e), v = hi + lo, to 26 NL bits
+template <int NL>
+void fx_limbs(double hi, double lo, int e, int (&l)[NL])
 {
-    __int128 n = (__int128)std::nearbyint(std::ldexp(hi, 78 - e)) + (__int128)std::nearbyint(std::ldexp(lo, 78 - e));
+    constexpr int B = NL * GM_FX_RADIX;
+    __int128 n = (__int128)std::nearbyint(std::ldexp(hi, B - e)) + (__int128)std::nearbyint(std::ldexp(lo, B - e));
     const int sg = n < 0 ? -1 : 1;
     if (n < 0) n = -n;
-    l[0] = sg * (int)(n & GM_FX_MASK);
-    l[1] = sg * (int)((n >> GM_FX_RADIX) & GM_FX_MASK);
-    l[2] = sg * (int)(n >> (2 * GM_FX_RADIX));
+    for (int i = 0; i < NL - 1; ++i, n >>= GM_FX_RADIX) l[i] = sg * (int)(n & GM_FX_MASK);
+    l[NL - 1] = sg * (int)n;
 }
 
 // Fixed-point copy of the reference operators: scaled by the power of two that
@@ -319,8 +320,12 @@ FlowFx gm_flow_fx(const gm_ctx* c, double cS, double cC)
         fx_limbs(v, std::fma(f, c->R64.M[i], -v), Q.eU, Q.m[i]);
     }
     // the fourth limb of the results covers coefficients 2^24 apart; the inputs'
-    // own grading is judged by the kernel as for the other blocks
-    Q.grade = std::ilogb(hi) - std::ilogb(lo) <= 24 ? GM_FX_GRADE - 2 : -1;
+    // own grading is judged by the kernel as for the other blocks.  A pressure that
+    // is uniform over an element meets its storage alone, however strong the flow:
+    // the storage entries have four limbs, and a product with them keeps 2^-98 of
+    // the scale, more than FP64's rounding of a storage up to 2^40 below it
+    const bool small_storage = storage > 0.0 && Q.eU - std::ilogb(storage) > 40;
+    Q.grade = std::ilogb(hi) - std::ilogb(lo) <= 24 && !small_storage ? GM_FX_GRADE - 2 : -1;
     return Q;
 }
 

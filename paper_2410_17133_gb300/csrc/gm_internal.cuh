@@ -175,13 +175,13 @@ struct RefFx {
 };
 
 // The flow block of one launch in the same form: Darcy entries (row sums at most
-// 1), storage per mode, and the scale 2^eU that bounds both (a quarter each, so
-// that 36 results of their sum meet in a node); topW is the biased exponent of
+// 1), storage per mode in four limbs, and the scale 2^eU that bounds both (a quarter
+// each, so that 36 results of their sum meet in a node); topW is the biased exponent of
 // the largest dt k/mu that the scale admits.  grade < 0: coefficients too far
 // apart for the fixed-point unit, use FP64.
 struct FlowFx {
     int l[GM_PP_MAXL][3];
-    int m[8][3];
+    int m[8][4];
     int topW, eU, grade;
 };
 
