@@ -60,7 +60,7 @@ __device__ __forceinline__ void gm_fx_k_mode(const RefFx& F, const int (&xv)[24]
     for (int j = 0; j < 24; ++j)
         if (PP.k[c * 8 + s][j] >= 0 && (j & 7) != 0) {
             const int* k = F.k[PP.k[c * 8 + s][j]];
-            gm_fx_mac2(acc, xv[j], k[1], k[0]);
+            gm_fx_mac3(acc, xv[j], k[2], k[1], k[0]);
         }
     int r[3];
     gm_fx_carry(acc, r);

@@ -12,7 +12,8 @@
 //   - 8-point transforms and sums of up to 28 (signed limbs: 36) results fit the words;
 //   - coefficients: |c| < 1 as c2 2^-26 + c1 2^-52 + c0 2^-78, exact for the
 //     53 bits of a double within 2^25 of the largest (moduli: within 2^21; the
-//     entries of K_b as two limbs, to 2^-57 of a row's sum);
+//     entries of K_b to 2^-83 of the largest row sum, so that those of flat cells,
+//     a^2 apart at an aspect ratio a, keep their bits);
 //   - a product sum loses at most about 2^3 units of the last place (the limb
 //     pairs below it), a node of the operators about 2^6, so results are exact
 //     to 2^-69 of the tile's largest term, 16 bits below FP64's rounding.
@@ -107,10 +108,9 @@ __host__ __device__ inline void gm_fx_mac(FxAcc& s, const int (&x)[3], int c2, i
     s.a0 += (int64_t)x[1] * c1;
     s.a0 += (int64_t)x[2] * c0;
 }
-// The same with a coefficient of two limbs, c2 2^-30 + c1 2^-56 (|c2| <= 2^30):
-// five multiplications instead of six.  Sums and carried limbs then weigh 2^4
-// less: (2^48, 2^22, 2^-4); multiplied by a coefficient whose top limb has 22 bits
-// (gm_fx_coef22) they are back at (2^52, 2^26, 1).
+// The same with a coefficient c2 2^-30 + c1 2^-56 (|c2| <= 2^30).  Sums and
+// carried limbs then weigh 2^4 less: (2^48, 2^22, 2^-4); multiplied by a coefficient
+// whose top limb has 22 bits (gm_fx_coef22) they are back at (2^52, 2^26, 1).
 __host__ __device__ inline void gm_fx_mac2(FxAcc& s, const int (&x)[3], int c2, int c1)
 {
     s.a2 += (int64_t)x[2] * c2;
@@ -118,6 +118,13 @@ __host__ __device__ inline void gm_fx_mac2(FxAcc& s, const int (&x)[3], int c2, 
     s.a1 += (int64_t)x[2] * c1;
     s.a0 += (int64_t)x[0] * c2;
     s.a0 += (int64_t)x[1] * c1;
+}
+// and with a third limb c0 2^-82 below (|c1|, |c0| <= 2^25): a product loses 2^-1
+// units, the carried sum 2^-3
+__host__ __device__ inline void gm_fx_mac3(FxAcc& s, const int (&x)[3], int c2, int c1, int c0)
+{
+    gm_fx_mac2(s, x, c2, c1);
+    s.a0 += (int64_t)x[2] * c0;
 }
 
 // carried limbs: l0, l1 in [0, 2^26), l2 signed

@@ -163,11 +163,14 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
     for (int i = 0; i < 24; ++i) {
         for (int j = 0; j < 24; ++j)
             if (PP.k[i][j] >= 0) {
-                // c2 2^-30 + c1 2^-56, c1 in [-2^25, 2^25]
-                const int64_t n = (int64_t)std::nearbyint(std::ldexp(Kt[i][j], 56 - F.eK));
-                const int64_t hi = (n + (1ll << 25)) >> 26;
-                F.k[PP.k[i][j]][1] = (int)hi;
-                F.k[PP.k[i][j]][0] = (int)(n - hi * (1ll << 26));
+                // c2 2^-30 + c1 2^-56 + c0 2^-82, c1 and c0 in [-2^25, 2^25)
+                __int128 n = (__int128)std::nearbyint(std::ldexp(Kt[i][j], 82 - F.eK));
+                int(&k)[3] = F.k[PP.k[i][j]];
+                for (int l = 0; l < 2; ++l) {
+                    k[l] = (int)(((int64_t)n + (1 << 25)) & GM_FX_MASK) - (1 << 25);
+                    n = (n - k[l]) >> GM_FX_RADIX;
+                }
+                k[2] = (int)n;
             }
         for (int j = 0; j < 8; ++j)
             if (PP.a[i][j] >= 0) {
@@ -175,11 +178,23 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
                 fx_limbs(hi, std::fma(alpha, At[i][j], -hi), F.eA, F.a[PP.a[i][j]]);
             }
     }
-    // moduli: limbs are exact while the smallest is within 2^21 of the largest;
-    // what a low modulus loses against the tile's unit comes off the grading
+    // Grading: what lies below the unit in the coefficients comes off it.  An output
+    // mode is off by about one unit of 2^(eK - 75), where FP64 rounds 2^-54 of a term
+    // K_jj x_j: exact enough while 20 bits less the distance of the smallest K_jj
+    // from 2^eK (5 for a cube, 16 for a cell of 100:100:1) cover the grading.  Moduli
+    // likewise (their limbs are exact within 2^21 of the largest).  A_pu: the forces
+    // that a uniform pressure exerts, field by field.
+    double kd = 0.0, ad = 0.0;
+    for (int i = 0; i < 24; ++i)
+        if ((i & 7) != 0 && (kd == 0.0 || Kt[i][i] < kd)) kd = Kt[i][i];
+    for (int c = 0; c < 3; ++c) {
+        double m = 0.0;
+        for (int s = 0; s < 8; ++s) m = std::max(m, std::fabs(alpha * At[c * 8 + s][0]));
+        if (m > 0.0 && (ad == 0.0 || m < ad)) ad = m;
+    }
     F.topE = std::ilogb(Emax) + 1023;
-    F.gradeK = GM_FX_GRADE - (std::ilogb(Emax) - std::ilogb(Emin));
-    F.gradeA = GM_FX_GRADE;
+    F.gradeK = kd > 0.0 ? std::min(GM_FX_GRADE, 20 - (F.eK - std::ilogb(kd))) - (std::ilogb(Emax) - std::ilogb(Emin)) : -1;
+    F.gradeA = ad > 0.0 ? std::min(GM_FX_GRADE, 21 - (F.eA - std::ilogb(ad))) : GM_FX_GRADE;
 }
 
 // Parity transform and packing of the entries the class's pattern allows;

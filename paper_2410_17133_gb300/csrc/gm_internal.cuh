@@ -161,15 +161,15 @@ struct RefPairs32 {
     float2 L[GM_PP_MAXL];
 };
 
-// The pattern entries of K_b as two limbs (26 bits below 30) and of alpha A as three
-// signed 26-bit limbs (gm_fixed.cuh, least significant first): entry = (limbs as a
+// The pattern entries of K_b (limbs of 26, 26 and 30 bits) and of alpha A (three
+// signed 26-bit limbs; gm_fixed.cuh, least significant first): entry = (limbs as a
 // fraction) 2^eK or 2^eA, scaled so
 // that the absolute sum of a row is at most 1 (K) or 1/2 (A: 36 results meet in
 // a node).  topE is the biased exponent of the largest Young's modulus; gradeK,
 // gradeA the grading of an input inside a tile, in bits, up to which the
 // fixed-point error stays below the rounding of FP64.
 struct RefFx {
-    int k[GM_PP_MAXK][2];
+    int k[GM_PP_MAXK][3];
     int a[GM_PP_MAXA][3];
     int eK, eA, topE, gradeK, gradeA;
 };
