@@ -3,19 +3,29 @@
 //
 // Why: the FP64 kernel is bound by the FP64 pipe (2 lanes per clock and SM).
 // In the parity basis a K_b element takes about 210 FP64 instructions, 64
-// issue slots each; the same element takes about 2200 integer instructions here
-// (490 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
-// per product: K_T on 128^3 dipping cells 1254 -> 376; K_T + A_pu + A_up + A22 on
-// 61x127x46 cells sheared both ways 804 -> 271 (A22 121 -> 46); J on 8^3 cells
-// 89 -> 42.
+// issue slots each; the same element takes about 2350 integer instructions here
+// (560 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
+// per product: K_T on 128^3 dipping cells 1254 -> 410; K_T + A_pu + A_up + A22 on
+// 61x127x46 cells sheared both ways 804 -> 285 (A22 121 -> 46); J on 8^3 cells
+// 89 -> 46.
 //
 // Each CTA first looks over its inputs: the largest exponent sets the tile's
 // unit, and the smallest of the elements' largest exponents says how far the
-// field is graded inside the tile.  Where the fixed-point error (2^-69 of the
-// tile's largest term) could exceed the rounding of FP64 arithmetic in some
-// element - values graded by more than a.fx_grade bits inside the tile, not
-// finite, or near the ends of the exponent range - the CTA runs the FP64 tile
-// of gm_bulk.cuh instead, so every element is at least as exact as in FP64.
+// field is graded inside the tile.  A tile that is graded by more than 16 bits
+// (less the contrast of the moduli), not finite, or near the ends of the exponent
+// range takes the FP64 tile of gm_bulk.cuh.
+//
+// The values alone do not say how exact FP64 would be: a field that is constant
+// over an element exerts no force however large it is, and the small ones beside
+// it (another component, a small strain on a large translation) keep all their
+// bits in FP64.  What counts is each element's modes, and they are at hand in
+// registers: FP64 rounds a term K_ij x_j by 2^-54 of itself, fixed point loses
+// about one unit, so an element is exact enough if, for every field of its
+// output, some mode that reaches the field's rows is above the limit from
+// which that rounding is the larger (RefFx.limK, limU; FlowFx.lim), or if all of
+// them are zero and none of the tile's inputs lost bits.  If an element is not,
+// the CTA starts over in FP64, so every element is at least as exact as in
+// FP64.  The look costs one comparison per mode and field (K_T on 128^3: 403 -> 410 us).
 //
 // A thread owns one face, 16 x 16 faces per CTA.  The limbs of the element's
 // modes take 63 registers and those of the carried tuples 36: kept in registers
@@ -44,8 +54,8 @@ struct FxSmem {
 template <int MODE>
 constexpr size_t gm_fx_smem()
 {
-    return sizeof(FxSmem<MODE>) > sizeof(BulkTileSmem<double, MODE>) ? sizeof(FxSmem<MODE>)
-                                                                     : sizeof(BulkTileSmem<double, MODE>);
+    constexpr size_t tile = sizeof(BulkTileSmem<double, MODE == GM_M_AUP ? GM_M_AUP | GM_FX_FLOW : MODE>);
+    return sizeof(FxSmem<MODE>) > tile ? sizeof(FxSmem<MODE>) : tile;
 }
 
 // Output mode s of displacement field c of one element with modulus limbs E:
@@ -70,11 +80,86 @@ __device__ __forceinline__ void gm_fx_k_mode(const RefFx& F, const int (&xv)[24]
 }
 
 // The FP64 tile as a function of its own: it needs twice the registers, and
-// inlined its spills would reach into the fixed-point part.
+// inlined its spills would reach into the fixed-point part.  A_up that adds to the
+// flow block's result runs both blocks: its own planes may be written already.
 template <int CLS, int MODE>
 __device__ __noinline__ void gm_fx_fp64_tile(const BulkArgs<double>& a, const RefOps<double>& R, void* sm)
 {
+    if constexpr (MODE == GM_M_AUP) {
+        constexpr int BOTH = GM_M_AUP | GM_FX_FLOW;
+        if (a.accumulate) {
+            BulkArgs<double> b = a;
+            b.accumulate = 0;
+            gm_bulk_tile<double, CLS, BOTH, false>(b, R, *static_cast<BulkTileSmem<double, BOTH>*>(sm));
+            return;
+        }
+    }
     gm_bulk_tile<double, CLS, MODE, false>(a, R, *static_cast<BulkTileSmem<double, MODE>*>(sm));
+}
+
+// Input mode j reaches the rows of displacement field c.
+template <int CLS>
+__host__ __device__ constexpr bool gm_fx_reaches(const ParPat& PP, int c, int j)
+{
+    for (int s = 1; s < 8; ++s)
+        if (PP.k[c * 8 + s][j] >= 0) return true;
+    return false;
+}
+template <int CLS>
+__host__ __device__ constexpr bool gm_fx_drains(const ParPat& PP, int j)
+{
+    for (int s = 0; s < 8; ++s)
+        if (PP.a[j][s] >= 0) return true;
+    return false;
+}
+
+// Whether the element's modes hold its part of K_b x (A_up x) as exactly as FP64
+// would; cut: some input of the tile lost bits below the unit.
+template <int CLS, int MODE>
+__device__ __forceinline__ bool gm_fx_exact(const RefFx& F, const int (&xv)[24][3], bool cut)
+{
+    constexpr ParPat PP = gm_make_parpat(CLS);
+    constexpr int NC = MODE == GM_M_K ? 3 : 1;
+    bool ok[NC] = {};
+#pragma unroll
+    for (int j = 0; j < 24; ++j) {
+        if ((j & 7) == 0) continue;
+        const int m = abs(xv[j][2]);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if constexpr (MODE == GM_M_K) {
+                if (gm_fx_reaches<CLS>(PP, c, j)) ok[c] |= m > F.limK[c][j];
+            } else {
+                if (gm_fx_drains<CLS>(PP, j)) ok[c] |= m > F.limU[j];
+            }
+        }
+    }
+    bool all = true;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) all &= ok[c];
+    if (all) return true;
+    if (cut) return false;
+    int any = 0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        if (!ok[c])
+#pragma unroll
+            for (int j = 0; j < 24; ++j)
+                if ((j & 7) != 0 && (MODE == GM_M_K ? gm_fx_reaches<CLS>(PP, c, j) : gm_fx_drains<CLS>(PP, j)))
+                    any |= xv[j][0] | xv[j][1] | xv[j][2];
+    return any == 0;
+}
+// The same for the flow block: a Darcy mode, or the storage of the mean pressure.
+__device__ __forceinline__ bool gm_fx_exact_flow(const FlowFx& Q, const int (&xv)[8][3], bool cut)
+{
+    bool ok = false;
+#pragma unroll
+    for (int s = 0; s < 8; ++s) ok |= abs(xv[s][2]) > Q.lim[s];
+    if (ok) return true;
+    int any = cut;
+#pragma unroll
+    for (int s = 1; s < 8; ++s) any |= xv[s][0] | xv[s][1] | xv[s][2];
+    return any == 0;
 }
 
 template <int CLS, int MODE, bool DOT>
@@ -96,7 +181,7 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
     constexpr int TN = 17, PL = TN * TN;
     constexpr ParPat PP = gm_make_parpat(CLS);
     extern __shared__ __align__(16) unsigned char raw[];
-    __shared__ int s_mx[8], s_mn[8];
+    __shared__ int s_mx[8], s_mn[8], s_lo[8];
     __shared__ double s_dot[8];
 
     if (a.skip != nullptr && *a.skip != 0) return;
@@ -119,7 +204,7 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
     // ---- the tile's unit and grading -------------------------------------
     const int kbeg = layer_exists(z0 - 1) ? z0 - 1 : z0;
     const int kend = layer_exists(z1 - 1) ? z1 : z1 - 1;      // last plane read
-    int mx = 0, mn = 0x7fffffff;
+    int mx = 0, mn = 0x7fffffff, least = 0x7fffffff;    // least: the smallest input that is not zero
     {
         int below = 0;
         for (int kk = kbeg; kk <= kend; ++kk) {
@@ -133,7 +218,10 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
 #pragma unroll
                     for (int f = 0; f < NI; ++f) {
                         const int hi = __ldg(reinterpret_cast<const int*>(xin + (long long)f * N + node) + 1) & 0x7fffffff;
-                        if (!((m >> (IN_P ? 3 : f)) & 1u)) m4 = max(m4, hi);
+                        if (!((m >> (IN_P ? 3 : f)) & 1u)) {
+                            m4 = max(m4, hi);
+                            if (hi != 0) least = min(least, hi);
+                        }
                     }
                 }
                 if (layer_exists(kk - 1) && kk > kbeg) {
@@ -146,19 +234,21 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
         }
         mx = __reduce_max_sync(0xffffffffu, mx);
         mn = __reduce_min_sync(0xffffffffu, mn);
-        if ((tid & 31) == 0) { s_mx[tid >> 5] = mx; s_mn[tid >> 5] = mn; }
+        least = __reduce_min_sync(0xffffffffu, least);
+        if ((tid & 31) == 0) { s_mx[tid >> 5] = mx; s_mn[tid >> 5] = mn; s_lo[tid >> 5] = least; }
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < 8; ++w) { mx = max(mx, s_mx[w]); mn = min(mn, s_mn[w]); }
+        for (int w = 0; w < 8; ++w) { mx = max(mx, s_mx[w]); mn = min(mn, s_mn[w]); least = min(least, s_lo[w]); }
     }
     mx >>= 20;
     mn = min(mn >> 20, mx);
+    // a double keeps its 53 bits above the unit, 75 bits below 2^(mx - 1022), within 2^22 of the largest
+    const bool cut = mx - min(least >> 20, mx) > 22;
     const int top = mx == 0 ? 1023 : mx;
     const int qe = (top - 1022 - GM_FX_IN) + (DO_K ? F.eK + F.topE - 1022 : DO_Q ? Q.eU : F.eA);
     const bool fixed_ok = top < 0x7ff && top >= 100 && qe >= -1000 && qe <= 900 &&
-                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : DO_Q ? Q.grade : F.gradeA));
-    if (!fixed_ok) {
-        // uniform over the CTA
+                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : DO_Q ? Q.grade : DO_AUP ? GM_FX_GRADE : F.gradeA));
+    auto fp64_tile = [&]() {
         gm_fx_fp64_tile<CLS, MODE>(a, R, raw);
         if constexpr (DOT) {
             // the thread's own outputs times its inputs, off the lips
@@ -176,6 +266,9 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
                 }
             gm_cta_dot(dot, s_dot, a.part);
         }
+    };
+    if (!fixed_ok) {                   // uniform over the CTA
+        fp64_tile();
         return;
     }
     FxSmem<MODE>& S = *reinterpret_cast<FxSmem<MODE>*>(raw);
@@ -294,6 +387,7 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
     // field: complete the face tuples of plane kb, transform them back and
     // exchange; in any case the layer's top contributions become the carry.
     int low[NO][NL];
+    bool inexact = false;
     auto layer = [&](int kb, bool exists, bool plane) {
         const bool work = exists && fval;
         int xv[NI * 8][3];
@@ -318,6 +412,9 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
             }
             if constexpr (DO_K) gm_fx_coef22(Ed, F.topE, E);
             if constexpr (DO_Q) gm_fx_coef(Ed, Q.topW, E);
+            if constexpr (DO_K || DO_AUP) inexact |= !gm_fx_exact<CLS, MODE>(F, xv, cut);
+            if constexpr (DO_Q)
+                if (a.cC != 0.0) inexact |= !gm_fx_exact_flow(Q, xv, cut);
         }
 #pragma unroll
         for (int c = 0; c < NO; ++c) {
@@ -399,12 +496,18 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
     for (int kk = kbeg; kk < z1; ++kk) {
         const bool next = kk + 2 <= kend;
         if (next) fetch(kk + 2);
-        __syncthreads();
+        if (__syncthreads_or(inexact)) {
+            fp64_tile();
+            return;
+        }
         if (kk > z0) node_stage(kk - 1);
         layer(kk, layer_exists(kk), kk >= z0);
         if (next) store((kk + 2 - kbeg) % 3);
     }
-    __syncthreads();
+    if (__syncthreads_or(inexact)) {
+        fp64_tile();
+        return;
+    }
     node_stage(z1 - 1);
     if constexpr (DOT) gm_cta_dot(dot, s_dot, a.part);
 }

@@ -25,7 +25,7 @@
 constexpr int GM_FX_RADIX = 26;
 constexpr int GM_FX_MASK = (1 << GM_FX_RADIX) - 1;
 constexpr int GM_FX_IN = 75;       // bits of an input value
-constexpr int GM_FX_GRADE = 16;    // bits of grading inside a tile that leave FP64's rounding the larger error
+constexpr int GM_FX_GRADE = 16;    // bits of grading inside a tile beyond which fixed point is not tried
 
 __host__ __device__ inline int64_t gm_fx_bits(double x)
 {

@@ -136,6 +136,14 @@ void fx_limbs(double hi, double lo, int e, int (&l)[NL])
     l[NL - 1] = sg * (int)n;
 }
 
+// top limb from which a mode with a coefficient m outweighs `units` of the last
+// place times 2^52 (8: what the limbs below it can add); none for m = 0
+int fx_limit(double units, double m)
+{
+    const double l = m > 0.0 ? units / m : HUGE_VAL;
+    return l < 1073741824.0 ? (int)l + 8 : 0x7fffffff;
+}
+
 // Fixed-point copy of the reference operators: scaled by the power of two that
 // bounds the absolute sum of every row (twice that for the couplings).
 void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat& PP, double alpha, double Emin,
@@ -178,22 +186,31 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
                 fx_limbs(hi, std::fma(alpha, At[i][j], -hi), F.eA, F.a[PP.a[i][j]]);
             }
     }
-    // Grading: what lies below the unit in the coefficients comes off it.  An output
-    // mode is off by about one unit of 2^(eK - 75), where FP64 rounds 2^-54 of a term
-    // K_jj x_j: exact enough while 20 bits less the distance of the smallest K_jj
-    // from 2^eK (5 for a cube, 16 for a cell of 100:100:1) cover the grading.  Moduli
-    // likewise (their limbs are exact within 2^21 of the largest).  A_pu: the forces
-    // that a uniform pressure exerts, field by field.
-    double kd = 0.0, ad = 0.0;
-    for (int i = 0; i < 24; ++i)
-        if ((i & 7) != 0 && (kd == 0.0 || Kt[i][i] < kd)) kd = Kt[i][i];
+    // Limits: an output mode of K_b is off by about one unit of 2^(eK - 75) E_max
+    // (A_up: 2.6 of 2^(eA - 75)), where FP64 rounds 2^-54 of a term K_ij x_j E.
+    const int contrast = std::ilogb(Emax) - std::ilogb(Emin);
+    for (int j = 0; j < 24; ++j) {
+        for (int c = 0; c < 3; ++c) {
+            double m = 0.0;
+            for (int s = 0; s < 8; ++s)
+                if (PP.k[c * 8 + s][j] >= 0) m = std::max(m, std::fabs(Kt[c * 8 + s][j]));
+            F.limK[c][j] = fx_limit(std::ldexp(4.0, F.eK + contrast), m);
+        }
+        double m = 0.0;
+        for (int s = 0; s < 8; ++s)
+            if (PP.a[j][s] >= 0) m = std::max(m, std::fabs(alpha * At[j][s]));
+        F.limU[j] = fx_limit(std::ldexp(12.0, F.eA), m);
+    }
+    // A_pu: the forces that a uniform pressure exerts, field by field, against the same
+    double ad = 0.0;
     for (int c = 0; c < 3; ++c) {
         double m = 0.0;
         for (int s = 0; s < 8; ++s) m = std::max(m, std::fabs(alpha * At[c * 8 + s][0]));
         if (m > 0.0 && (ad == 0.0 || m < ad)) ad = m;
     }
+    // moduli: limbs are exact while the smallest is within 2^21 of the largest
     F.topE = std::ilogb(Emax) + 1023;
-    F.gradeK = kd > 0.0 ? std::min(GM_FX_GRADE, 20 - (F.eK - std::ilogb(kd))) - (std::ilogb(Emax) - std::ilogb(Emin)) : -1;
+    F.gradeK = GM_FX_GRADE - contrast;
     F.gradeA = ad > 0.0 ? std::min(GM_FX_GRADE, 21 - (F.eA - std::ilogb(ad))) : GM_FX_GRADE;
 }
 
@@ -202,7 +219,8 @@ void make_fx(const double (&Kt)[24][24], const double (&At)[24][8], const ParPat
 // does not belong to the class, or the pattern rule does not hold).
 template <int CLS>
 bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8],
-              const double L[8][8], RefOps<double>& R, RefFx& F, double alpha, double Emin, double Emax, double& Lsum)
+              const double L[8][8], RefOps<double>& R, RefFx& F, double alpha, double Emin, double Emax, double& Lsum,
+              double (&Lcol)[8])
 {
     constexpr ParPat PP = gm_make_parpat(CLS);
     static double Kt[24][24], At[24][8], Mt[8][8], Lt[8][8];   // index (c*8+s)
@@ -264,10 +282,14 @@ bool pack_ref(const double K[24][24], const double A[24][8], const double M[8][8
         }
     make_fx(Kt, At, PP, alpha, Emin, Emax, F);
     Lsum = 0.0;
+    for (double& m : Lcol) m = 0.0;
     for (int i = 0; i < 8; ++i) {
         double t = 0.0;
         for (int j = 0; j < 8; ++j)
-            if (PP.l[i][j] >= 0) t += std::fabs(Lt[i][j]);
+            if (PP.l[i][j] >= 0) {
+                t += std::fabs(Lt[i][j]);
+                Lcol[j] = std::max(Lcol[j], std::fabs(Lt[i][j]));
+            }
         Lsum = std::max(Lsum, t);
     }
     return true;
@@ -334,6 +356,11 @@ FlowFx gm_flow_fx(const gm_ctx* c, double cS, double cC)
         const double f = cS / c->M, v = f * c->R64.M[i];
         fx_limbs(v, std::fma(f, c->R64.M[i], -v), Q.eU, Q.m[i]);
     }
+    // limits as for K_b, 2.3 units here; mode 0 by the storage that it meets in an
+    // element of the largest k
+    const double unitL = std::ldexp(12.0, eL);
+    for (int s = 1; s < 8; ++s) Q.lim[s] = fx_limit(unitL, c->Lcol[s]);
+    Q.lim[0] = cC > 0.0 ? fx_limit(unitL * cC * c->kap_hi, storage) : 0x7fffffff;
     // the fourth limb of the results covers coefficients 2^24 apart; the inputs'
     // own grading is judged by the kernel as for the other blocks.  A pressure that
     // is uniform over an element meets its storage alone, however strong the flow:
@@ -966,9 +993,9 @@ int bind_impl(gm_ctx* c)
     if (!ref_cell(c->h, c->shear, c->nu, K, A, M, L)) return c->set_err(GM_EINVAL, "bind: degenerate cell");
     const auto Er = std::minmax_element(c->E.begin(), c->E.end());
     const double E0 = *Er.first, E1 = *Er.second;
-    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum)
-            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum)
-                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum);
+    bool ok = c->cls == GM_CLS_BOX ? pack_ref<GM_CLS_BOX>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum, c->Lcol)
+            : c->cls == GM_CLS_MONO ? pack_ref<GM_CLS_MONO>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum, c->Lcol)
+                                    : pack_ref<GM_CLS_GEN>(K, A, M, L, c->R64, c->Rfx, c->alpha, E0, E1, c->Lsum, c->Lcol);
     if (!ok) return c->set_err(GM_EINVAL, "bind: cell operators break the expected parity pattern");
     cast_ref(c->R64, c->R32);
     for (int i = 0; i < GM_PP_MAXK; ++i) c->R32p.K[i] = make_float2(c->R32.K[i], c->R32.K[i]);

@@ -166,23 +166,27 @@ struct RefPairs32 {
 // fraction) 2^eK or 2^eA, scaled so
 // that the absolute sum of a row is at most 1 (K) or 1/2 (A: 36 results meet in
 // a node).  topE is the biased exponent of the largest Young's modulus; gradeK,
-// gradeA the grading of an input inside a tile, in bits, up to which the
-// fixed-point error stays below the rounding of FP64.
+// gradeA the grading of an input inside a tile, in bits, beyond which a tile is not
+// tried (A_pu: up to which its error stays below the rounding of FP64).  limK[c][j],
+// limU[j]: top limb above which input mode j alone has FP64 round more in the rows of
+// field c (of A_up) than fixed point loses.
 struct RefFx {
     int k[GM_PP_MAXK][3];
     int a[GM_PP_MAXA][3];
     int eK, eA, topE, gradeK, gradeA;
+    int limK[3][24], limU[24];
 };
 
 // The flow block of one launch in the same form: Darcy entries (row sums at most
 // 1), storage per mode in four limbs, and the scale 2^eU that bounds both (a quarter
 // each, so that 36 results of their sum meet in a node); topW is the biased exponent of
 // the largest dt k/mu that the scale admits.  grade < 0: coefficients too far
-// apart for the fixed-point unit, use FP64.
+// apart for the fixed-point unit, use FP64.  lim as in RefFx (mode 0: by its storage).
 struct FlowFx {
     int l[GM_PP_MAXL][3];
     int m[8][4];
     int topW, eU, grade;
+    int lim[8];
 };
 
 // Per-node mask bits: 1,2,4 = ux,uy,uz fixed, 8 = p fixed.
@@ -433,6 +437,7 @@ struct gm_ctx {
     RefPairs32 R32p{};
     RefFx Rfx{};
     double Lsum = 0.0;            // largest absolute row sum of the Darcy operator in the parity basis (k/mu = 1)
+    double Lcol[8] = {};          // and largest entry of each column
     double kap_lo = 0.0, kap_hi = 0.0;   // smallest positive and largest k/mu of an element (0: none)
     bool kap_zero = false;        // some element has k = 0
     double Kblk_ref[8][9] = {};   // nodal 3x3 diagonal blocks of K_ref (E = 1)
