@@ -249,7 +249,8 @@ int gm_set_friction(gm_ctx* ctx, const double* f_host, int64_t n);
  * first use (its set-up synchronises); grids whose cell counts or fault index
  * cannot be halved keep kind 0.  The environment variables GM_MG_MIN_CELLS,
  * GM_MG_SMOOTH_DEG, GM_MG_COARSE_DEG, GM_MG_SMOOTH_LO and GM_MG_COARSE_LO,
- * read at set-up, override these choices (tuning only).  The converged solutions agree to the solver tolerances.  GM_EINVAL
+ * read at set-up, override these choices, and GM_MG_COARSE_CLUSTER=0 runs the
+ * coarsest level as launches instead of one kernel (tuning only).  The converged solutions agree to the solver tolerances.  GM_EINVAL
  * for another kind. */
 int gm_set_preconditioner(gm_ctx* ctx, int kind);
 

@@ -70,6 +70,14 @@ int mg_coarse_deg()
     return (n >= 1 && n <= MG_MAX_COARSE_DEG) ? n : MG_COARSE_DEG;
 }
 
+// the coarsest level's polynomial as one cluster kernel where it fits (default), or
+// with GM_MG_COARSE_CLUSTER=0 always as launches
+bool mg_coarse_cluster()
+{
+    const char* v = std::getenv("GM_MG_COARSE_CLUSTER");
+    return !v || std::atoi(v) != 0;
+}
+
 // grid of a level's vector kernels: one thread per node up to the fixed grid
 int mg_blocks(long long N)
 {
@@ -730,8 +738,10 @@ int build(gm_ctx* c)
     c->mg[0].b = nullptr;
     c->mg[0].x = nullptr;
     MGLevel& last = c->mg.back();
-    last.cluster32 = coarse_cluster<float>(last.cx);
-    last.cluster64 = coarse_cluster<double>(last.cx);
+    if (mg_coarse_cluster()) {
+        last.cluster32 = coarse_cluster<float>(last.cx);
+        last.cluster64 = coarse_cluster<double>(last.cx);
+    }
     int off = 1;
     for (size_t l = 0; l < c->mg.size(); ++l) {
         MGLevel& L = c->mg[l];
