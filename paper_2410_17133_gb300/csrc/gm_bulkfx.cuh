@@ -113,13 +113,12 @@ __host__ __device__ constexpr bool gm_fx_drains(const ParPat& PP, int j)
     return false;
 }
 
-// Whether the element's modes hold its part of K_b x (A_up x) as exactly as FP64
-// would; cut: some input of the tile lost bits below the unit.
-template <int CLS, int MODE>
+// Whether the element's modes hold its part of K_b x (fields C0 to C0 + NC - 1; or of
+// A_up x) as exactly as FP64 would; cut: some input of the tile lost bits below the unit.
+template <int CLS, int MODE, int C0 = 0, int NC = MODE == GM_M_K ? 3 : 1>
 __device__ __forceinline__ bool gm_fx_exact(const RefFx& F, const int (&xv)[24][3], bool cut)
 {
     constexpr ParPat PP = gm_make_parpat(CLS);
-    constexpr int NC = MODE == GM_M_K ? 3 : 1;
     bool ok[NC] = {};
 #pragma unroll
     for (int j = 0; j < 24; ++j) {
@@ -128,7 +127,7 @@ __device__ __forceinline__ bool gm_fx_exact(const RefFx& F, const int (&xv)[24][
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             if constexpr (MODE == GM_M_K) {
-                if (gm_fx_reaches<CLS>(PP, c, j)) ok[c] |= m > F.limK[c][j];
+                if (gm_fx_reaches<CLS>(PP, C0 + c, j)) ok[c] |= m > F.limK[C0 + c][j];
             } else {
                 if (gm_fx_drains<CLS>(PP, j)) ok[c] |= m > F.limU[j];
             }
@@ -145,7 +144,7 @@ __device__ __forceinline__ bool gm_fx_exact(const RefFx& F, const int (&xv)[24][
         if (!ok[c])
 #pragma unroll
             for (int j = 0; j < 24; ++j)
-                if ((j & 7) != 0 && (MODE == GM_M_K ? gm_fx_reaches<CLS>(PP, c, j) : gm_fx_drains<CLS>(PP, j)))
+                if ((j & 7) != 0 && (MODE == GM_M_K ? gm_fx_reaches<CLS>(PP, C0 + c, j) : gm_fx_drains<CLS>(PP, j)))
                     any |= xv[j][0] | xv[j][1] | xv[j][2];
     return any == 0;
 }

@@ -574,7 +574,7 @@ int coarse_launch(gm_ctx* c, const MGLevel& L, int n, const int* skip, cudaStrea
     cfg.attrs = at;
     const int chained = gm_capturing(s) ? 0 : 1;
     cfg.numAttrs = 1 + chained;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, mg_coarse_kernel<T, MT, CLS>, chained, a, x->R32, x->Rfx);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, mg_coarse_kernel<T, MT, CLS>, chained, a, x->R32, x->Rfx, x->R64);
     if (e != cudaSuccess) return c->set_err(GM_ECUDA, std::string("multigrid: coarsest level: ") + cudaGetErrorString(e));
     x->applies += L.deg - 1;
     GM_LAUNCHED(c);

@@ -14,9 +14,10 @@
 // items as there are: elements of the two layers around the row (FP64: and
 // output fields), then (node, component) twice.  FP32 multiplies in the parity
 // basis like gm_bulk32.cuh; FP64 in wide fixed point like gm_bulkfx.cuh with the
-// unit of the CTA's rows (a preconditioner needs no grading test; values that
-// are not finite give NaN).  The march direction is y here: a mode's bit 1
-// (s & 2) separates a layer's lower and upper rows.
+// unit of the CTA's rows, and a step whose values that would not hold as exactly
+// as FP64 (the same test, element by element) is done again in FP64 by that CTA.
+// The march direction is y here: a mode's bit 1 (s & 2) separates a layer's lower
+// and upper rows.
 // Included by gm_mg.cu only.
 #pragma once
 
@@ -98,10 +99,100 @@ __host__ __device__ inline MgcLayout mgc_layout(const GridDesc& g, int rows)
     return L;
 }
 
+// Modes of the element whose lower row is `row` of the staged rows, first node nd.
+template <typename W, int NL>
+__device__ __forceinline__ void mgc_modes(const W* st, int row, int nd, int rn, int rowlen, W (&xv)[24][NL])
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            W t[2][4];                                          // [ay][sx + 2 sz]
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const W* v = st + ((size_t)((row + s) * 3 + c) * NL + l) * rn + nd;
+                const W a0 = v[0] + v[1], a1 = v[0] - v[1];
+                const W b0 = v[rowlen] + v[rowlen + 1], b1 = v[rowlen] - v[rowlen + 1];
+                t[s][0] = a0 + b0;
+                t[s][1] = a1 + b1;
+                t[s][2] = a0 - b0;
+                t[s][3] = a1 - b1;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int s0 = (q & 1) | ((q & 2) << 1);        // mode (sx, 0, sz)
+                xv[c * 8 + s0][l] = t[0][q] + t[1][q];
+                xv[c * 8 + (s0 | 2)][l] = t[0][q] - t[1][q];
+            }
+        }
+}
+
+// What the element gives its upper (lay 0) or lower row in one field, corner by
+// corner (ax + 2 az): mode(s, y) forms output mode s.
+template <typename W, int NL, class Mode>
+__device__ __forceinline__ void mgc_corners(W* w, int faces, int lay, Mode mode)
+{
+    W o[4][NL];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        W lo[NL] = {}, hi[NL];
+        const int s0 = (q & 1) | ((q & 2) << 1);
+        if (s0 != 0) mode(s0, lo);                              // the constant mode carries no force
+        mode(s0 | 2, hi);
+#pragma unroll
+        for (int l = 0; l < NL; ++l) o[q][l] = lay == 0 ? lo[l] - hi[l] : lo[l] + hi[l];
+    }
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const W p0 = o[0][l] + o[1][l], p1 = o[0][l] - o[1][l];
+        const W q0 = o[2][l] + o[3][l], q1 = o[2][l] - o[3][l];
+        w[(size_t)l * faces] = p0 + q0;
+        w[(size_t)(NL + l) * faces] = p1 + q1;
+        w[(size_t)(2 * NL + l) * faces] = p0 - q0;
+        w[(size_t)(3 * NL + l) * faces] = p1 - q1;
+    }
+}
+
+// The layers' results of a step in FP64, from staged doubles: as the fixed-point
+// items, for the steps whose values those would not hold (see below).
+template <int CLS>
+__device__ __noinline__ void mgc_layers_f64(const RefOps<double>& R, const GridDesc& g, int j0, int own, unsigned m_faces,
+                                            unsigned m_nx, const double* st, const double* sE, double* out)
+{
+    constexpr ParPat PP = gm_make_parpat(CLS);
+    const int rowlen = g.nx + 1, rn = rowlen * g.nplanes, faces = g.nx * g.nz;
+    for (int it = threadIdx.x; it < own * 6 * faces; it += blockDim.x) {
+        const int blk = mgc_div(it, m_faces), f = it - blk * faces, rl = blk / 3, cc = blk - rl * 3;
+        const int row = rl >> 1, lay = rl & 1, j = j0 + row;
+        double* w = out + (size_t)(rl * 3 + cc) * 4 * faces + f;
+        if (lay == 0 ? j == 0 : j == g.ny) {
+            for (int q = 0; q < 4; ++q) w[(size_t)q * faces] = 0.0;
+            continue;
+        }
+        const int ek = mgc_div(f, m_nx), fi = f - ek * g.nx;
+        double xv[24][1];
+        mgc_modes<double, 1>(st, row + lay, fi + rowlen * (ek + (g.kf >= 0 && ek >= g.kf ? 1 : 0)), rn, rowlen, xv);
+        const double Ee = sE[(size_t)(row + lay) * faces + f];
+        auto field = [&](auto c_) {
+            constexpr int c = decltype(c_)::value;
+            mgc_corners<double, 1>(w, faces, lay, [&](int s, double (&y)[1]) {
+                double t = 0.0;
+#pragma unroll
+                for (int i = 0; i < 24; ++i)
+                    if (PP.k[c * 8 + s][i] >= 0 && (i & 7) != 0) t = fma(R.K[PP.k[c * 8 + s][i]], xv[i][0], t);
+                y[0] = Ee * t;
+            });
+        };
+        if (cc == 0) field(std::integral_constant<int, 0>{});
+        if (cc == 1) field(std::integral_constant<int, 1>{});
+        if (cc == 2) field(std::integral_constant<int, 2>{});
+    }
+}
+
 template <typename T, typename MT, int CLS>
 __global__ void __launch_bounds__(mgc_threads<T>(), 1)
 mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const __grid_constant__ RefOps<float> R,
-                 const __grid_constant__ RefFx F)
+                 const __grid_constant__ RefFx F, const __grid_constant__ RefOps<double> R64)
 {
     gm_chain(chained);
     constexpr bool FX = sizeof(T) == 8;
@@ -114,7 +205,7 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
     const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
 
     extern __shared__ __align__(16) unsigned char mgc_raw[];
-    __shared__ int s_top[NT / 32];
+    __shared__ int s_top[NT / 32], s_least[NT / 32];
     const GridDesc& g = a.g;
     const MgcLayout L = mgc_layout<T, MT>(g, a.rows);
     const int rowlen = g.nx + 1, rn = rowlen * g.nplanes, faces = g.nx * g.nz;
@@ -184,22 +275,28 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
         const T* xi = sx + (step & 1 ? 0 : buf);                    // written by the step before
         T* xo = sx + (step & 1 ? buf : 0);
         double scale = 0.0;
+        bool inexact = false, cut = false, f64 = false;             // FP64: see gm_fx_exact
+        const T* from[2] = {xi, xi};
+        // field f of staged node q: rows j0 - 1 .. j1, own rows and the neighbours' nearest ones
+        auto value = [&](int q, int f) -> T {
+            const int r = mgc_div(q, a.m_rn), n = q - r * rn, j = j0 - 1 + r;
+            if (j < 0 || j > g.ny || ((sm[q] >> f) & 1u)) return T(0);
+            const T* p = r == 0 ? from[0] : r == own + 1 ? from[1] : xi + (size_t)(r - 1) * 3 * rn;
+            return p[(size_t)f * rn + n];
+        };
         if (step > 0 && own > 0) {
-            // stage rows j0 - 1 .. j1: own rows, and the neighbours' nearest ones
-            int top = 0;
-            const T* from[2] = {xi, xi};
+            int top = 0, least = 0x7ff;
             if (rank > 0 && j0 > 0) from[0] = cl.map_shared_rank(const_cast<T*>(xi), rank - 1) +
                                               (size_t)(j0 - 1 - mgc_row(g, rank - 1, ncta)) * 3 * rn;
             if (rank + 1 < ncta && j1 <= g.ny) from[1] = cl.map_shared_rank(const_cast<T*>(xi), rank + 1);
             const int count = (own + 2) * rn;
-            auto value = [&](int q, int f) -> T {
-                const int r = mgc_div(q, a.m_rn), n = q - r * rn, j = j0 - 1 + r;
-                if (j < 0 || j > g.ny || ((sm[q] >> f) & 1u)) return T(0);
-                const T* p = r == 0 ? from[0] : r == own + 1 ? from[1] : xi + (size_t)(r - 1) * 3 * rn;
-                return p[(size_t)f * rn + n];
-            };
             if constexpr (FX) {
                 constexpr int MAXQ = 8;                             // values kept between the two passes
+                auto extent = [&](T v) {
+                    const int e = (__double2hiint(v) & 0x7fffffff) >> 20;
+                    top = max(top, e);
+                    if (v != T(0)) least = min(least, e);
+                };
                 T keep[MAXQ];
 #pragma unroll
                 for (int u = 0; u < MAXQ; ++u) {
@@ -208,22 +305,25 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
                     if (i < 3 * count) {
                         const int f = (i >= count) + (i >= 2 * count);
                         keep[u] = value(i - f * count, f);
-                        top = max(top, (__double2hiint(keep[u]) & 0x7fffffff) >> 20);
+                        extent(keep[u]);
                     }
                 }
                 for (int i = tid + MAXQ * NT; i < 3 * count; i += NT) {
                     const int f = (i >= count) + (i >= 2 * count);
-                    top = max(top, (__double2hiint(value(i - f * count, f)) & 0x7fffffff) >> 20);
+                    extent(value(i - f * count, f));
                 }
                 top = __reduce_max_sync(0xffffffffu, top);
-                if ((tid & 31) == 0) s_top[tid >> 5] = top;
+                least = __reduce_min_sync(0xffffffffu, least);
+                if ((tid & 31) == 0) { s_top[tid >> 5] = top; s_least[tid >> 5] = least; }
                 __syncthreads();
 #pragma unroll
-                for (int w = 0; w < NT / 32; ++w) top = max(top, s_top[w]);
-                // a field of zeros or subnormals gives zero; not finite gives NaN
+                for (int w = 0; w < NT / 32; ++w) { top = max(top, s_top[w]); least = min(least, s_least[w]); }
+                // values at the ends of the exponent range, or not finite: FP64
                 const int qe = (top - 1022 - GM_FX_IN) + F.eK + F.topE - 1022;
-                scale = top == 0x7ff || qe > 900 ? nan("")
-                      : qe < -1000 || top < 100 ? 0.0 : gm_fx_real((int64_t)(qe + 1023) << 52);
+                const bool ends = least != 0x7ff && (top == 0x7ff || top < 100 || qe > 900 || qe < -1000);
+                cut = top - least > 22;
+                inexact = ends;
+                scale = ends || least == 0x7ff ? 0.0 : gm_fx_real((int64_t)(qe + 1023) << 52);
                 auto limbs = [&](int i, T v) {
                     const int f = (i >= count) + (i >= 2 * count), q = i - f * count, r = mgc_div(q, a.m_rn), n = q - r * rn;
                     int l[3];
@@ -265,71 +365,45 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
                 const int ek = mgc_div(f, a.m_nx), fi = f - ek * g.nx;
                 const int nd = fi + rowlen * (ek + (g.kf >= 0 && ek >= g.kf ? 1 : 0));
                 W xv[24][NL];
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        W t[2][4];                              // [ay][sx + 2 sz]
-#pragma unroll
-                        for (int s = 0; s < 2; ++s) {
-                            const W* v = st + ((size_t)((row + lay + s) * 3 + c) * NL + l) * rn + nd;
-                            const W a0 = v[0] + v[1], a1 = v[0] - v[1];
-                            const W b0 = v[rowlen] + v[rowlen + 1], b1 = v[rowlen] - v[rowlen + 1];
-                            t[s][0] = a0 + b0;
-                            t[s][1] = a1 + b1;
-                            t[s][2] = a0 - b0;
-                            t[s][3] = a1 - b1;
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int s0 = (q & 1) | ((q & 2) << 1);     // mode (sx, 0, sz)
-                            xv[c * 8 + s0][l] = t[0][q] + t[1][q];
-                            xv[c * 8 + (s0 | 2)][l] = t[0][q] - t[1][q];
-                        }
-                    }
+                mgc_modes<W, NL>(st, row + lay, nd, rn, rowlen, xv);
                 const T Ee = sE[(size_t)(row + lay) * faces + f];
                 int El[3] = {0, 0, 0};
                 if constexpr (FX) gm_fx_coef22(Ee, F.topE, El);
                 auto field = [&](auto c_) {
                     constexpr int c = decltype(c_)::value;
-                    W o[4][NL];
+                    if constexpr (FX) inexact |= !gm_fx_exact<CLS, GM_M_K, c, 1>(F, xv, cut);
+                    mgc_corners<W, NL>(out + (size_t)(rl * 3 + c) * 4 * NL * faces + f, faces, lay, [&](int s, W (&y)[NL]) {
+                        if constexpr (FX) {
+                            gm_fx_k_mode<CLS>(F, xv, c, s, El, y);
+                        } else {
+                            float t = 0.f;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        W lo[NL] = {}, hi[NL];
-                        auto mode = [&](int s, W (&y)[NL]) {
-                            if constexpr (FX) {
-                                gm_fx_k_mode<CLS>(F, xv, c, s, El, y);
-                            } else {
-                                float t = 0.f;
-#pragma unroll
-                                for (int i = 0; i < 24; ++i)
-                                    if (PP.k[c * 8 + s][i] >= 0 && (i & 7) != 0)
-                                        t = fmaf(R.K[PP.k[c * 8 + s][i]], xv[i][0], t);
-                                y[0] = Ee * t;
-                            }
-                        };
-                        const int s0 = (q & 1) | ((q & 2) << 1);
-                        if (s0 != 0) mode(s0, lo);              // the constant mode carries no force
-                        mode(s0 | 2, hi);
-#pragma unroll
-                        for (int l = 0; l < NL; ++l) o[q][l] = lay == 0 ? lo[l] - hi[l] : lo[l] + hi[l];
-                    }
-#pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        const W p0 = o[0][l] + o[1][l], p1 = o[0][l] - o[1][l];
-                        const W q0 = o[2][l] + o[3][l], q1 = o[2][l] - o[3][l];
-                        W* w = out + (size_t)((rl * 3 + c) * 4 * NL + l) * faces + f;
-                        w[0] = p0 + q0;                         // corner ax + 2 az
-                        w[(size_t)NL * faces] = p1 + q1;
-                        w[(size_t)2 * NL * faces] = p0 - q0;
-                        w[(size_t)3 * NL * faces] = p1 - q1;
-                    }
+                            for (int i = 0; i < 24; ++i)
+                                if (PP.k[c * 8 + s][i] >= 0 && (i & 7) != 0) t = fmaf(R.K[PP.k[c * 8 + s][i]], xv[i][0], t);
+                            y[0] = Ee * t;
+                        }
+                    });
                 };
                 if (NC == 1 || cc == 0) field(std::integral_constant<int, 0>{});
                 if (NC == 1 || cc == 1) field(std::integral_constant<int, 1>{});
                 if (NC == 1 || cc == 2) field(std::integral_constant<int, 2>{});
             }
-            __syncthreads();
+            if constexpr (FX) {
+                f64 = __syncthreads_or(inexact);
+                if (f64) {
+                    double* sv = reinterpret_cast<double*>(st);
+                    for (int i = tid; i < 3 * (own + 2) * rn; i += NT) {
+                        const int q = mgc_div(i, a.m_rn), n = i - q * rn, r = q / 3, f = q - 3 * r;
+                        sv[i] = value(r * rn + n, f);
+                    }
+                    __syncthreads();
+                    mgc_layers_f64<CLS>(R64, g, j0, own, a.m_faces, a.m_nx, sv, reinterpret_cast<const double*>(sE),
+                                        reinterpret_cast<double*>(out));
+                    __syncthreads();
+                }
+            } else {
+                __syncthreads();
+            }
         }
         // residual r = b - K_T x
         for (int it = tid; it < own * 3 * rn; it += NT) {
@@ -337,19 +411,32 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
             const int fl = item.y;
             T r = sb[it];
             if (step > 0 && !(fl & FIXED)) {
-                W s[NL];
+                if (FX && f64) {
+                    // the item's first result, counted in values instead of limbs
+                    const int blk = mgc_div(it, a.m_rn), rc = (blk / 3) * 6 + blk % 3;
+                    const T* w0 = reinterpret_cast<const T*>(out) + item.x - (size_t)rc * 4 * (NL - 1) * faces;
+                    T s = T(0);
 #pragma unroll
-                for (int l = 0; l < NL; ++l) s[l] = W(0);
+                    for (int q = 0; q < 4; ++q) {
+                        const T* w = w0 + q * faces - (q & 1) - (q >> 1) * g.nx;
+                        if (fl & (1 << q)) s += w[0] + w[(size_t)12 * faces];
+                    }
+                    r -= s;
+                } else {
+                    W s[NL];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int dx = q & 1, dz = q >> 1;
-                    const W* w = out + item.x + q * NL * faces - dx - dz * g.nx;
-                    if (fl & (1 << q))
+                    for (int l = 0; l < NL; ++l) s[l] = W(0);
 #pragma unroll
-                        for (int l = 0; l < NL; ++l) s[l] += w[l * faces] + w[(12 * NL + l) * faces];
+                    for (int q = 0; q < 4; ++q) {
+                        const int dx = q & 1, dz = q >> 1;
+                        const W* w = out + item.x + q * NL * faces - dx - dz * g.nx;
+                        if (fl & (1 << q))
+#pragma unroll
+                            for (int l = 0; l < NL; ++l) s[l] += w[l * faces] + w[(12 * NL + l) * faces];
+                    }
+                    if constexpr (FX) r -= scale * gm_fx_to_double(s[0], s[1], s[2]);
+                    else r -= s[0];
                 }
-                if constexpr (FX) r -= scale * gm_fx_to_double(s[0], s[1], s[2]);
-                else r -= s[0];
                 if (fl & LIP) {
                     // cohesive force +-A_i D [[x]]
                     const int blk = mgc_div(it, a.m_rn), row = blk / 3, c = blk - row * 3, j = j0 + row;

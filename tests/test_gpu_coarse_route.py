@@ -93,3 +93,22 @@ def test_iterations_in_single_precision_do_not_depend_on_the_route(monkeypatch):
     (n0, k0, l0, u0), (n1, k1, l1, u1) = out
     assert n0 == n1 and abs(k0 - k1) <= 0.1 * k1 and l0 < l1
     assert np.linalg.norm(u0 - u1) <= 1e-6 * np.linalg.norm(u1)
+
+
+@pytest.mark.parametrize("shear", [(0.0, 0.0), DIP, SKEW])
+def test_values_far_below_the_largest_keep_their_bits(monkeypatch, shear):
+    """Two patches of forces, one 2^-40 of the other, on rows that one CTA owns, and polynomials so
+    short that neither reaches the other: around the small patch both routes agree within some
+    ten roundings of 24 products each, 500 eps < 1e-13 of the values there."""
+    need_gpu()
+    monkeypatch.setenv("GM_MG_COARSE_DEG", "2")
+    monkeypatch.setenv("GM_MG_SMOOTH_DEG", "1")
+    prob = block(8, 20, 60, False, shear=shear)
+    k = np.arange(prob.n_nodes) // (9 * 21)
+    size = np.where(abs(k - 10) <= 1, 1.0, 0.0) + np.where(abs(k - 50) <= 1, 2.0 ** -40, 0.0)
+    b = cuda(np.random.default_rng(5).normal(size=(3, prob.n_nodes)) * size)
+    (x, n), (y, m) = (one_cycle(monkeypatch, c, prob, b) for c in (True, False))
+    assert m - n >= 2                                       # degree 2: three launches in one
+    far = k >= 40
+    assert np.abs(y[:, far]).max() > 0.0
+    assert np.abs(x - y)[:, far].max() <= 1e-13 * np.abs(y[:, far]).max()
