@@ -47,7 +47,7 @@ def host(tmp_path_factory):
     d = tmp_path_factory.mktemp("host")
     (d / "runtime.cpp").write_text(src)
     so = str(d / "host.so")
-    subprocess.run(["g++", "-O1", "-shared", "-fPIC", f"-DFAIL=({EFAIL})", "-o", so, str(d / "runtime.cpp"), obj], check=True)
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-DFAIL=({EFAIL})", "-o", so, str(d / "runtime.cpp"), obj], check=True)
     return ctypes.CDLL(so)
 
 
