@@ -21,6 +21,8 @@
 // Included by gm_mg.cu only.
 #pragma once
 
+#include <mutex>
+
 #include <cooperative_groups.h>
 
 #include "gm_bulkfx.cuh"
@@ -488,12 +490,15 @@ mg_coarse_kernel(int chained, const __grid_constant__ CoarseArgs<T, MT> a, const
     }
 }
 
-// Cluster size the kernel runs with on this device (0: not available).
+// Cluster size the kernel runs with on this device (0: not available).  Solvers of
+// several threads may ask at the same time: the second waits for the first's answer.
 constexpr int MGC_SMEM = 226 * 1024;
 template <typename T, typename MT, int CLS>
 int mgc_setup(int dev)
 {
+    static std::mutex lock;
     static int size[64] = {};
+    const std::lock_guard<std::mutex> held(lock);
     int& r = size[dev & 63];
     if (r != 0) return r < 0 ? 0 : r;
     const void* k = (const void*)mg_coarse_kernel<T, MT, CLS>;
