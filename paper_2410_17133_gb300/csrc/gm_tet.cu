@@ -16,6 +16,7 @@
 //   C:    y_a = (k/mu) V g_a . sum_b g_b p_b
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <functional>
 #include <string>
 #include <unordered_map>
@@ -226,11 +227,13 @@ namespace {
 // Assemble the operators once mesh and materials are there (structure per mesh,
 // values per material).  Rows that would take more than half of the free device
 // memory, or an allocation that fails, leave csr_ready false: products then
-// walk the elements.
+// walk the elements, as they do with GM_TET_ROWS=0.
 void tet_assemble(gm_tet* t)
 {
     t->csr_ready = false;
     if (!t->has_mesh || !t->has_mat) return;
+    const char* wanted = std::getenv("GM_TET_ROWS");
+    if (wanted && std::atoi(wanted) == 0) return;
     cudaSetDevice(t->device);
     const int N = (int)t->N;
     const unsigned wblocks = (unsigned)((N + 3) / 4);
