@@ -73,7 +73,11 @@ int gm_tet_surface_load(gm_tet* t, const int64_t* tris_host, int64_t n_tris, dou
  * Solved by Prevost's partitioned CG (Sec. 3.3.2): CG on the Schur complement
  * (S + dt C) + A^T K^-1 A, preconditioned by the diagonal of S + dt C,
  * relative tolerance rtol; inner K solves by PCG with 3x3 nodal block Jacobi
- * to rtol/100, their scalars kept on the device.  FP64.  report: outer iterations and final relative residual.
+ * to rtol/100, their scalars kept on the device.  Meshes whose rows fit the SMs'
+ * shared memory (about 20 k nodes) run a K solve as one cooperative launch; with
+ * GM_TET_GRID=0, read with the mesh, or where such a launch is refused or one of its
+ * bounded waits runs out (GM_TET_GRID_POLLS), as two launches per iteration.
+ * FP64.  report: outer iterations and final relative residual.
  * GM_ENOCONV if an iteration limit (maxit) is reached.  Synchronises. */
 int gm_tet_step(gm_tet* t, double dt, double* u_dev, double* p_dev, double rtol, int maxit,
                 gm_solve_report* report_host, void* stream);

@@ -581,10 +581,14 @@ struct Stepper {
     // x = K^-1 b (x from 0), PCG with 3x3 nodal block Jacobi to ||r|| <= rtol ||b||,
     // device-resident (scratch 0-3, 14 and 15)
     int solve_k(const double* b, double* x, double rtol, int maxit, long long* its) {
-        const int rc = t->csr_ready && t->grid_rows ? solve_k_grid(b, x, rtol, maxit, its) : solve_k_loop(b, x, rtol, maxit, its);
+        int rc = 5;
+        if (t->csr_ready && t->grid_rows) {
+            rc = solve_k_grid(b, x, rtol, maxit, its);
+            if (rc == 5) t->grid_rows = 0;       // not on this device as it is now: two launches until the next mesh
+        }
+        if (rc == 5) rc = solve_k_loop(b, x, rtol, maxit, its);
         if (rc == 2) return t->set_err(GM_ENAN, "tet step: K not positive on a direction");
         if (rc == 3) return t->set_err(GM_ENOCONV, "tet step: K solve did not converge");
-        if (rc == 5) return t->set_err(GM_ECUDA, "tet step: the solve's blocks waited for one another too long");
         if (rc < 0) return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(cudaGetLastError()));
         return GM_OK;
     }
@@ -592,7 +596,7 @@ struct Stepper {
         return tgrid_solve(TetGridArgs{N, t->grid_rows, maxit, rtol * rtol, t->crow.as<int>(), t->ccol.as<int>(),
                                        t->cK64.as<double>(), t->Kinv.as<double>(), t->mask.as<uint8_t>(), b, x,
                                        t->w[2].as<double>(), t->grid_box.as<ulonglong2>(),
-                                       t->pcg_st.as<TetPcgState>()},
+                                       t->pcg_st.as<TetPcgState>(), tgrid_polls()},
                            t->grid_ctas, t->grid_smem, s, its);
     }
     int solve_k_loop(const double* b, double* x, double rtol, int maxit, long long* its) {

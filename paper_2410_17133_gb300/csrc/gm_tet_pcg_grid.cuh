@@ -16,7 +16,8 @@
 // An unwritten word of a box holds the bit pattern GRID_EMPTY (a NaN that no sum
 // is stored as); three sets of words take turns.  Waits are bounded: a CTA that
 // gives up marks the solve and returns, and so do the others.  The launch is
-// cooperative, so all CTAs are resident.
+// cooperative, so all CTAs are resident.  Where the launch is refused or a wait
+// runs out, the caller solves with two launches per iteration instead.
 // Included by gm_tet.cu only.
 #pragma once
 
@@ -31,7 +32,7 @@ constexpr int TGRID_MIN_ROWS = 16;                    // fewer do not fill the f
 constexpr int TGRID_CTAS = 256;
 constexpr size_t TGRID_SMEM = 208 * 1024;              // beside 12 KB of row vectors
 constexpr unsigned long long GRID_EMPTY = ~0ull;
-constexpr int TGRID_SPIN = 1 << 23;                   // polls of an L2 word: some seconds
+constexpr int TGRID_POLLS = 1 << 23;                  // polls of an L2 word before a wait runs out: some seconds
 constexpr int TGRID_LOST = -1;
 inline size_t tgrid_box_bytes(int grid) { return (size_t)grid * 3 * TGRID_CTAS * sizeof(ulonglong2); }
 
@@ -48,6 +49,7 @@ struct TetGridArgs {
     double* z;                           // 3N: (z0, z1) of each node, then all z2
     ulonglong2* box;                     // per CTA 3 sets of TGRID_CTAS partials; empty at the start
     TetPcgState* st;
+    int polls;
 };
 
 // entries of a CTA: 9 of K, 3 of the direction, the column
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(TGRID_NT, 1) tet_pcg_grid(const TetGridArgs a)
                 got[j].x = got[j].y = 32 * j + lane < G ? GRID_EMPTY : 0ull;
             }
             bool wait = true;
-            for (int spin = 0; wait && spin < TGRID_SPIN; ++spin) {
+            for (int spin = 0; wait && spin < a.polls; ++spin) {
 #pragma unroll
                 for (int j = 0; j < PER; ++j)
                     if (got[j].x == GRID_EMPTY || got[j].y == GRID_EMPTY) got[j] = tgrid_load(from + 32 * j);
@@ -332,9 +334,11 @@ __global__ void __launch_bounds__(TGRID_NT, 1) tet_pcg_grid(const TetGridArgs a)
 
 // Node rows per CTA for the mesh, 0 where the solve keeps its two launches per
 // iteration: rows that do not fit (more FP64 work than latency by then), or a
-// device without cooperative launches.  crow: N + 1 row starts.
+// device without cooperative launches, or GM_TET_GRID=0.  crow: N + 1 row starts.
 inline int tgrid_plan(int device, int N, const std::vector<int>& crow, size_t& smem, int& grid)
 {
+    const char* wanted = std::getenv("GM_TET_GRID");
+    if (wanted && std::atoi(wanted) == 0) return 0;
     int sms = 0, coop = 0, occ = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop) {
@@ -357,8 +361,16 @@ inline int tgrid_plan(int device, int N, const std::vector<int>& crow, size_t& s
     return rows;
 }
 
-// x = K^-1 b on the stream; 0, 2 / 3 (breakdown / iteration limit), 5 (a wait
-// between the CTAs ran out) or -1 (CUDA error); *its += iterations
+// polls of a wait: GM_TET_GRID_POLLS for the tests of what follows when one runs out
+inline int tgrid_polls()
+{
+    const char* v = std::getenv("GM_TET_GRID_POLLS");
+    const int n = v ? std::atoi(v) : TGRID_POLLS;
+    return n < 0 ? 0 : n < TGRID_POLLS ? n : TGRID_POLLS;
+}
+
+// x = K^-1 b on the stream; 0, 2 / 3 (breakdown / iteration limit), 5 (not solved: the
+// launch was refused or a wait between the CTAs ran out) or -1 (CUDA error); *its += iterations
 inline int tgrid_solve(const TetGridArgs& a, int grid, size_t smem, cudaStream_t s, long long* its)
 {
     if (cudaMemsetAsync(a.box, 0xff, tgrid_box_bytes(grid), s) != cudaSuccess ||
@@ -366,14 +378,16 @@ inline int tgrid_solve(const TetGridArgs& a, int grid, size_t smem, cudaStream_t
         return -1;
     TetGridArgs copy = a;
     void* args[] = {&copy};
-    if (cudaLaunchCooperativeKernel((const void*)tet_pcg_grid, dim3(grid), dim3(TGRID_NT), args, smem, s) != cudaSuccess)
-        return -1;
+    if (cudaLaunchCooperativeKernel((const void*)tet_pcg_grid, dim3(grid), dim3(TGRID_NT), args, smem, s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 5;
+    }
     TetPcgState h;
     if (cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
-    *its += h.its;
     if (h.ticket != 0u) return 5;
+    *its += h.its;
     return h.done == 1 ? 0 : h.done;
 }
 
