@@ -15,9 +15,11 @@
 //   S:    y_a = (V / 20 M) (sum_b p_b + p_a)
 //   C:    y_a = (k/mu) V g_a . sum_b g_b p_b
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <functional>
+#include <mutex>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -168,8 +170,11 @@ struct gm_tet {
     bool has_mesh = false, has_mat = false;
     double E = 0, nu = 0, alpha = 0, Mb = 0, k = 0, mu_f = 0;
     DBuf G64, G32, V64, V32, tets, rowptr, adj;
-    // assembled rows (gm_tet_csr.cuh); false where they do not fit the device
+    // assembled rows (gm_tet_csr.cuh); false where they do not fit the device.  Their
+    // FP32 copies are made by the first FP32 product (1 made, -1 no room for them)
     bool csr_ready = false;
+    std::atomic<int> csr32{0};
+    std::mutex csr32_lock;
     long long nnz = 0;
     int grid_rows = 0, grid_ctas = 0;       // one-launch PCG (gm_tet_pcg_grid.cuh): rows per CTA, 0: not used
     size_t grid_smem = 0;
@@ -224,6 +229,85 @@ struct gm_tet {
 
 namespace {
 
+// The context's device for the length of a scope.
+struct OnDevice {
+    int before = -1;
+    explicit OnDevice(int d)
+    {
+        if (cudaGetDevice(&before) != cudaSuccess) before = -1;
+        cudaSetDevice(d);
+    }
+    ~OnDevice() { if (before >= 0) cudaSetDevice(before); }
+};
+
+// Gives the rows' memory back; products then walk the elements.  False if there was none.
+bool tet_drop_rows(gm_tet* t)
+{
+    DBuf* const rows[] = {&t->crow, &t->ccol, &t->cK64, &t->cA64, &t->cSC64, &t->cK32, &t->cA32, &t->cSC32};
+    bool any = false;
+    for (DBuf* b : rows) any = any || b->p;
+    t->csr_ready = false;
+    t->csr32 = 0;
+    t->nnz = 0;
+    if (!any) return false;
+    cudaDeviceSynchronize();      // products in flight may read them
+    t->drop_graphs();
+    for (DBuf* b : rows) b->drop();
+    (void)cudaGetLastError();
+    return true;
+}
+
+// Runs place(), the allocations of a call; where they find no memory, once more
+// without the rows.
+template <class Place>
+cudaError_t tet_place(gm_tet* t, Place&& place)
+{
+    cudaError_t e = place();
+    if (e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    return tet_drop_rows(t) ? place() : e;
+}
+
+// Room for `bytes` more of rows: half of the free device memory at most.
+bool tet_row_room(double bytes)
+{
+    size_t free_b = 0, total_b = 0;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= 0.5 * (double)free_b;
+}
+
+void tet_cast_rows(gm_tet* t, cudaStream_t s)
+{
+    tcsr_cast<<<608, 256, 0, s>>>(9 * t->nnz, t->cK64.as<double>(), t->cK32.as<float>());
+    tcsr_cast<<<608, 256, 0, s>>>(6 * t->nnz, t->cA64.as<double>(), t->cA32.as<float>());
+    tcsr_cast<<<608, 256, 0, s>>>(2 * t->nnz, t->cSC64.as<double>(), t->cSC32.as<float>());
+}
+
+// The rows in FP32, made on first use (on a stream of their own: the caller's may be
+// capturing); false where they have no room.
+bool tet_rows32(gm_tet* t)
+{
+    if (t->csr32 != 0) return t->csr32 > 0;
+    const std::lock_guard<std::mutex> held(t->csr32_lock);
+    if (t->csr32 != 0) return t->csr32 > 0;
+    OnDevice on(t->device);
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaStream_t s = nullptr;
+    bool ok = tet_row_room(68.0 * t->nnz) && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && t->cK32.alloc(t->nnz * 36) == cudaSuccess && t->cA32.alloc(t->nnz * 24) == cudaSuccess &&
+         t->cSC32.alloc(t->nnz * 8) == cudaSuccess;
+    if (ok) tet_cast_rows(t, s);
+    ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
+    if (s) cudaStreamDestroy(s);
+    if (!ok) {
+        (void)cudaGetLastError();
+        for (DBuf* b : {&t->cK32, &t->cA32, &t->cSC32}) b->drop();
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    t->csr32 = ok ? 1 : -1;
+    return ok;
+}
+
 // Assemble the operators once mesh and materials are there (structure per mesh,
 // values per material).  Rows that would take more than half of the free device
 // memory, or an allocation that fails, leave csr_ready false: products then
@@ -232,16 +316,18 @@ void tet_assemble(gm_tet* t)
 {
     t->csr_ready = false;
     if (!t->has_mesh || !t->has_mat) return;
+    OnDevice on(t->device);
     const char* wanted = std::getenv("GM_TET_ROWS");
-    if (wanted && std::atoi(wanted) == 0) return;
-    cudaSetDevice(t->device);
+    if (wanted && std::atoi(wanted) == 0) {
+        tet_drop_rows(t);
+        return;
+    }
     const int N = (int)t->N;
     const unsigned wblocks = (unsigned)((N + 3) / 4);
     DBuf count, rows;
     auto give_up = [&]() {
         (void)cudaGetLastError();
-        t->nnz = 0;
-        for (DBuf* b : {&t->crow, &t->ccol, &t->cK64, &t->cA64, &t->cSC64, &t->cK32, &t->cA32, &t->cSC32}) b->drop();
+        tet_drop_rows(t);
     };
     cudaDeviceSynchronize();      // products in flight may read the arrays that change below
     if (t->nnz == 0) {
@@ -252,15 +338,11 @@ void tet_assemble(gm_tet* t)
         if (cudaMemcpy(h.data() + 1, count.p, (size_t)N * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return give_up();
         long long nnz = 0;
         for (int n = 0; n < N; ++n) nnz += h[n + 1];
-        size_t free_b = 0, total_b = 0;
-        if (nnz >= (1LL << 31) - 1 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
-            (double)nnz * (17 * 12 + 8) > 0.5 * (double)free_b)
-            return give_up();
+        if (nnz >= (1LL << 31) - 1 || !tet_row_room(144.0 * nnz)) return give_up();
         for (int n = 0; n < N; ++n) h[n + 1] += h[n];
         if (t->crow.put(h.data(), h.size() * 4) != cudaSuccess || t->ccol.alloc(nnz * 4) != cudaSuccess ||
             t->cK64.alloc(nnz * 72) != cudaSuccess || t->cA64.alloc(nnz * 48) != cudaSuccess ||
-            t->cSC64.alloc(nnz * 16) != cudaSuccess || t->cK32.alloc(nnz * 36) != cudaSuccess ||
-            t->cA32.alloc(nnz * 24) != cudaSuccess || t->cSC32.alloc(nnz * 8) != cudaSuccess)
+            t->cSC64.alloc(nnz * 16) != cudaSuccess)
             return give_up();
         t->grid_rows = tgrid_plan(t->device, N, h, t->grid_smem, t->grid_ctas);
         t->nnz = nnz;
@@ -275,9 +357,7 @@ void tet_assemble(gm_tet* t)
                                                         t->ccol.as<int>(), rows.as<int>(), lam, mu, t->alpha,
                                                         1.0 / t->Mb, t->k / t->mu_f, t->cK64.as<double>(),
                                                         t->cA64.as<double>(), t->cSC64.as<double>());
-    tcsr_cast<<<608, 256>>>(9 * nnz, t->cK64.as<double>(), t->cK32.as<float>());
-    tcsr_cast<<<608, 256>>>(6 * nnz, t->cA64.as<double>(), t->cA32.as<float>());
-    tcsr_cast<<<608, 256>>>(2 * nnz, t->cSC64.as<double>(), t->cSC32.as<float>());
+    if (t->csr32 > 0) tet_cast_rows(t, 0);
     if (cudaDeviceSynchronize() != cudaSuccess) return give_up();
     t->csr_ready = true;
 }
@@ -365,6 +445,7 @@ int gm_tet_mesh(gm_tet* t, const double* nodes, int64_t n_nodes, const int64_t* 
         for (int b = 0; b < 4; ++b) adj[fill[tv[4 * e + b]]++] = (int)(4 * e + b);
     std::vector<float> G32(G.begin(), G.end()), V32(V.begin(), V.end());
     cudaSetDevice(t->device);
+    tet_drop_rows(t);             // of the mesh before: the new one takes their place
     cudaError_t ce;
     if ((ce = t->G64.put(G.data(), G.size() * 8)) != cudaSuccess || (ce = t->G32.put(G32.data(), G32.size() * 4)) != cudaSuccess ||
         (ce = t->V64.put(V.data(), V.size() * 8)) != cudaSuccess || (ce = t->V32.put(V32.data(), V32.size() * 4)) != cudaSuccess ||
@@ -385,7 +466,6 @@ int gm_tet_mesh(gm_tet* t, const double* nodes, int64_t n_nodes, const int64_t* 
     t->has_fault = false;
     t->fault_ready = false;
     t->has_mesh = true;
-    t->nnz = 0;
     tet_assemble(t);
     return GM_OK;
 }
@@ -421,7 +501,7 @@ void launch(gm_tet* t, const TetCoef<T>& c, const T* xu, const T* xp, T* yu, T* 
             const T* V, const int* skip)
 {
     const int N = (int)t->N;
-    if (t->csr_ready) {
+    if (t->csr_ready && (sizeof(T) == 8 || tet_rows32(t))) {
         gm_launch_chained(tcsr_apply<T, MODE, false>, (unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s,
             N, csr<T>(t), c.cApu, c.cC, xu, xp, yu, yp, skip, TetDir<T>{});
         return;
@@ -665,17 +745,20 @@ int tet_prepare(gm_tet* t)
     std::vector<double> fu = t->fu;
     for (long long i = 0; i < 3 * N; ++i)
         if (t->fixed[i]) fu[i] = 0.0;
-    cudaError_t ce;
-    if ((ce = t->Kinv.put(Kinv.data(), Kinv.size() * 8)) != cudaSuccess || (ce = t->Sd.put(Sd.data(), N * 8)) != cudaSuccess ||
-        (ce = t->Cd.put(Cd.data(), N * 8)) != cudaSuccess || (ce = t->mask.put(mk.data(), N)) != cudaSuccess ||
-        (ce = t->dfu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (ce = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
-        (t->grid_rows && (ce = t->grid_box.alloc(tgrid_box_bytes(t->grid_ctas))) != cudaSuccess) ||
-        (ce = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
-        (ce = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
-        return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(ce));
-    for (auto& b : t->w)
-        if ((ce = b.alloc(3 * N * 8)) != cudaSuccess)
-            return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(ce));
+    const cudaError_t ce = tet_place(t, [&]() {
+        cudaError_t e;
+        if ((e = t->Kinv.put(Kinv.data(), Kinv.size() * 8)) != cudaSuccess || (e = t->Sd.put(Sd.data(), N * 8)) != cudaSuccess ||
+            (e = t->Cd.put(Cd.data(), N * 8)) != cudaSuccess || (e = t->mask.put(mk.data(), N)) != cudaSuccess ||
+            (e = t->dfu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (e = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
+            (t->csr_ready && t->grid_rows && (e = t->grid_box.alloc(tgrid_box_bytes(t->grid_ctas))) != cudaSuccess) ||
+            (e = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
+            (e = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
+            return e;
+        for (auto& b : t->w)
+            if ((e = b.alloc(3 * N * 8)) != cudaSuccess) return e;
+        return cudaSuccess;
+    });
+    if (ce != cudaSuccess) return t->set_err(GM_ECUDA, std::string("tet step: ") + cudaGetErrorString(ce));
     t->prec_ready = true;
     return GM_OK;
 }
@@ -1149,25 +1232,27 @@ int tetf_prepare(gm_tet* t)
             }
         }
     t->f0sq = f0;
-    cudaError_t ce;
-    if ((ce = t->f_Kblk.put(B.data(), B.size() * 8)) != cudaSuccess || (ce = t->f_Kinv.alloc(9 * N * 8)) != cudaSuccess ||
-        (ce = t->f_fu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (ce = t->f_fpv.put(fpv.data(), N * 8)) != cudaSuccess ||
-        (ce = t->f_Sd.put(Sd.data(), N * 8)) != cudaSuccess || (ce = t->f_Cd.put(Cd.data(), N * 8)) != cudaSuccess ||
-        (ce = t->f_dKm.put(dKm.data(), 3 * N * 8)) != cudaSuccess ||
-        (ce = t->f_invdK.put(invdK.data(), 3 * N * 8)) != cudaSuccess || (ce = t->f_dAm.alloc(N * 8)) != cudaSuccess ||
-        (ce = t->f_invdA.alloc(N * 8)) != cudaSuccess || (ce = t->f_mask.put(mk.data(), N)) != cudaSuccess ||
-        (ce = t->f_err.alloc(sizeof(int))) != cudaSuccess || (ce = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
-        (ce = t->f_Pinv.alloc(36 * P * 8)) != cudaSuccess || (ce = t->f_Pinv32.alloc(36 * P * 4)) != cudaSuccess ||
-        (ce = t->f_Kinv32.alloc(9 * N * 4)) != cudaSuccess || (ce = t->f_D32.alloc(6 * P * 4)) != cudaSuccess ||
-        (ce = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
-        (ce = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
-        return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
-    for (auto& b : t->fw)
-        if ((ce = b.alloc(3 * N * 8)) != cudaSuccess)
-            return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
-    for (auto& b : t->fw32)
-        if ((ce = b.alloc(3 * N * 4)) != cudaSuccess)
-            return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
+    const cudaError_t ce = tet_place(t, [&]() {
+        cudaError_t e;
+        if ((e = t->f_Kblk.put(B.data(), B.size() * 8)) != cudaSuccess || (e = t->f_Kinv.alloc(9 * N * 8)) != cudaSuccess ||
+            (e = t->f_fu.put(fu.data(), 3 * N * 8)) != cudaSuccess || (e = t->f_fpv.put(fpv.data(), N * 8)) != cudaSuccess ||
+            (e = t->f_Sd.put(Sd.data(), N * 8)) != cudaSuccess || (e = t->f_Cd.put(Cd.data(), N * 8)) != cudaSuccess ||
+            (e = t->f_dKm.put(dKm.data(), 3 * N * 8)) != cudaSuccess ||
+            (e = t->f_invdK.put(invdK.data(), 3 * N * 8)) != cudaSuccess || (e = t->f_dAm.alloc(N * 8)) != cudaSuccess ||
+            (e = t->f_invdA.alloc(N * 8)) != cudaSuccess || (e = t->f_mask.put(mk.data(), N)) != cudaSuccess ||
+            (e = t->f_err.alloc(sizeof(int))) != cudaSuccess || (e = t->part.alloc(TET_RED_BLOCKS * 8)) != cudaSuccess ||
+            (e = t->f_Pinv.alloc(36 * P * 8)) != cudaSuccess || (e = t->f_Pinv32.alloc(36 * P * 4)) != cudaSuccess ||
+            (e = t->f_Kinv32.alloc(9 * N * 4)) != cudaSuccess || (e = t->f_D32.alloc(6 * P * 4)) != cudaSuccess ||
+            (e = t->pcg_st.alloc(sizeof(TetPcgState))) != cudaSuccess ||
+            (e = t->pcg_part.alloc(pcg_part_bytes(t))) != cudaSuccess)
+            return e;
+        for (auto& b : t->fw)
+            if ((e = b.alloc(3 * N * 8)) != cudaSuccess) return e;
+        for (auto& b : t->fw32)
+            if ((e = b.alloc(3 * N * 4)) != cudaSuccess) return e;
+        return cudaSuccess;
+    });
+    if (ce != cudaSuccess) return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
     t->fault_ready = true;
     return GM_OK;
 }
@@ -1279,6 +1364,7 @@ struct FStepper {
         double* part = t->pcg_part.as<double>();
         const uint8_t* mk = t->f_mask.as<uint8_t>();
         if (f32) {
+            if (t->csr_ready) tet_rows32(t);         // before the iterations are captured
             float* v[5];
             for (int k = 0; k < 5; ++k) v[k] = t->fw32[k].as<float>();
             TetPcg<float> e{N, s, v[0], v[1], v[2], v[3], v[4], ps, part,
@@ -1511,21 +1597,25 @@ extern "C" int gm_tet_fault(gm_tet* t, const int64_t* pairs, int64_t n_pairs, co
     cudaSetDevice(t->device);
     std::vector<double> zero2(2 * P, 0.0);
     std::vector<int8_t> stick(P, (int8_t)GM_STICK);
-    cudaError_t ce;
-    if ((ce = t->f_pm.put(pm.data(), P * 4)) != cudaSuccess || (ce = t->f_pp.put(pp.data(), P * 4)) != cudaSuccess ||
-        (ce = t->f_n2p.put(n2p.data(), N * 4)) != cudaSuccess || (ce = t->f_area.put(area.data(), P * 8)) != cudaSuccess ||
-        (ce = t->f_fr.put(fr.data(), 9 * P * 8)) != cudaSuccess || (ce = t->f_Lt.put(Lt.data(), 9 * NT * 8)) != cudaSuccess ||
-        (ce = t->f_tri.put(tri.data(), 3 * NT * 4)) != cudaSuccess ||
-        (ce = t->f_prow.put(cnt.data(), (P + 1) * 4)) != cudaSuccess ||
-        (ce = t->f_padj.put(padj.data(), 3 * NT * 4)) != cudaSuccess ||
-        (ce = t->f_dlie_n.put(zero2.data(), 2 * P * 8)) != cudaSuccess || (ce = t->f_dlie.alloc(2 * P * 8)) != cudaSuccess ||
-        (ce = t->f_state.alloc(P)) != cudaSuccess || (ce = t->f_T.alloc(3 * P * 8)) != cudaSuccess ||
-        (ce = t->f_D.put(std::vector<double>(6 * P, 0.0).data(), 6 * P * 8)) != cudaSuccess ||
-        (ce = t->f_tn.alloc(P * 8)) != cudaSuccess || (ce = t->f_F.alloc(P * 8)) != cudaSuccess ||
-        (ce = t->f_dn.alloc(P * 8)) != cudaSuccess || (ce = t->f_gs.alloc(2 * P * 8)) != cudaSuccess ||
-        (ce = t->f_flags_acc.put(stick.data(), P)) != cudaSuccess ||
-        (ce = t->f_gs_acc.put(zero2.data(), 2 * P * 8)) != cudaSuccess)
-        return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
+    const cudaError_t ce = tet_place(t, [&]() {
+        cudaError_t e;
+        if ((e = t->f_pm.put(pm.data(), P * 4)) != cudaSuccess || (e = t->f_pp.put(pp.data(), P * 4)) != cudaSuccess ||
+            (e = t->f_n2p.put(n2p.data(), N * 4)) != cudaSuccess || (e = t->f_area.put(area.data(), P * 8)) != cudaSuccess ||
+            (e = t->f_fr.put(fr.data(), 9 * P * 8)) != cudaSuccess || (e = t->f_Lt.put(Lt.data(), 9 * NT * 8)) != cudaSuccess ||
+            (e = t->f_tri.put(tri.data(), 3 * NT * 4)) != cudaSuccess ||
+            (e = t->f_prow.put(cnt.data(), (P + 1) * 4)) != cudaSuccess ||
+            (e = t->f_padj.put(padj.data(), 3 * NT * 4)) != cudaSuccess ||
+            (e = t->f_dlie_n.put(zero2.data(), 2 * P * 8)) != cudaSuccess || (e = t->f_dlie.alloc(2 * P * 8)) != cudaSuccess ||
+            (e = t->f_state.alloc(P)) != cudaSuccess || (e = t->f_T.alloc(3 * P * 8)) != cudaSuccess ||
+            (e = t->f_D.put(std::vector<double>(6 * P, 0.0).data(), 6 * P * 8)) != cudaSuccess ||
+            (e = t->f_tn.alloc(P * 8)) != cudaSuccess || (e = t->f_F.alloc(P * 8)) != cudaSuccess ||
+            (e = t->f_dn.alloc(P * 8)) != cudaSuccess || (e = t->f_gs.alloc(2 * P * 8)) != cudaSuccess ||
+            (e = t->f_flags_acc.put(stick.data(), P)) != cudaSuccess ||
+            (e = t->f_gs_acc.put(zero2.data(), 2 * P * 8)) != cudaSuccess)
+            return e;
+        return cudaSuccess;
+    });
+    if (ce != cudaSuccess) return t->set_err(GM_ECUDA, std::string("tet fault: ") + cudaGetErrorString(ce));
     t->P = P;
     t->NTRI = NT;
     t->fpar = *fp;

@@ -113,3 +113,47 @@ def test_a_refused_cooperative_launch_leaves_the_solve_to_the_launches(host):
     host.refuse_cooperative(1)
     assert t.step() == 0
     assert n1 == n0 and host.launched() > n1            # one launch first, captured iterations then
+
+
+def test_rows_make_room_for_the_vectors_of_a_step(host):
+    """With a byte less than rows and vectors take together, the step still has its vectors."""
+    start = host.in_use()
+    t = Tet(host, 2)
+    assert t.materials() == 0 and t.step() == 0
+    whole = host.in_use() - start
+    host.gm_tet_destroy(t.h)
+    assert host.in_use() == start
+    t = Tet(host, 2)
+    host.set_limit(start + whole - 1)
+    assert t.materials() == 0
+    with_rows = host.in_use()
+    assert t.step() == 0 and t.step() == 0
+    rows = 15 * 8 * 140                                     # 15 entries at 8 nodes
+    assert with_rows - start > rows and host.in_use() - start < whole - rows
+    assert t.materials(2e9) == 0 and t.step() == 0
+    host.gm_tet_destroy(t.h)
+    assert host.in_use() == start
+
+
+def test_single_precision_rows_come_with_the_first_product_in_it(host):
+    t = Tet(host, 8)
+    assert t.materials() == 0
+    x = np.zeros(4 * 32)
+    apply = lambda dtype: host.gm_tet_apply(t.h, 0, ctypes.c_void_p(x.ctypes.data), ctypes.c_void_p(x.ctypes.data),
+                                            ctypes.c_double(1.0), dtype, None)
+    used = [host.in_use()]
+    for dtype in (0, 0, 1, 1):
+        assert apply(dtype) == 0
+        used.append(host.in_use())
+    assert used[0] == used[1] == used[2] and used[3] == used[4] == used[0] + 15 * 32 * 68
+    assert t.materials(2e9) == 0 and host.in_use() == used[4]
+    host.gm_tet_destroy(t.h)
+
+
+def test_materials_leave_the_device_of_the_caller(host):
+    t = Tet(host)
+    host.cudaSetDevice(5)
+    assert t.materials() == 0
+    d = ctypes.c_int()
+    host.cudaGetDevice(ctypes.byref(d))
+    assert d.value == 5
