@@ -515,10 +515,15 @@ int smooth(gm_ctx* c, const MGLevel& L, int deg, bool xzero, const int* skip, cu
     return GM_OK;
 }
 
-// The coarsest level's polynomial as one cluster kernel where that is the faster
-// way: its rows fit the CTAs' shared memory, the smoother's pair threads add the
-// fault rows, and a CTA has few elements (FP32: 4,096, FP64: 1,024; beyond, a product spread over all
-// SMs wins).  Called at set-up: it sets kernel attributes, outside any capture.
+// The coarsest level's polynomial as one cluster kernel where its rows fit the CTAs'
+// shared memory (FP64: about 200 cells in x and z with two rows a CTA, FP32: 500) and the
+// smoother's pair threads add the fault rows.  It is the faster way wherever it fits; us per
+// K_T iteration, one kernel against launches, with its element products per CTA:
+//   FP64 12^3 (288) 457 / 680, 14^3 (392) 539 / 784, 18x14x18 (648) 733 / 799,
+//        12x30x12 (576) 681 / 819, 10x46x10 (600) 710 / 765;
+//   FP32 12^3 (288) 329 / 519, 16^3 (1024) 344 / 549, 18^3 (1296) 378 / 540,
+//        20x30x20 (1600) 444 / 653, 10x126x10 (1600) 479 / 605.
+// Called at set-up: it sets kernel attributes, outside any capture.
 template <typename T, int CLS>
 int coarse_cluster(gm_ctx* x)
 {
@@ -535,8 +540,7 @@ int coarse_cluster(gm_ctx* x)
     if (mgc_layout<T, MT>(x->g, rows).total > MGC_SMEM) return 0;
     const long long rn = (long long)(x->nx + 1) * x->g.nplanes, faces = (long long)x->nx * x->nz;
     if (rn * 3 * (rows + 2) >= 65536 || faces * 6 * rows >= 65536) return 0;     // quotients by multiplication
-    const long long work = 2LL * rows * faces;
-    return work <= (sizeof(T) == 8 ? 1024 : 4096) ? n : 0;
+    return n;
 }
 template <typename T>
 int coarse_cluster(gm_ctx* x)
