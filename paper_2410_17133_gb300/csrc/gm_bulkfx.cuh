@@ -216,7 +216,7 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
                     const unsigned m = a.mask[node];
 #pragma unroll
                     for (int f = 0; f < NI; ++f) {
-                        const int hi = __ldg(reinterpret_cast<const int*>(xin + (long long)f * N + node) + 1) & 0x7fffffff;
+                        const int hi = reinterpret_cast<const int*>(xin + (long long)f * N + node)[1] & 0x7fffffff;
                         if (!((m >> (IN_P ? 3 : f)) & 1u)) {
                             m4 = max(m4, hi);
                             if (hi != 0) least = min(least, hi);

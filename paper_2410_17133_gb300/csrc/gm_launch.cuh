@@ -8,8 +8,10 @@
 // A kernel launched this way takes `chained` first and calls gm_chain(chained)
 // before it touches global memory, in every thread and on every path, so
 // completion is transitive along the chain: a kernel cannot complete before its
-// predecessors have.  Kernels in between that are launched normally wait for
-// completion as usual.  Measured, chained against plain launches: outside graphs
+// predecessors have.  Its loads are coherent ones: the kernel is already there while
+// its predecessor writes, so nothing that it reads is read-only for its lifetime, and
+// a non-coherent load (__ldg, __restrict__) could be served or moved ahead of the wait.
+// Kernels in between that are launched normally wait for completion as usual.  Measured, chained against plain launches: outside graphs
 // J on 8^3 cells 46.8 -> 43 us, five tetrahedral products 103 -> 94.5 us, the
 // FP32 products at 160^3 551 -> 533 us; in captured graphs it loses (FP32 step at
 // 64^3 84 -> 89 ms, FP64 K_T solve at 48^3 60.5 -> 66.8 ms), so there the launches
