@@ -42,10 +42,10 @@ int gm_tet_mesh(gm_tet* t, const double* nodes_host, int64_t n_nodes, const int6
 /* Homogeneous materials (Sec. 2.1): Young's modulus E, Poisson ratio nu, Biot
  * coefficient alpha, Biot modulus M, permeability k, fluid viscosity mu_f.
  * With mesh and materials set, the operators are assembled into block rows on
- * the device where these fit half of its free memory (about 2.2 kB per node, and
- * 1 kB from the first FP32 product on); products walk the elements otherwise, and
- * with the environment variable GM_TET_ROWS=0, read when either is set.  Where a
- * later call finds no memory for its vectors, the rows make room.  Synchronises. */
+ * the device where these fit half of its free memory (about 3 kB per node);
+ * products walk the elements otherwise, and with the environment variable
+ * GM_TET_ROWS=0, read when either is set.  Where a later call finds no memory for
+ * its vectors, the rows make room.  Synchronises. */
 int gm_tet_materials(gm_tet* t, double E, double nu, double alpha, double M, double k, double mu_f);
 
 /* y = A x for `which` in GM_OP_KB (= GM_OP_KT: no fault), GM_OP_APU, GM_OP_AUP,

@@ -15,11 +15,9 @@
 //   S:    y_a = (V / 20 M) (sum_b p_b + p_a)
 //   C:    y_a = (k/mu) V g_a . sum_b g_b p_b
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <functional>
-#include <mutex>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -170,11 +168,9 @@ struct gm_tet {
     bool has_mesh = false, has_mat = false;
     double E = 0, nu = 0, alpha = 0, Mb = 0, k = 0, mu_f = 0;
     DBuf G64, G32, V64, V32, tets, rowptr, adj;
-    // assembled rows (gm_tet_csr.cuh); false where they do not fit the device.  Their
-    // FP32 copies are made by the first FP32 product (1 made, -1 no room for them)
+    // assembled rows (gm_tet_csr.cuh); false where they do not fit the device
     bool csr_ready = false;
-    std::atomic<int> csr32{0};
-    std::mutex csr32_lock;
+    bool rows_captured = false;             // a caller's graph holds products by these rows
     long long nnz = 0;
     int grid_rows = 0, grid_ctas = 0;       // one-launch PCG (gm_tet_pcg_grid.cuh): rows per CTA, 0: not used
     size_t grid_smem = 0;
@@ -240,14 +236,15 @@ struct OnDevice {
     ~OnDevice() { if (before >= 0) cudaSetDevice(before); }
 };
 
-// Gives the rows' memory back; products then walk the elements.  False if there was none.
+// Gives the rows' memory back; products then walk the elements.  False if there was
+// none, or if a caller's graph holds it: that stays good until the next mesh.
 bool tet_drop_rows(gm_tet* t)
 {
     DBuf* const rows[] = {&t->crow, &t->ccol, &t->cK64, &t->cA64, &t->cSC64, &t->cK32, &t->cA32, &t->cSC32};
     bool any = false;
     for (DBuf* b : rows) any = any || b->p;
     t->csr_ready = false;
-    t->csr32 = 0;
+    if (t->rows_captured) return false;
     t->nnz = 0;
     if (!any) return false;
     cudaDeviceSynchronize();      // products in flight may read them
@@ -268,50 +265,11 @@ cudaError_t tet_place(gm_tet* t, Place&& place)
     return tet_drop_rows(t) ? place() : e;
 }
 
-// Room for `bytes` more of rows: half of the free device memory at most.
-bool tet_row_room(double bytes)
-{
-    size_t free_b = 0, total_b = 0;
-    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= 0.5 * (double)free_b;
-}
-
-void tet_cast_rows(gm_tet* t, cudaStream_t s)
-{
-    tcsr_cast<<<608, 256, 0, s>>>(9 * t->nnz, t->cK64.as<double>(), t->cK32.as<float>());
-    tcsr_cast<<<608, 256, 0, s>>>(6 * t->nnz, t->cA64.as<double>(), t->cA32.as<float>());
-    tcsr_cast<<<608, 256, 0, s>>>(2 * t->nnz, t->cSC64.as<double>(), t->cSC32.as<float>());
-}
-
-// The rows in FP32, made on first use (on a stream of their own: the caller's may be
-// capturing); false where they have no room.
-bool tet_rows32(gm_tet* t)
-{
-    if (t->csr32 != 0) return t->csr32 > 0;
-    const std::lock_guard<std::mutex> held(t->csr32_lock);
-    if (t->csr32 != 0) return t->csr32 > 0;
-    OnDevice on(t->device);
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaStream_t s = nullptr;
-    bool ok = tet_row_room(68.0 * t->nnz) && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-    ok = ok && t->cK32.alloc(t->nnz * 36) == cudaSuccess && t->cA32.alloc(t->nnz * 24) == cudaSuccess &&
-         t->cSC32.alloc(t->nnz * 8) == cudaSuccess;
-    if (ok) tet_cast_rows(t, s);
-    ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
-    if (s) cudaStreamDestroy(s);
-    if (!ok) {
-        (void)cudaGetLastError();
-        for (DBuf* b : {&t->cK32, &t->cA32, &t->cSC32}) b->drop();
-    }
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    t->csr32 = ok ? 1 : -1;
-    return ok;
-}
-
 // Assemble the operators once mesh and materials are there (structure per mesh,
 // values per material).  Rows that would take more than half of the free device
 // memory, or an allocation that fails, leave csr_ready false: products then
-// walk the elements, as they do with GM_TET_ROWS=0.
+// walk the elements, as they do with GM_TET_ROWS=0.  Both precisions at once: FP32 copies
+// that the first FP32 product made took it from 56 to 280 us (36^3-cell octant).
 void tet_assemble(gm_tet* t)
 {
     t->csr_ready = false;
@@ -338,11 +296,15 @@ void tet_assemble(gm_tet* t)
         if (cudaMemcpy(h.data() + 1, count.p, (size_t)N * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return give_up();
         long long nnz = 0;
         for (int n = 0; n < N; ++n) nnz += h[n + 1];
-        if (nnz >= (1LL << 31) - 1 || !tet_row_room(144.0 * nnz)) return give_up();
+        size_t free_b = 0, total_b = 0;
+        if (nnz >= (1LL << 31) - 1 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+            (double)nnz * (17 * 12 + 8) > 0.5 * (double)free_b)
+            return give_up();
         for (int n = 0; n < N; ++n) h[n + 1] += h[n];
         if (t->crow.put(h.data(), h.size() * 4) != cudaSuccess || t->ccol.alloc(nnz * 4) != cudaSuccess ||
             t->cK64.alloc(nnz * 72) != cudaSuccess || t->cA64.alloc(nnz * 48) != cudaSuccess ||
-            t->cSC64.alloc(nnz * 16) != cudaSuccess)
+            t->cSC64.alloc(nnz * 16) != cudaSuccess || t->cK32.alloc(nnz * 36) != cudaSuccess ||
+            t->cA32.alloc(nnz * 24) != cudaSuccess || t->cSC32.alloc(nnz * 8) != cudaSuccess)
             return give_up();
         t->grid_rows = tgrid_plan(t->device, N, h, t->grid_smem, t->grid_ctas);
         t->nnz = nnz;
@@ -357,7 +319,9 @@ void tet_assemble(gm_tet* t)
                                                         t->ccol.as<int>(), rows.as<int>(), lam, mu, t->alpha,
                                                         1.0 / t->Mb, t->k / t->mu_f, t->cK64.as<double>(),
                                                         t->cA64.as<double>(), t->cSC64.as<double>());
-    if (t->csr32 > 0) tet_cast_rows(t, 0);
+    tcsr_cast<<<608, 256>>>(9 * nnz, t->cK64.as<double>(), t->cK32.as<float>());
+    tcsr_cast<<<608, 256>>>(6 * nnz, t->cA64.as<double>(), t->cA32.as<float>());
+    tcsr_cast<<<608, 256>>>(2 * nnz, t->cSC64.as<double>(), t->cSC32.as<float>());
     if (cudaDeviceSynchronize() != cudaSuccess) return give_up();
     t->csr_ready = true;
 }
@@ -445,6 +409,7 @@ int gm_tet_mesh(gm_tet* t, const double* nodes, int64_t n_nodes, const int64_t* 
         for (int b = 0; b < 4; ++b) adj[fill[tv[4 * e + b]]++] = (int)(4 * e + b);
     std::vector<float> G32(G.begin(), G.end()), V32(V.begin(), V.end());
     cudaSetDevice(t->device);
+    t->rows_captured = false;
     tet_drop_rows(t);             // of the mesh before: the new one takes their place
     cudaError_t ce;
     if ((ce = t->G64.put(G.data(), G.size() * 8)) != cudaSuccess || (ce = t->G32.put(G32.data(), G32.size() * 4)) != cudaSuccess ||
@@ -501,7 +466,8 @@ void launch(gm_tet* t, const TetCoef<T>& c, const T* xu, const T* xp, T* yu, T* 
             const T* V, const int* skip)
 {
     const int N = (int)t->N;
-    if (t->csr_ready && (sizeof(T) == 8 || tet_rows32(t))) {
+    if (t->csr_ready) {
+        if (s != t->cap_stream && gm_capturing(s)) t->rows_captured = true;
         gm_launch_chained(tcsr_apply<T, MODE, false>, (unsigned)((8LL * N + TPCG_NT - 1) / TPCG_NT), TPCG_NT, 0, s,
             N, csr<T>(t), c.cApu, c.cC, xu, xp, yu, yp, skip, TetDir<T>{});
         return;
@@ -1364,7 +1330,6 @@ struct FStepper {
         double* part = t->pcg_part.as<double>();
         const uint8_t* mk = t->f_mask.as<uint8_t>();
         if (f32) {
-            if (t->csr_ready) tet_rows32(t);         // before the iterations are captured
             float* v[5];
             for (int k = 0; k < 5; ++k) v[k] = t->fw32[k].as<float>();
             TetPcg<float> e{N, s, v[0], v[1], v[2], v[3], v[4], ps, part,

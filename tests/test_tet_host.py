@@ -48,7 +48,7 @@ int cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void*) { copy(d,
 int cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = limit - used; return 0; }
 int cudaDeviceGetAttribute(int* v, int, int) { *v = 152; return 0; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return 0; }
-int cudaStreamIsCapturing(void*, int* s) { *s = 0; return 0; }
+int cudaStreamIsCapturing(void* s, int* c) { *c = s == (void*)8; return 0; }     // stream 8 captures
 int cudaGetDevice(int* d) { *d = device; return 0; }
 int cudaSetDevice(int d) { device = d; return 0; }
 int cudaLaunchCooperativeKernel() { return refused ? 720 : 0; }
@@ -128,26 +128,29 @@ def test_rows_make_room_for_the_vectors_of_a_step(host):
     assert t.materials() == 0
     with_rows = host.in_use()
     assert t.step() == 0 and t.step() == 0
-    rows = 15 * 8 * 140                                     # 15 entries at 8 nodes
+    rows = 15 * 8 * 208                                     # 15 entries at 8 nodes
     assert with_rows - start > rows and host.in_use() - start < whole - rows
     assert t.materials(2e9) == 0 and t.step() == 0
     host.gm_tet_destroy(t.h)
     assert host.in_use() == start
 
 
-def test_single_precision_rows_come_with_the_first_product_in_it(host):
-    t = Tet(host, 8)
+def test_rows_that_a_captured_product_holds_stay(host):
+    """The same, after a product was captured: the step reports the missing memory, and the rows that
+    the caller's graph reads stay until the next mesh."""
+    start = host.in_use()
+    t = Tet(host, 2)
     assert t.materials() == 0
-    x = np.zeros(4 * 32)
-    apply = lambda dtype: host.gm_tet_apply(t.h, 0, ctypes.c_void_p(x.ctypes.data), ctypes.c_void_p(x.ctypes.data),
-                                            ctypes.c_double(1.0), dtype, None)
-    used = [host.in_use()]
-    for dtype in (0, 0, 1, 1):
-        assert apply(dtype) == 0
-        used.append(host.in_use())
-    assert used[0] == used[1] == used[2] and used[3] == used[4] == used[0] + 15 * 32 * 68
-    assert t.materials(2e9) == 0 and host.in_use() == used[4]
+    with_rows = host.in_use()
+    x = np.zeros(4 * 8)
+    p = ctypes.c_void_p(x.ctypes.data)
+    assert host.gm_tet_apply(t.h, 0, p, p, ctypes.c_double(1.0), 0, ctypes.c_void_p(8)) == 0
+    host.set_limit(with_rows + 4096)
+    assert t.step() == -2 and host.in_use() >= with_rows
+    host.set_limit(1 << 30)
+    assert t.step() == 0
     host.gm_tet_destroy(t.h)
+    assert host.in_use() == start
 
 
 def test_materials_leave_the_device_of_the_caller(host):
