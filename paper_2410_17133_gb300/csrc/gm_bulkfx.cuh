@@ -216,7 +216,9 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
                     const unsigned m = a.mask[node];
 #pragma unroll
                     for (int f = 0; f < NI; ++f) {
-                        const int hi = reinterpret_cast<const int*>(xin + (long long)f * N + node)[1] & 0x7fffffff;
+                        // exponent and upper bits; 1 for a value below 2^-1042, which is not zero either
+                        const double v = xin[(long long)f * N + node];
+                        const int h = __double2hiint(v) & 0x7fffffff, hi = h | (int)(__double2loint(v) != 0);
                         if (!((m >> (IN_P ? 3 : f)) & 1u)) {
                             m4 = max(m4, hi);
                             if (hi != 0) least = min(least, hi);
@@ -239,14 +241,15 @@ gm_bulk_fx_kernel(int chained, const __grid_constant__ BulkArgs<double> a, const
 #pragma unroll
         for (int w = 0; w < 8; ++w) { mx = max(mx, s_mx[w]); mn = min(mn, s_mn[w]); least = min(least, s_lo[w]); }
     }
+    const bool zero = mx == 0;
     mx >>= 20;
     mn = min(mn >> 20, mx);
     // a double keeps its 53 bits above the unit, 75 bits below 2^(mx - 1022), within 2^22 of the largest
     const bool cut = mx - min(least >> 20, mx) > 22;
-    const int top = mx == 0 ? 1023 : mx;
+    const int top = zero ? 1023 : mx;
     const int qe = (top - 1022 - GM_FX_IN) + (DO_K ? F.eK + F.topE - 1022 : DO_Q ? Q.eU : F.eA);
     const bool fixed_ok = top < 0x7ff && top >= 100 && qe >= -1000 && qe <= 900 &&
-                          (mx == 0 || mx - mn <= (DO_K ? F.gradeK : DO_Q ? Q.grade : DO_AUP ? GM_FX_GRADE : F.gradeA));
+                          (zero || mx - mn <= (DO_K ? F.gradeK : DO_Q ? Q.grade : DO_AUP ? GM_FX_GRADE : F.gradeA));
     auto fp64_tile = [&]() {
         gm_fx_fp64_tile<CLS, MODE>(a, R, raw);
         if constexpr (DOT) {

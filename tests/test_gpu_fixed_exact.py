@@ -142,6 +142,22 @@ def test_large_parts_without_force_take_no_bits_from_small_ones(cell, op, name, 
     compare(op, prob, u, k >= 5)
 
 
+@pytest.mark.parametrize("op", ["KB", "J"])
+@pytest.mark.parametrize("above", [0.0, 1.0])
+@pytest.mark.parametrize("size", [2.0 ** -1040, 2.0 ** -1046])
+def test_subnormal_fields_exert_their_forces(size, above, op, monkeypatch):
+    """Multiples of a subnormal, alone and with ones in the planes below: the stiffness carries their
+    forces into the normal range."""
+    need_gpu()
+    prob = problem("cube", monkeypatch)
+    k = nodes()[2]
+    noise = size * np.random.default_rng(7).integers(-8, 9, (3, k.size))
+    u = np.where(k >= 8, noise, np.where((k >= 3) & (k <= 6), above, 0.0))
+    if op == "J":
+        u = np.concatenate([u, np.zeros((1, k.size))])
+    compare(op, prob, u, k >= 9)
+
+
 @pytest.mark.parametrize("direction", [0, 1, 2])
 @pytest.mark.parametrize("dt", [1e-3, 1e3, 1e8])
 @pytest.mark.parametrize("cell", ["cube", "dip", "flat100"])
