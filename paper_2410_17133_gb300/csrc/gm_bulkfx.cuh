@@ -5,15 +5,15 @@
 // In the parity basis a K_b element takes about 210 FP64 instructions, 64
 // issue slots each; the same element takes about 2350 integer instructions here
 // (560 of them IMAD.WIDE, 2 slots each).  Measured against the FP64 kernel, us
-// per product: K_T on 128^3 dipping cells 1254 -> 410; K_T + A_pu + A_up + A22 on
-// 61x127x46 cells sheared both ways 804 -> 285 (A22 121 -> 46); J on 8^3 cells
-// 89 -> 46.
+// per product: K_T on 128^3 dipping cells 1256 -> 413; K_T + A_pu + A_up + A22 on
+// 61x127x46 cells sheared both ways 806 -> 287 (A22 121 -> 48); J on 8^3 cells
+// 90 -> 46.
 //
 // Each CTA first looks over its inputs: the largest exponent sets the tile's
 // unit, and the smallest of the elements' largest exponents says how far the
 // field is graded inside the tile.  A tile that is graded by more than 16 bits
-// (less the contrast of the moduli), not finite, or near the ends of the exponent
-// range takes the FP64 tile of gm_bulk.cuh.
+// (less the contrast of the moduli), not finite, subnormal, or near the ends of the
+// exponent range takes the FP64 tile of gm_bulk.cuh.
 //
 // The values alone do not say how exact FP64 would be: a field that is constant
 // over an element exerts no force however large it is, and the small ones beside

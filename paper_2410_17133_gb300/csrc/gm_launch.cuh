@@ -11,11 +11,11 @@
 // predecessors have.  Its loads are coherent ones: the kernel is already there while
 // its predecessor writes, so nothing that it reads is read-only for its lifetime, and
 // a non-coherent load (__ldg, __restrict__) could be served or moved ahead of the wait.
-// Kernels in between that are launched normally wait for completion as usual.  Measured, chained against plain launches: outside graphs
-// J on 8^3 cells 46.8 -> 43 us, five tetrahedral products 103 -> 94.5 us, the
-// FP32 products at 160^3 551 -> 533 us; in captured graphs it loses (FP32 step at
-// 64^3 84 -> 89 ms, FP64 K_T solve at 48^3 60.5 -> 66.8 ms), so there the launches
-// are plain and gm_chain returns at once.
+// Kernels in between that are launched normally wait for completion as usual.
+// Measured, chained against plain launches: outside graphs J on 8^3 cells 49.2 -> 45.7 us,
+// five tetrahedral products 102.9 -> 94.3 us, the FP32 products at 160^3 551 -> 528 us; in
+// captured graphs it loses (FP32 step at 64^3 84 -> 89 ms, FP64 K_T solve at 48^3
+// 60.5 -> 66.8 ms), so there the launches are plain and gm_chain returns at once.
 #pragma once
 
 #include <cuda_runtime.h>
